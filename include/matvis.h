@@ -95,12 +95,16 @@ typedef struct {
     int overlap_batches;        /* 1: with two or more batches, build the Z matrices of one batch
                                    on a second stream while the HERK of the previous one runs (two
                                    workspace sets); 0 (default): one set, strictly in order */
-    int fuse_zbuild;            /* 1 (default): with two or more batches and a tensor-core
-                                   precision, the HERK launch of batch b also builds the Z matrices
-                                   of batch b + 1 on extra warps of every SM (two workspace sets;
-                                   one feed and one axis, or two and two), unless mv_autotune timed
-                                   separate launches faster for the call's shape; 0: the Z build
-                                   runs as its own launch.  Takes precedence over overlap_batches. */
+    int fuse_zbuild;            /* 1 (default): with a tensor-core precision the launch that computes
+                                   V also builds Z.  With the herk_* options at 0 it streams Z of
+                                   many instances through a ring that stays in L2 (Z is never held
+                                   as a whole); with one of them set, or where mv_autotune timed it
+                                   faster, the HERK launch of batch b builds the Z matrices of batch
+                                   b + 1 on extra warps of every SM (two or more batches, two
+                                   workspace sets; one feed and one axis, or two and two), unless
+                                   mv_autotune timed separate launches faster for the call's shape;
+                                   0: the Z build runs as its own launch.  Takes precedence over
+                                   overlap_batches. */
 } mv_options;
 
 /* A tensor-core HERK configuration chosen by mv_autotune. */
@@ -111,7 +115,8 @@ typedef struct {
     int candidates;      /* configurations timed */
     double herk_ms;      /* best time of one batch: the HERK launch (with the next batch's Z build when
                             fused), or the HERK and the batch's own Z-side launches */
-    int fused;           /* 1: the HERK launch of a batch builds the next batch's Z planes;
+    int fused;           /* 1: the launch that computes V also builds Z (streamed through L2, with
+                            128-column tiles, or the next batch's Z planes);
                             0: every batch's Z build runs as its own launches */
 } mv_tuning;
 
@@ -224,8 +229,10 @@ mv_status mv_simulate_pairs(mv_ctx *ctx, int n_pairs, const double *lst, const d
  * HERK of that batch under each candidate (tile width 128 or 256 -- 128 only
  * when the Z build is fused, and then every trial also builds a batch of Z
  * planes --, split of the source axis 1 to 64, flush every 4, 8 or 16
- * k-blocks) with CUDA events on the context's stream, and keeps the fastest
- * for later calls with the same matrix size, batch size and precision.
+ * k-blocks), and the streamed schedule (see mv_options.fuse_zbuild) on up to 64
+ * instances of the call where the options allow it, with CUDA events on the
+ * context's stream, and keeps the fastest for later calls with the same matrix
+ * size, batch size and precision.
  * Synchronises.  prec must be a tensor-core precision.  out may be NULL. */
 mv_status mv_autotune(mv_ctx *ctx, int n_t, const double *lst, int n_nu, const double *nu,
                       mv_precision prec, int pairs, mv_tuning *out);

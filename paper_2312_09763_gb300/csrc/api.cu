@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <map>
 #include <string>
 #include <thread>
 #include <vector>
@@ -15,6 +16,7 @@
 #include "matvis.h"
 #include "common.cuh"
 #include "redund.h"
+#include "zherk.h"
 
 using namespace mv;
 
@@ -66,6 +68,11 @@ struct mv_ctx {
     int red_nf = 0;  // feeds the plan was made for
     Buf red_e, red_n, red_u, red_b, red_uidx, red_tl[2];  // red_tl: 128- and 256-column tiles
     int red_ntl[2] = {0, 0};
+    std::vector<ZherkTile> red_tiles;  // the 128-column tiles, and the limits of their blocks
+    std::vector<int2> red_limits;
+    // streamed Z build + HERK (zherk_tc.cu): the ring, and the tables of a call
+    Buf ring, ztab, zcount, zscale, zorder, zwave, zamax;
+    std::map<std::vector<long long>, ZherkPlan> zplans;  // by shape (bounded)
     // model buffers
     std::vector<double> h_flux;  // I at nu_ref (host copy, for the polarised sky's coherency)
     Buf xeq, sqrt_flux, half_alpha, pol_m, ant_e, ant_n, ant_u, bidx, grid;
@@ -86,6 +93,7 @@ struct mv_ctx {
         int rows = 0, slots = 0, zprec = 0;
         HerkCfg cfg;
         bool fuse = true;  // the timed schedule: fused Z build, or separate Z-side launches
+        bool stream = false;  // or the streamed one
         double ms = 0;
     } tuned;
     // captured launch sequence of the last call shape
@@ -290,6 +298,17 @@ struct Plan {
     struct Batch { int inst0, n, g0, ng; };
     std::vector<Batch> batches;
     bool unique = false;  // one value per redundant group instead of the full V
+    bool pairs = false;   // explicit (LST, frequency) pairs
+};
+
+// One launch of the streamed schedule: instances [inst0, inst0 + n) and where
+// its tables lie in the call's table buffer (bytes).
+struct StreamBatch {
+    int inst0, n, g0, ng;  // groups [g0, g0 + ng) of the plan: entries of the antenna phase table
+    const ZherkPlan* plan;
+    size_t jobs, groups, items, group0, tiles, tile_of, limits;
+    int n_groups, ant_block, np;
+    long long max_chunks;
 };
 
 // A group of consecutive instances [i0, i0+n) of one time: equally spaced
@@ -367,6 +386,7 @@ void plan_grid(mv_ctx* c, int n_t, const double* lst, int n_nu, const double* nu
 void plan_pairs(mv_ctx* c, int n_pairs, const double* lst, const double* nu, Plan& P) {
     P.lst.assign(lst, lst + n_pairs);
     P.nu.assign(nu, nu + n_pairs);
+    P.pairs = true;
     const long long N = (long long)c->model.n_feed * c->model.n_ant;
     for (int i = 0; i < n_pairs; ++i) P.inst.push_back(Inst{i, i, (long long)i * N * N});
     const int B = auto_batch(c, slot_bytes_of(c));
@@ -395,7 +415,128 @@ struct Prepared {
     size_t v_bytes = 0;
     long long per_inst = 0;  // output values per instance: N^2, or n_unique n_feed^2
     HerkOut ho{};             // unique output: group lookup and tile lists (ho.tl set per tile width)
+    bool stream = false;      // the streamed schedule (zherk_tc.cu)
+    std::vector<StreamBatch> sb;
+    int sflush = 8;           // (stream) 32-column stages per TMEM flush
 };
+
+// Bytes the ring of Z may take: it has to stay in L2 (129 MB over two dies) beside
+// the WA tables in flight.
+constexpr long long kRingBytes = 96ll << 20;
+
+// Plan the streamed schedule: batches of consecutive instances (whose WA tables
+// fit the budget), and for each the jobs, channel groups and Z items of its
+// waves in one table buffer.  Replaces the plan's groups and batches.  False
+// where it does not apply (the tiles of one instance exceed the SMs).
+bool plan_stream(mv_ctx* c, Plan& P, Prepared& p, std::vector<uint8_t>& tab) {
+    const Model& m = c->model;
+    static const std::vector<ZherkTile> whole_v;
+    const bool covered = P.unique && c->red.kind != 0;
+    const std::vector<ZherkTile> cover = covered ? c->red_tiles : P.unique ? zherk_triangle(p.rows) : whole_v;
+    const long long wa_slot = 8ll * p.ncomp * p.pitch;
+    const long long budget = 8ll << 30;
+    int B = (int)std::max(1ll, std::min<long long>(kMaxBatch, budget / wa_slot));
+    if (c->opt.max_batch > 0) B = std::min(B, c->opt.max_batch);
+    auto plan_for = [&](int n) -> const ZherkPlan* {
+        std::vector<long long> key = {p.rows, m.n_ax, n, m.n_src};
+        for (const ZherkTile& t : cover) key.push_back((long long)t.r0 << 32 | (unsigned)t.c0);
+        auto it = c->zplans.find(key);
+        if (it == c->zplans.end()) {
+            ZherkPlan z;
+            if (!zherk_plan(p.N, cover, m.n_ax, n, 0.5 * (double)m.n_src, c->n_sms, kRingBytes, z)) z.V = 0;
+            it = c->zplans.emplace(key, std::move(z)).first;
+        }
+        return it->second.V > 0 ? &it->second : nullptr;
+    };
+    if (c->zplans.size() > 64) c->zplans.clear();
+    const ZherkPlan* whole = plan_for(std::min(B, p.n_inst));
+    if (!whole) return false;
+    // full batches hold whole waves
+    if (p.n_inst > B && whole->S == 1 && B > whole->V) B = B / whole->V * whole->V;
+    P.groups.clear();
+    P.batches.clear();
+    p.sb.clear();
+    p.max_slots = 0;
+    auto put = [&](const void* d, size_t bytes) {
+        const size_t at = (tab.size() + 15) / 16 * 16;
+        tab.resize(at + bytes);
+        std::memcpy(tab.data() + at, d, bytes);
+        return at;
+    };
+    for (int i0 = 0; i0 < p.n_inst; i0 += B) {
+        const int n = std::min(B, p.n_inst - i0);
+        const ZherkPlan* z = plan_for(n);
+        if (!z) return false;
+        StreamBatch b{};
+        b.inst0 = i0;
+        b.n = n;
+        b.plan = z;
+        b.g0 = (int)P.groups.size();
+        std::vector<ZherkGroup> groups;
+        std::vector<int> items(z->waves), group0(z->waves);
+        if (P.pairs)
+            for (int j = 0; j < n; ++j) P.groups.push_back(make_group(P, i0 + j, 1, j));
+        const int total = n * z->S;
+        int most = 1;
+        for (int w = 0; w < z->waves; ++w) {
+            group0[w] = (int)groups.size();
+            const int v_n = std::min(z->V, total - w * z->V);
+            for (int v = 0; v < v_n;) {
+                const int ks = (w * z->V + v) / n, r = (w * z->V + v) % n;
+                int k = 1;
+                if (!P.pairs)
+                    while (v + k < v_n && r + k < n && P.inst[i0 + r + k].t == P.inst[i0 + r].t &&
+                           (w * z->V + v + k) / n == ks && (k + 1) * m.n_feed * m.n_ax <= kZherkChan)
+                        ++k;
+                ZherkGroup g{v, k, 0, 1, 0, 0, 0, 0, w * z->V + v, 0, 0, 0};
+                if (!P.pairs) {
+                    const ZGroup zg = make_group(P, i0 + r, k, r);
+                    g.aph = (int)P.groups.size() - b.g0;
+                    g.uniform = zg.uniform;
+                    P.groups.push_back(zg);
+                }
+                groups.push_back(g);
+                v += k;
+            }
+            items[w] = (int)groups.size() - group0[w];
+            most = std::max(most, items[w]);
+        }
+        int chan = 1;
+        for (const ZherkGroup& g : groups) chan = std::max(chan, g.n);
+        b.ant_block = zherk_ant_block(*z, m.n_ant, m.n_ax * m.n_feed, most, chan, c->n_sms);
+        if (b.ant_block < 1) return false;
+        b.ng = (int)P.groups.size() - b.g0;
+        b.n_groups = (int)groups.size();
+        b.jobs = put(z->jobs.data(), z->jobs.size() * sizeof(ZherkJob));
+        b.groups = put(groups.data(), groups.size() * sizeof(ZherkGroup));
+        b.items = put(items.data(), items.size() * sizeof(int));
+        b.group0 = put(group0.data(), group0.size() * sizeof(int));
+        b.tiles = put(z->tiles.data(), z->tiles.size() * sizeof(ZherkTile));
+        b.np = (p.N + 127) / 128;
+        if (z->form == kZherkGauss) {
+            std::vector<int> of(2 * b.np * b.np, 0);
+            for (size_t k = 0; k < z->tiles.size(); ++k) {
+                const ZherkTile& t = z->tiles[k];
+                of[(t.kind * b.np + t.r0 / 128) * b.np + t.c0 / 128] = (int)k;
+            }
+            b.tile_of = put(of.data(), of.size() * sizeof(int));
+        }
+        if (covered) {
+            std::vector<int> lim;
+            for (const int2& l : c->red_limits) {
+                lim.push_back(l.x);
+                lim.push_back(l.y);
+            }
+            b.limits = put(lim.data(), lim.size() * sizeof(int));
+        }
+        const long long nch = (m.n_src + kZherkChunk - 1) / kZherkChunk;
+        b.max_chunks = z->waves * ((nch + z->S - 1) / z->S + 1);
+        p.sb.push_back(b);
+        P.batches.push_back(Plan::Batch{i0, n, b.g0, b.ng});
+        p.max_slots = std::max(p.max_slots, n);
+    }
+    return true;
+}
 
 // Heuristic HERK configuration: wide tiles unless the matrix is narrow; a
 // split giving the persistent grid about 16 units per SM while each unit keeps
@@ -437,7 +578,8 @@ HerkCfg chosen_cfg(mv_ctx* c, const Prepared& p) {
     return heuristic_cfg(c, p);
 }
 
-mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_device, cudaStream_t st, Prepared& out) {
+mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_device, cudaStream_t st, Prepared& out,
+                  bool allow_stream = true, bool ignore_tuning = false) {
     Model& m = c->model;
     if (!c->have_sky || !c->have_ant || !c->have_beam)
         return fail(MV_ERR_STATE, "simulate needs init_sky, set_antennas and a beam first");
@@ -514,6 +656,23 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
         p.ho.n_ant = m.n_ant;
         p.ho.n_feed = m.n_feed;
     }
+    // the streamed schedule unless an option asks for a particular HERK or
+    // Z-build schedule, or the autotuner timed another one faster for calls of
+    // this shape
+    std::vector<uint8_t> ztab;
+    const mv_options& o = c->opt;
+    if (allow_stream && p.zprec != 0 && o.fuse_zbuild && !o.overlap_batches && o.herk_tile_n == 0 && o.herk_split == 0 &&
+        o.herk_flush_kblocks == 0 && (ignore_tuning || !(tuned_for(c, p) && !c->tuned.stream))) {
+        std::vector<ZGroup> groups = P.groups;
+        std::vector<Plan::Batch> batches = P.batches;
+        const int slots = p.max_slots;
+        p.stream = plan_stream(c, P, p, ztab);
+        if (!p.stream) {
+            P.groups = groups;
+            P.batches = batches;
+            p.max_slots = slots;
+        }
+    }
     const int n_times = p.n_times, max_slots = p.max_slots;
     const long long pitch = p.pitch;
 
@@ -537,10 +696,10 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
     // cover is the whole triangle: a cover of fewer tiles leaves the HERK too
     // short to hide the next batch's Z build (350-antenna array, 9 of 21
     // tiles: 250 ms per step fused against 210 ms separate)
-    p.fuse = c->opt.fuse_zbuild && p.zprec != 0 && P.batches.size() > 1 &&
+    p.fuse = !p.stream && c->opt.fuse_zbuild && p.zprec != 0 && P.batches.size() > 1 &&
              herk_tc_fusable(128, p.zprec, m.n_ax, m.n_feed) && !(tuned_for(c, p) && !c->tuned.fuse) &&
              (!P.unique || c->red.kind == 0);
-    p.nbuf = (P.batches.size() > 1 && (c->opt.overlap_batches || p.fuse)) ? 2 : 1;
+    p.nbuf = (!p.stream && P.batches.size() > 1 && (c->opt.overlap_batches || p.fuse)) ? 2 : 1;
     // antenna phase factors: per batch, groups x wavenumbers per group x antennas
     p.n_phase = 2;
     int max_groups = 1;
@@ -558,8 +717,26 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
     for (int k = 0; k < p.nbuf; ++k)
         if ((s = ensure(c, c->aph[k], sizeof(AntPhase) * (size_t)max_groups * p.n_phase * m.n_ant))) return s;
     if ((s = ensure(c, c->sched, sizeof(int) * (size_t)(max_slots + 8)))) return s;
+    if (p.stream) {
+        size_t ring = 0, part = 0, waves = 0, chunks = 0, vinsts = 0;
+        for (const StreamBatch& b : p.sb) {
+            ring = std::max(ring, (size_t)zherk_row_bytes(c->model.n_ax) * b.plan->rows * b.plan->V);
+            part = std::max(part, sizeof(float) * 128 * 128 * (size_t)b.n * b.plan->tiles.size() * b.plan->S);
+            waves = std::max(waves, (size_t)b.plan->waves + 1);
+            chunks = std::max(chunks, (size_t)b.max_chunks);
+            vinsts = std::max(vinsts, (size_t)b.n * b.plan->S);
+        }
+        if ((s = upload(c, c->ztab, ztab.data(), ztab.size(), st))) return s;
+        if ((s = ensure(c, c->ring, ring))) return s;
+        if ((s = ensure(c, c->partial, part))) return s;
+        if ((s = ensure(c, c->zwave, sizeof(int) * waves))) return s;
+        if ((s = ensure(c, c->zcount, sizeof(int) * 2 * chunks))) return s;
+        if ((s = ensure(c, c->zscale, sizeof(float) * max_slots))) return s;
+        if ((s = ensure(c, c->zamax, sizeof(float) * max_slots))) return s;
+        if ((s = ensure(c, c->zorder, sizeof(int4) * vinsts))) return s;
+    }
     const size_t plane_elems = (size_t)p.rows * p.k_pitch * max_slots;
-    for (int k = 0; k < p.nbuf; ++k) {
+    for (int k = 0; k < p.nbuf && !p.stream; ++k) {
         if (p.zprec == 0) {
             if ((s = ensure(c, c->u[k], sizeof(float) * plane_elems))) return s;
         } else {
@@ -567,7 +744,7 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
             if ((s = ensure(c, c->ulo[k], 2 * plane_elems))) return s;
         }
     }
-    if (p.zprec != 0) {
+    if (p.zprec != 0 && !p.stream) {
         // partial tiles for the largest split any configuration may use
         const HerkCfg h = chosen_cfg(c, p);
         size_t units = (size_t)herk_tc_units(p.rows, max_slots, h.split, h.bn);
@@ -664,14 +841,15 @@ mv_status enqueue_wa(mv_ctx* c, const Prepared& p, const Plan::Batch& b, int k, 
     return launched(e, "beam evaluation", st);
 }
 
-// Antenna phase table of one batch into workspace set k (fused Z build).
+// Antenna phase table of one batch into workspace set k (fused Z build, which
+// also wants one max |WA| per Z group, and the streamed schedule).
 mv_status enqueue_ant_phase(mv_ctx* c, const Prepared& p, const Plan::Batch& b, int k, cudaStream_t st,
-                            long long* L, int kw = -1) {
+                            long long* L, int kw = -1, bool group_max = true) {
     if (kw < 0) kw = k;
     Timed tz(c, MV_KERNEL_ZBUILD, st);
     cudaError_t e = launch_ant_phase(c->model, (const Inst*)c->inst.p, (const Chan*)c->chan.p,
                                      (const ZGroup*)c->groups.p, b.g0, b.ng, (AntPhase*)c->aph[k].p, p.n_phase,
-                                     p.zprec == 2 ? (float*)c->amax[kw].p : nullptr, st, L);
+                                     p.zprec == 2 && group_max ? (float*)c->amax[kw].p : nullptr, st, L);
     tz.end();
     return launched(e, "phase table", st);
 }
@@ -689,6 +867,74 @@ mv_status enqueue_zside(mv_ctx* c, const Prepared& p, const Plan::Batch& b, int 
                       p.n_phase, st, L);
     tz.end();
     return launched(e, "Z build", st);
+}
+
+// One batch of the streamed schedule: beam evaluation, phase table, then the
+// launch that builds Z and expands it, and the sum of its partial tiles into V.
+mv_status enqueue_stream(mv_ctx* c, const Prepared& p, size_t i, cudaStream_t st, long long* L) {
+    mv_status s;
+    const StreamBatch& b = p.sb[i];
+    const Plan::Batch pb{b.inst0, b.n, b.g0, b.ng};
+    if ((s = enqueue_wa(c, p, pb, 0, st, L))) return s;
+    if ((s = enqueue_ant_phase(c, p, pb, 0, st, L, -1, false))) return s;
+    const uint8_t* tab = (const uint8_t*)c->ztab.p;
+    ZherkArgs z{};
+    z.m = c->model;
+    z.inst = (const Inst*)c->inst.p;
+    z.inst0 = b.inst0;
+    z.n_inst = b.n;
+    z.lt = p.lt;
+    z.wa = (const float2*)c->wa[0].p;
+    z.wa_pitch = p.pitch;
+    z.scale = (const float*)c->zscale.p;
+    z.aph = (const AntPhase*)c->aph[0].p;
+    z.n_phase = p.n_phase;
+    z.zv = (const int4*)c->zorder.p;
+    z.ring = (uint8_t*)c->ring.p;
+    z.rows = b.plan->rows;
+    z.map_rows = b.plan->form == kZherkReal ? b.plan->rows : p.N;
+    z.V = b.plan->V;
+    z.S = b.plan->S;
+    z.n_waves = b.plan->waves;
+    z.v_last = b.n * z.S - (z.n_waves - 1) * z.V;
+    z.wave_base = (const int*)c->zwave.p;
+    z.wave_items = (const int*)(tab + b.items);
+    z.wave_group0 = (const int*)(tab + b.group0);
+    z.groups = (const ZherkGroup*)(tab + b.groups);
+    z.jobs = (const ZherkJob*)(tab + b.jobs);
+    z.n_jobs = b.plan->n_jobs;
+    z.n_jobs_last = b.plan->n_jobs_last;
+    z.ant_block = b.ant_block;
+    z.flush = p.sflush;
+    z.n_tiles = (int)b.plan->tiles.size();
+    z.ready = (int*)c->zcount.p;
+    z.done = z.ready + b.max_chunks;
+    z.partial = (float*)c->partial.p;
+    z.err = (int*)c->err.p;
+    Timed th(c, MV_KERNEL_HERK, st);
+    if ((s = cuda_check(cudaMemsetAsync(c->zcount.p, 0, sizeof(int) * 2 * b.max_chunks, st), "chunk counters"))) return s;
+    cudaError_t e = launch_zherk_prep(z, (const float*)c->amax[0].p, (float*)c->zamax.p, (float*)c->zscale.p,
+                                      (int4*)c->zorder.p, (int*)c->zwave.p, (ZherkGroup*)((uint8_t*)c->ztab.p + b.groups),
+                                      b.n_groups, p.plan->pairs, st, L);
+    if (e == cudaSuccess) e = launch_zherk(z, b.plan->form, c->n_sms, st, L);
+    ZherkFinalArgs f{};
+    f.inst = z.inst;
+    f.inst0 = b.inst0;
+    f.n_inst = b.n;
+    f.amax = (const float*)c->zamax.p;
+    f.partial = z.partial;
+    f.tiles = (const ZherkTile*)(tab + b.tiles);
+    f.tile_of = (const int*)(tab + b.tile_of);
+    f.n_tiles = z.n_tiles;
+    f.S = z.S;
+    f.N = p.N;
+    f.np = b.np;
+    f.V = p.Vout;
+    f.ho = p.ho;
+    f.limits = p.ho.uidx && c->red.kind != 0 ? (const int2*)(tab + b.limits) : nullptr;
+    if (e == cudaSuccess) e = launch_zherk_final(f, b.plan->form, st, L);
+    th.end();
+    return launched(e, "streamed Z build and HERK", st);
 }
 
 // The whole launch sequence of a call: cull, beam planes, then per batch
@@ -733,6 +979,13 @@ mv_status enqueue_all(mv_ctx* c, Plan& P, Prepared& p, const HerkCfg& h, cudaStr
                                st, L);
         tb.end();
         if ((s = launched(e, "beam planes", st))) return s;
+    }
+    if (p.stream) {
+        for (size_t i = 0; i < p.sb.size(); ++i) {
+            if ((s = enqueue_stream(c, p, i, st, L))) return s;
+            if ((s = copy_out(P.batches[i]))) return s;
+        }
+        return join_copies();
     }
     if (p.fuse) {
         // batch 0 alone; then the HERK launch of batch b also builds the Z
@@ -849,7 +1102,7 @@ std::vector<long long> graph_key(mv_ctx* c, const Plan& P, const Prepared& p, co
                          &c->wa[1], &c->amax[1], &c->u[1], &c->ulo[1], &c->wa[2], &c->amax[2], &c->partial,
                          &c->planes, &c->grid, &c->err,
                          &c->lsfix, &c->lseps, &c->aph[0], &c->aph[1], &c->pol_m, &c->red_uidx, &c->red_tl[0],
-                         &c->red_tl[1]};
+                         &c->red_tl[1], &c->ring, &c->ztab, &c->zcount, &c->zscale, &c->zorder, &c->zwave, &c->zamax};
     for (const Buf* b : bufs) k.push_back((long long)(uintptr_t)b->p);
     for (const auto& b : P.batches) {
         k.push_back(b.inst0);
@@ -857,6 +1110,17 @@ std::vector<long long> graph_key(mv_ctx* c, const Plan& P, const Prepared& p, co
         k.push_back(b.g0);
         k.push_back(b.ng);
     }
+    k.push_back(p.stream ? p.sflush : 0);
+    k.push_back(P.pairs ? 1 : 0);
+    k.push_back(p.n_phase);
+    for (const StreamBatch& b : p.sb)
+        for (long long x : {(long long)b.plan->V, (long long)b.plan->S, (long long)b.plan->waves, (long long)b.plan->form,
+                            (long long)b.plan->n_jobs, (long long)b.plan->n_jobs_last, (long long)b.plan->rows,
+                            (long long)b.plan->tiles.size(),
+                            (long long)b.jobs, (long long)b.groups, (long long)b.items, (long long)b.group0,
+                            (long long)b.tiles, (long long)b.tile_of, (long long)b.limits, (long long)b.n_groups,
+                            (long long)b.ant_block, b.max_chunks})
+            k.push_back(x);
     return k;
 }
 
@@ -966,7 +1230,7 @@ mv_status autotune(mv_ctx* c, Plan& P, mv_precision prec, cudaStream_t st, mv_tu
     mv_status s;
     if ((s = ensure(c, c->vdev, sizeof(float2)))) return s;
     // V for the trial runs: the context's staging buffer
-    if ((s = prepare(c, P, prec, c->vdev.p, 0, st, p))) return s;
+    if ((s = prepare(c, P, prec, c->vdev.p, 0, st, p, false))) return s;
     if (p.n_inst == 0) return MV_OK;
     const Plan::Batch b0 = P.batches[0];
     std::vector<HerkCfg> cands;
@@ -1043,22 +1307,59 @@ mv_status autotune(mv_ctx* c, Plan& P, mv_precision prec, cudaStream_t st, mv_tu
             best_fused = fused_trial[i];
         }
     }
+    // the streamed schedule (Z never in HBM), on the call's first instances: it runs
+    // many instances of any time per launch, so it is compared per instance
+    bool best_stream = false;
+    int n_cands = (int)cands.size();
+    {
+        Plan P2 = P;
+        P2.inst.resize(std::min<size_t>(P.inst.size(), 64));
+        Prepared p2;
+        if ((s = prepare(c, P2, prec, c->vdev.p, 0, st, p2, true, true))) return s;
+        if (p2.stream) {
+            ++n_cands;
+            if ((s = cuda_check(launch_cull(m, (const double*)c->R.p, p2.n_times, p2.lt, (int*)c->counts.p,
+                                            (int*)c->offsets.p, p2.bpt, st, &L), "cull")))
+                return s;
+            double sms = 1e300;
+            for (int r = 0; r <= reps; ++r) {  // the first run warms up
+                cudaEventRecord(e0, st);
+                for (size_t i = 0; i < p2.sb.size(); ++i)
+                    if ((s = enqueue_stream(c, p2, i, st, &L))) return s;
+                cudaEventRecord(e1, st);
+                if ((s = cuda_check(cudaEventSynchronize(e1), "trial timing"))) return s;
+                float ms = 0.f;
+                cudaEventElapsedTime(&ms, e0, e1);
+                if (r > 0) sms = std::min(sms, (double)ms);
+            }
+            // (a batch's beam evaluation is in every schedule's time here but the fused one's)
+            const double per_batch = sms / (double)P2.inst.size() * b0.n;
+            if (per_batch < best_ms) {
+                best_ms = per_batch;
+                best_stream = best_fused = true;
+                best = HerkCfg{};
+                best.bn = 128;
+                best.split = p2.sb[0].plan->S;
+            }
+        }
+    }
     c->pool.push_back(e0);
     c->pool.push_back(e1);
     if ((s = mv_check_device_status(c, st))) return s;
     c->tuned.valid = true;
+    c->tuned.stream = best_stream;
     c->tuned.rows = p.rows;
     c->tuned.slots = p.max_slots;
     c->tuned.zprec = p.zprec;
     c->tuned.cfg = best;
-    c->tuned.fuse = best_fused;
+    c->tuned.fuse = best_fused && !best_stream;
     c->tuned.ms = best_ms;
     if (out) {
         out->tile_n = best.bn;
         out->split = best.split;
         out->flush_kblocks = best.flush;
         out->herk_ms = best_ms;
-        out->candidates = (int)cands.size();
+        out->candidates = n_cands;
         out->fused = best_fused ? 1 : 0;
     }
     return MV_OK;
@@ -1096,7 +1397,7 @@ mv_status mv_create(mv_ctx** out, int device, const mv_options* opt) {
     mv_ctx* c = new mv_ctx();
     c->device = device;
     c->n_sms = pr.multiProcessorCount;
-    if (herk_tc_init() != cudaSuccess || mlp_tc_init() != cudaSuccess || gemm_tc_init() != cudaSuccess ||
+    if (herk_tc_init() != cudaSuccess || zherk_init() != cudaSuccess || mlp_tc_init() != cudaSuccess || gemm_tc_init() != cudaSuccess ||
         mlp_chain_init() != cudaSuccess || wgrad_tc_init() != cudaSuccess) {
         cudaGetLastError();
         delete c;
@@ -1367,6 +1668,12 @@ mv_status mv_set_redundancy(mv_ctx* c, double tol_m, int64_t* n_unique) {
                     }
             }
         }
+    c->red_tiles.clear();
+    c->red_limits.clear();
+    for (const TileDesc& t : tl[0]) {
+        c->red_tiles.push_back(ZherkTile{t.r0, t.c0, t.r0, t.c0, 0, 0});
+        c->red_limits.push_back(make_int2(t.rlim, t.clim));
+    }
     DeviceGuard g(c->device);
     mv_status s;
     if ((s = upload(c, c->red_e, e.data(), n * sizeof(double), c->stream))) return s;

@@ -112,6 +112,14 @@ __device__ __forceinline__ void apply_sky_sqrt(float2 a0, float2 a1, float4 M, f
     z1.y = w * (a1.y * M.w);
 }
 
+// Where source s of a WA component row lies: sources in pairs, (re, re, im, im),
+// so that a thread building two sources has their real and imaginary parts as
+// packed pairs.
+__device__ __forceinline__ void put_wa(float2* row, long long s, float2 v) {
+    float* p = reinterpret_cast<float*>(row) + (s >> 1) * 4 + (s & 1);
+    p[0] = v.x;
+    p[2] = v.y;
+}
 // WA[slot] = sqrt(I_s) A(s) for the live sources and zero for the rest of
 // the pitch; amax[slot] (zeroed by the caller) receives max |WA| over the
 // slot's components, as float bits.

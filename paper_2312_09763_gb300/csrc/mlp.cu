@@ -292,7 +292,8 @@ __global__ void k_wa_rows(Model m, int K, long long r0, int R, int t, float ln_r
             const float w = m.sqrt_flux[src] * spec;
             for (int c = 0; c < ncomp; ++c) {
                 const float2 v = make_float2(w * Y[(long long)i * 8 + 2 * c], w * Y[(long long)i * 8 + 2 * c + 1]);
-                wa_slot[((long long)b * ncomp + c) * wa_pitch + s] = v;
+                put_wa(wa_slot + ((long long)b * ncomp + c) * wa_pitch, s, v);
+                if (s == K - 1 && (s & 1) == 0) put_wa(wa_slot + ((long long)b * ncomp + c) * wa_pitch, K, make_float2(0.f, 0.f));
                 mx = fmaxf(mx, hypotf(v.x, v.y));
             }
         } else {  // two axes per feed: z = A M (eq. "fullz")
@@ -301,8 +302,13 @@ __global__ void k_wa_rows(Model m, int K, long long r0, int R, int t, float ln_r
                 const float* y = Y + (long long)i * 8 + 2 * c;
                 float2 z0, z1;
                 apply_sky_sqrt(make_float2(y[0], y[1]), make_float2(y[2], y[3]), M, spec, z0, z1);
-                wa_slot[((long long)b * ncomp + c) * wa_pitch + s] = z0;
-                wa_slot[((long long)b * ncomp + c + 1) * wa_pitch + s] = z1;
+                float2* row = wa_slot + ((long long)b * ncomp + c) * wa_pitch;
+                put_wa(row, s, z0);
+                put_wa(row + wa_pitch, s, z1);
+                if (s == K - 1 && (s & 1) == 0) {
+                    put_wa(row, K, make_float2(0.f, 0.f));
+                    put_wa(row + wa_pitch, K, make_float2(0.f, 0.f));
+                }
                 mx = fmaxf(mx, fmaxf(hypotf(z0.x, z0.y), hypotf(z1.x, z1.y)));
             }
         }
@@ -1065,9 +1071,11 @@ cudaError_t surrogate_wa(Surrogate* S, const Model& m, const std::vector<Inst>& 
             ++*L;
             e = cudaGetLastError();
         }
-        // zeros past the live count (the Z build reads whole source pairs)
-        if (e == cudaSuccess && K < wa_pitch)
-            e = cudaMemset2DAsync(wslot + K, sizeof(float2) * wa_pitch, 0, sizeof(float2) * (wa_pitch - K),
+        // zeros past the live count (the Z build reads whole source pairs; the last
+        // live source's pair is completed by its writer)
+        const int K2 = (K + 1) & ~1;
+        if (e == cudaSuccess && K2 < wa_pitch)
+            e = cudaMemset2DAsync(wslot + K2, sizeof(float2) * wa_pitch, 0, sizeof(float2) * (wa_pitch - K2),
                                   (size_t)m.n_beam * ncomp, st);
     }
     return e;

@@ -499,14 +499,20 @@ k_mlp_wa(const __grid_constant__ Maps maps, const __grid_constant__ Net net, Mod
                 if (valid) {
                     const float spec = expf(g_alpha[row] * ln_ratio);
                     const float4 gm = g_m[row];
-                    float2* wb = wa + (long long)b * ncomp * wa_pitch + s;
+                    float* wb = reinterpret_cast<float*>(wa + (long long)b * ncomp * wa_pitch) + (s >> 1) * 4 + (s & 1);
+                    auto put = [&](int c, float2 v) {
+                        float* p = wb + 2 * (long long)c * wa_pitch;
+                        __stcs(p, v.x);
+                        __stcs(p + 2, v.y);
+                        if (s == K - 1 && (s & 1) == 0) p[1] = p[3] = 0.f;  // the pair's other half
+                    };
                     if (!m.pol_m) {
                         const float w = gm.x * spec;
 #pragma unroll
                         for (int c = 0; c < 4; ++c)
                             if (c < ncomp) {
                                 const float2 v = make_float2(w * y[2 * c], w * y[2 * c + 1]);
-                                __stcs(wb + (long long)c * wa_pitch, v);
+                                put(c, v);
                                 mx = fmaxf(mx, hypotf(v.x, v.y));
                             }
                     } else {  // two axes per feed: z = A M (eq. "fullz")
@@ -516,8 +522,8 @@ k_mlp_wa(const __grid_constant__ Maps maps, const __grid_constant__ Net net, Mod
                                 float2 z0, z1;
                                 apply_sky_sqrt(make_float2(y[2 * c], y[2 * c + 1]),
                                                make_float2(y[2 * c + 2], y[2 * c + 3]), gm, spec, z0, z1);
-                                __stcs(wb + (long long)c * wa_pitch, z0);
-                                __stcs(wb + (long long)(c + 1) * wa_pitch, z1);
+                                put(c, z0);
+                                put(c + 1, z1);
                                 mx = fmaxf(mx, fmaxf(hypotf(z0.x, z0.y), hypotf(z1.x, z1.y)));
                             }
                     }

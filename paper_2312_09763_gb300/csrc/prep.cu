@@ -148,7 +148,8 @@ __device__ __forceinline__ float keys(float x) {
 }
 
 // WA[slot][b][p][k][s] = sqrt(I_s(nu)) * A^{pk}_b(az_s, za_s, nu) for the live
-// sources of each instance (Algorithm 2 step ii, with the flux weight of step iv).
+// sources of each instance (Algorithm 2 step ii, with the flux weight of step iv),
+// in pairs of sources (common.cuh).
 // Max of |value| over a warp, folded into amax (non-negative floats order
 // like their bit patterns).
 __device__ __forceinline__ void fold_amax(float v, float* amax) {
@@ -169,11 +170,11 @@ k_wa(Model m, const float2* __restrict__ planes, const Chan* __restrict__ chan,
     const int nl = lt.n_live[in.t];
     const int ncomp = m.n_beam * m.n_feed * m.n_ax;
     float mx = 0.f;
-    float2* out = wa + (long long)slot * ncomp * wa_pitch + s;
+    float2* out = wa + (long long)slot * ncomp * wa_pitch;
     if (s < nl) {
         mx = wa_eval(m, planes, chan[in.c], in, lt, s, out, wa_pitch);
     } else if (s < wa_pitch) {  // zeros past the live count: the Z build reads whole source pairs
-        for (int comp = 0; comp < ncomp; ++comp) out[(long long)comp * wa_pitch] = make_float2(0.f, 0.f);
+        for (int comp = 0; comp < ncomp; ++comp) put_wa(out + (long long)comp * wa_pitch, s, make_float2(0.f, 0.f));
     }
     fold_amax(mx, amax + slot);
 }
@@ -191,7 +192,7 @@ __device__ float wa_eval(const Model& m, const float2* __restrict__ planes, cons
     const int ncomp = m.n_beam * m.n_feed * m.n_ax;
     if (m.beam_kind == 1) {
         const float a = w * expf(-m.gauss_c * azza.y * azza.y);
-        out[0] = make_float2(a, 0.f);
+        put_wa(out, s, make_float2(a, 0.f));
         return fabsf(a);
     }
     // stencil in za (pole-reflected, clamped) and az (periodic)
@@ -240,15 +241,15 @@ __device__ float wa_eval(const Model& m, const float2* __restrict__ planes, cons
         }
         if (!m.pol_m) {
             const float2 v = make_float2(w * re, w * im);
-            out[(long long)comp * wa_pitch] = v;
+            put_wa(out + (long long)comp * wa_pitch, s, v);
             mx = fmaxf(mx, hypotf(v.x, v.y));
         } else if ((comp & 1) == 0) {  // axis 0 of a (beam, feed): wait for axis 1
             a_prev = make_float2(re, im);
         } else {
             float2 z0, z1;
             apply_sky_sqrt(a_prev, make_float2(re, im), M, w, z0, z1);
-            out[(long long)(comp - 1) * wa_pitch] = z0;
-            out[(long long)comp * wa_pitch] = z1;
+            put_wa(out + (long long)(comp - 1) * wa_pitch, s, z0);
+            put_wa(out + (long long)comp * wa_pitch, s, z1);
             mx = fmaxf(mx, fmaxf(hypotf(z0.x, z0.y), hypotf(z1.x, z1.y)));
         }
     }

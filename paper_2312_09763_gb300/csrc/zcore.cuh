@@ -178,10 +178,10 @@ __device__ __forceinline__ void zbuild_item(const Model& m, const Inst* __restri
                 for (int k = 0; k < NAX; ++k) {
                     const float4 a4 = A[p * NAX + k];
                     // Z = WA * exp(-2 pi i phase) = WA * (c - i s)
-                    re[k] = fmaf(a4.x, c0, a4.y * sn0);
-                    im[k] = fmaf(a4.y, c0, -a4.x * sn0);
-                    re[NAX + k] = fmaf(a4.z, c1, a4.w * sn1);
-                    im[NAX + k] = fmaf(a4.w, c1, -a4.z * sn1);
+                    re[k] = fmaf(a4.x, c0, a4.z * sn0);
+                    im[k] = fmaf(a4.z, c0, -a4.x * sn0);
+                    re[NAX + k] = fmaf(a4.y, c1, a4.w * sn1);
+                    im[NAX + k] = fmaf(a4.w, c1, -a4.y * sn1);
                 }
                 const long long r0 = 2ll * p * k_pitch;
                 put_row<PREC, NAX>(ur + r0, PREC != 0 ? lr + r0 : nullptr, re);

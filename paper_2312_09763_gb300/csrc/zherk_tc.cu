@@ -1,0 +1,1160 @@
+// zherk_tc.cu -- Algorithm 2 steps (iii)-(v) of arXiv:2312.09763 (Sec. 3.1) in
+// one persistent launch: the Z build (eq. "littlez" / "fullz") streams U = the
+// real form of Z, split in FP16 hi + lo, through a ring that stays in L2, and
+// the tensor cores expand V = Z Z^dagger from it as it is written.
+//
+// Why: the 350-antenna x 1e5-source instance's U is 140 MB.  Built by a launch
+// of its own (or inside the HERK of the batch before) it goes to HBM and comes
+// back, 280 MB per instance.  Here every SM owns one 128 x 256 product of some
+// instance for the whole source axis, so Z is needed only in source order, by
+// all products at about the same time: a ring of several hundred sources per
+// instance (62 MB in all there, inside the 129 MB L2) is enough, and Z never
+// reaches HBM (ncu: 0.3 % of the DRAM rate).
+//
+// A wave is V virtual instances (an instance, or one of S ranges of its
+// sources) whose products fill the SMs.  The ring is cut into chunks of 64
+// sources.  The SMs form teams that build every teams-th chunk of the wave
+// each: an SM keeps one channel group and up to 12 x ant_block antennas of it.
+// A finished chunk is counted in ready[chunk]; an SM's TMA warp loads it for
+// the SM's own product once every SM of the team has counted it, and counts the
+// SM up in done[chunk] when the loads have landed, which frees the chunk's
+// place in the ring.  Everybody takes the chunks in the same order, so the
+// oldest one never waits for a newer one; the launch is cooperative (all CTAs
+// resident).  Every wait is bounded (tc.cuh).
+//
+// Roles of a CTA (one per SM): warp 0 TMA, warp 1 MMA, warps 2-9 drain the
+// accumulator into FP32 running sums (both in TMEM) every `flush` stages,
+// COUNT_WARP publishes finished chunks, FEED_WARP copies each chunk's source
+// directions and WA into shared memory for the Z warps and watches the ring,
+// and 12 (8 with several components) warps build Z.
+//
+// What bounds it (350 antennas x 1e5 sources, 19 instances a wave): shared
+// memory.  A 64-source chunk costs an SM 128 KB of MMA operand reads, 80 KB of
+// TMA writes, 34 KB of Z stores and 22 KB of WA reads, about 2100 of its 2700
+// cycles at 128 bytes a cycle; the MMAs alone would take 1536, the Z build alone
+// (no loads, no MMAs) 1800.  56 instances take 3.39 ms against 4.79 with the Z
+// build fused into the HERK of the previous batch through HBM.
+//
+// Layout of a ring row: blocks of 32 columns, 128 bytes each, hi and lo halves of
+// 64 bytes (in turn, see the Z warps), so that one 128-byte-swizzled TMA box of
+// 128 rows brings both.
+#include <cuda.h>
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <cmath>
+#include "common.cuh"
+#include "tc.cuh"
+#include "zcore.cuh"
+#include "zherk.h"
+
+namespace mv {
+namespace {
+
+using namespace tc;
+using namespace zcore;
+
+constexpr int BOX = 128 * 128;            // bytes of a box: 128 rows x 32 columns, hi and lo
+constexpr int MAX_BOX = 3;                // boxes of a stage: A and two of B
+constexpr int STAGE = MAX_BOX * BOX;      // 48 KB
+constexpr int STAGES = 4;
+constexpr int EPI_WARPS = 8;              // four per 128 columns: warps 2-9
+constexpr int COUNT_WARP = 2 + EPI_WARPS, FEED_WARP = COUNT_WARP + 1, FIRST_Z = COUNT_WARP + 2;
+constexpr int TMEM_COLS = 512;            // the accumulator and the running sums, 256 columns each
+constexpr int RUN_COL = 256;
+constexpr int Z_BLOCK = 16;               // antennas a Z warp may have (half with channel stepping)
+constexpr int Z_APH_B = Z_BLOCK * (int)sizeof(AntPhase);  // their phase factors, per Z warp
+constexpr int Z_SRC_B = 6 * kZherkChunk * 4;              // a chunk's directions: 3 x S, 3 x eps
+constexpr int Z_CHAN = kZherkChan;        // channels x components of a chunk's WA in shared memory
+constexpr int Z_WA_B = Z_CHAN * kZherkChunk * 8;
+constexpr int Z_BUF = Z_SRC_B + Z_WA_B;   // one of two buffers
+// Z-build warps per SM: as many as the registers allow (24 warps of 80
+// registers in all with one component, 20 of 96 with several).
+__host__ __device__ constexpr int z_warps(int nc) { return nc == 1 ? 12 : 8; }
+constexpr int threads_for(int nc) { return (FIRST_Z + z_warps(nc)) * 32; }
+constexpr int smem_for(int nc) { return STAGES * STAGE + 2 * Z_BUF + z_warps(nc) * Z_APH_B + 1024 + 256; }
+static_assert(smem_for(1) <= 232448 && smem_for(2) <= 232448, "227 KB of shared memory");
+static_assert(Z_BUF % 16 == 0 && Z_SRC_B % 16 == 0 && Z_APH_B % 16 == 0, "16-byte copies");
+
+__device__ __forceinline__ int ld_relaxed(const int* p) {
+    int v;
+    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+    return p != 0;
+}
+__device__ __forceinline__ void red_release(int* p, int v) {
+    asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void red_add(int* p, int v) {
+    asm volatile("red.relaxed.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// -------------------------------------------------------------- Z build
+// The first two products of a K step share A: the first keeps it in the collector
+// buffer for the second (12 % fewer shared-memory reads; 0.95 -> 0.89 us a chunk).
+template <bool FIRST>
+__device__ __forceinline__ void tc_mma_shared_a(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    if constexpr (FIRST)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+            "l"(a), "l"(b), "r"(idesc), "r"(acc)
+            : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+            "l"(a), "l"(b), "r"(idesc), "r"(acc)
+            : "memory");
+}
+
+// a * b + c on two packed FP32 values (FFMA2: two products per issue slot)
+struct F2 {
+    unsigned long long u;
+};
+__device__ __forceinline__ F2 pack2(float a, float b) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.u) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(F2 v, float& a, float& b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v.u));
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(a.u), "l"(b.u));
+    return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.u) : "l"(a.u), "l"(b.u), "l"(c.u));
+    return r;
+}
+
+// hi and lo halves of two values (x - hi in one mixed-precision step)
+__device__ __forceinline__ void split2(float x0, float x1, uint32_t& hi, uint32_t& lo) {
+    const __half2 h = __floats2half2_rn(x0, x1);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    float l0, l1;
+    asm("{\n\t.reg .f16 a, b, m;\n\tmov.b32 {a, b}, %2;\n\tmov.b16 m, 0xBC00;\n\t"
+        "fma.rn.f32.f16 %0, a, m, %3;\n\tfma.rn.f32.f16 %1, b, m, %4;\n\t}"
+        : "=f"(l0), "=f"(l1) : "r"(hi), "f"(x0), "f"(x1));
+    const __half2 l = __floats2half2_rn(l0, l1);
+    lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.u) : "l"(a.u), "l"(b.u));
+    return r;
+}
+
+// Where an item's stores go and what they are multiplied with.
+struct ZOut {
+    uint8_t *hi, *lo;    // this lane's columns in the first row of antenna 0, first instance
+    unsigned inst_b;     // bytes of an instance's rows
+    const float2* wa;    // this lane's sources, first instance, beam 0
+    const float4* ws;    // the same in shared memory (one beam)
+    long long wa_slot, wa_pitch;
+    float scale;
+};
+
+// Two sources (times NAX columns) of one row, hi and lo.
+template <int NAX>
+__device__ __forceinline__ void put_row(uint8_t* ph, uint8_t* pl, const float (&v)[2 * NAX]) {
+    uint32_t h[NAX], l[NAX];
+#pragma unroll
+    for (int k = 0; k < NAX; ++k) split2(v[2 * k], v[2 * k + 1], h[k], l[k]);
+    if constexpr (NAX == 1) {
+        *reinterpret_cast<uint32_t*>(ph) = h[0];
+        *reinterpret_cast<uint32_t*>(pl) = l[0];
+    } else {
+        *reinterpret_cast<uint2*>(ph) = make_uint2(h[0], h[1]);
+        *reinterpret_cast<uint2*>(pl) = make_uint2(l[0], l[1]);
+    }
+}
+
+// Z of antenna a for every instance of group g: each lane two adjacent sources.
+// tab: the antenna's phase factors (shared memory; kappa0, then dkappa per_e
+// entries on).  A row of the ring has a fixed length and an antenna-feed's rows
+// (Re, Im and, with the gauss form, their sum) follow each other, so that all
+// stores of an instance have fixed offsets from two pointers.  ONE: one beam,
+// whose WA is in shared memory.
+template <int FORM, int NAX, int NFD, bool ONE>
+__device__ __forceinline__ void z_ant(const ZherkArgs& P, const ZherkGroup& g, const ZOut& o, const AntPhase* tab,
+                                      int per_e, int a, const unsigned (&S0)[3], const unsigned (&S1)[3],
+                                      const float (&E0)[3], const float (&E1)[3]) {
+    constexpr int NC = NFD * NAX, NP = FORM == kZherkReal ? 2 : 3, ROW_B = zherk_row_bytes(NAX);
+    const float2* w = ONE ? nullptr : o.wa + (long long)P.m.beam_idx[a] * NC * o.wa_pitch;
+    const float4* ws = o.ws;
+    uint8_t* hi = o.hi + (unsigned)(a * NFD * NP) * ROW_B;
+    uint8_t* lo = o.lo + (unsigned)(a * NFD * NP) * ROW_B;
+    // WA of the next instance
+    auto load_wa = [&](float4 (&A)[NC]) {
+        if constexpr (ONE) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) A[c] = ws[c * (kZherkChunk / 2)];
+            ws += NC * (kZherkChunk / 2);
+        } else {
+#pragma unroll
+            for (int c = 0; c < NC; ++c) A[c] = *reinterpret_cast<const float4*>(w + (long long)c * o.wa_pitch);
+            w += o.wa_slot;
+        }
+    };
+    // one instance, at phase (c, s), scaled
+    auto emit = [&](const float4 (&A)[NC], F2 c, F2 s) {
+#pragma unroll
+        for (int p = 0; p < NFD; ++p) {
+            float re[2 * NAX], im[2 * NAX], sm[2 * NAX];
+#pragma unroll
+            for (int k = 0; k < NAX; ++k) {
+                const float4 a4 = A[p * NAX + k];
+                // Z = WA (c - i s): re = x c + y s, im = y c - x s
+                const F2 x = pack2(a4.x, a4.y), y = pack2(a4.z, a4.w), nx = pack2(-a4.x, -a4.y);
+                const F2 r2 = fma2(x, c, mul2(y, s)), i2 = fma2(y, c, mul2(nx, s));
+                unpack2(r2, re[k], re[NAX + k]);
+                unpack2(i2, im[k], im[NAX + k]);
+                if constexpr (FORM == kZherkGauss) unpack2(add2(r2, i2), sm[k], sm[NAX + k]);
+            }
+            put_row<NAX>(hi + p * NP * ROW_B, lo + p * NP * ROW_B, re);
+            put_row<NAX>(hi + (p * NP + 1) * ROW_B, lo + (p * NP + 1) * ROW_B, im);
+            if constexpr (FORM == kZherkGauss) put_row<NAX>(hi + (p * NP + 2) * ROW_B, lo + (p * NP + 2) * ROW_B, sm);
+        }
+        hi += o.inst_b;
+        lo += o.inst_b;
+    };
+    if (g.uniform && g.n > 1) {
+        // equally spaced channels: exact fixed-point phase every kAnchor
+        // channels, complex recurrence in between (as zbuild_item)
+        const AntPhase p0 = tab[0], pd = tab[per_e];
+        unsigned long long F0 = phase64(p0, S0, E0), F1 = phase64(p0, S1, E1);
+        const unsigned long long Q0 = phase64(pd, S0, E0), Q1 = phase64(pd, S1, E1);
+        float r0c, r0s, r1c, r1s;
+        cos_sin_turns(Q0, r0c, r0s);
+        cos_sin_turns(Q1, r1c, r1s);
+        const F2 rc = pack2(r0c, r1c), rs = pack2(r0s, r1s), nrs = pack2(-r0s, -r1s);
+        constexpr int PF = NC == 1 ? 2 : 1;
+        for (int left = g.n; left > 0; left -= kAnchor) {
+            float c0, sn0, c1, sn1;
+            cos_sin_turns(F0, c0, sn0);
+            cos_sin_turns(F1, c1, sn1);
+            F2 c = pack2(c0 * o.scale, c1 * o.scale), s = pack2(sn0 * o.scale, sn1 * o.scale);
+            F0 += Q0 * kAnchor;
+            F1 += Q1 * kAnchor;
+            auto turn = [&]() {  // (c + i s) e^{2 pi i dF}
+                const F2 nc = fma2(c, rc, mul2(s, nrs));
+                s = fma2(s, rc, mul2(c, rs));
+                c = nc;
+            };
+            if (left >= kAnchor) {
+#pragma unroll
+                for (int jb = 0; jb < kAnchor; jb += PF) {
+                    float4 B[PF][NC];
+#pragma unroll
+                    for (int jj = 0; jj < PF; ++jj) load_wa(B[jj]);
+#pragma unroll
+                    for (int jj = 0; jj < PF; ++jj) {
+                        emit(B[jj], c, s);
+                        if (jb + jj + 1 < kAnchor) turn();
+                    }
+                }
+            } else {
+#pragma unroll 1
+                for (int j = 0; j < left; ++j) {
+                    float4 B[NC];
+                    load_wa(B);
+                    emit(B, c, s);
+                    turn();
+                }
+            }
+        }
+        return;
+    }
+    // one instance, or unevenly spaced channels: the phase of each from its own factors
+    const AntPhase* t = P.aph + (long long)g.aph * P.n_phase * P.m.n_ant + a;
+    for (int j = 0; j < g.n; ++j) {
+        float4 A[NC];
+        load_wa(A);
+        AntPhase p;
+        if (j == 0) p = tab[0];
+        else p = load_phase(t);
+        t += P.m.n_ant;
+        float c0, sn0, c1, sn1;
+        cos_sin_turns(phase64(p, S0, E0), c0, sn0);
+        cos_sin_turns(phase64(p, S1, E1), c1, sn1);
+        emit(A, pack2(c0 * o.scale, c1 * o.scale), pack2(sn0 * o.scale, sn1 * o.scale));
+    }
+}
+
+// The chunks this SM builds in wave w: every teams-th one from `team` on, of
+// group gi, antennas from a0 on (team < 0: none).
+struct ZShare {
+    int teams, team, gi, a0;
+};
+__device__ __forceinline__ ZShare z_share(const ZherkArgs& P, int w, int ants) {
+    const int n_groups = P.wave_items[w], nab = (P.m.n_ant + ants - 1) / ants, per = n_groups * nab;
+    ZShare s;
+    s.teams = (int)gridDim.x / per;
+    s.team = (int)blockIdx.x / per;
+    const int r = (int)blockIdx.x - s.team * per;
+    s.gi = r / nab;
+    s.a0 = (r - s.gi * nab) * ants;
+    if (s.team >= s.teams) s.team = -1;
+    return s;
+}
+
+// -------------------------------------------------------------- kernel
+template <int FORM, int NAX, int NFD, bool ONE>
+__global__ void __launch_bounds__(threads_for(NAX * NFD), 1)
+k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkArgs P) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    constexpr int Z_WARPS = z_warps(NAX * NFD), NC = NAX * NFD;
+    uint8_t* zsm = smem + STAGES * STAGE;      // two buffers, then the Z warps' phase factors
+    // barriers: full[STAGES], empty[STAGES], tfull, tempty, zfull[2], zdone[2], zfree[2]
+    uint64_t* bars = reinterpret_cast<uint64_t*>(zsm + 2 * Z_BUF + Z_WARPS * Z_APH_B);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 8);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    volatile int* freed = reinterpret_cast<volatile int*>(tmem_slot + 2);  // chunks every SM has loaded, in a row
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto full = [&](int s) { return smem_u32(&bars[s]); };
+    auto empty = [&](int s) { return smem_u32(&bars[STAGES + s]); };
+    const uint32_t tfull = smem_u32(&bars[2 * STAGES]), tempty = smem_u32(&bars[2 * STAGES + 1]);
+    auto zfull = [&](int b) { return smem_u32(&bars[2 * STAGES + 2 + b]); };
+    auto zdone = [&](int b) { return smem_u32(&bars[2 * STAGES + 4 + b]); };
+    auto zfree = [&](int b) { return smem_u32(&bars[2 * STAGES + 6 + b]); };
+    constexpr int SPC = kZherkChunk * NAX / 32, RC = zherk_ring_chunks(NAX);  // stages per chunk, chunks in the ring
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
+        mbar_init(tfull, 1);
+        mbar_init(tempty, EPI_WARPS);
+        for (int b = 0; b < 2; ++b) { mbar_init(zfull(b), 1); mbar_init(zdone(b), Z_WARPS); mbar_init(zfree(b), 1); }
+        *abort_flag = 0;
+        *freed = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(TMEM_COLS));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        tc_fence_before();
+    }
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t sbase = smem_u32(smem);
+    const ZherkJob& J = P.jobs[blockIdx.x];   // this SM's job, the same in every wave
+    const int jn = J.n;
+    // whether the job's instance is in wave w
+    auto has_job = [&](int w) { return jn > 0 && (w < P.n_waves - 1 || J.v < P.v_last); };
+
+    if (warp >= 2 && warp < 2 + EPI_WARPS) {
+        // epilogue: TMEM lane quadrant q4, 128-column half h; FP32 running sums in TMEM
+        const int q4 = warp & 3, h = (warp - 2) >> 2;
+        const uint32_t tl = tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(h * 128);
+        const uint32_t trun = tl + RUN_COL;
+        int cg = 0;
+        bool ok = true;
+        for (int w = 0; w < P.n_waves && ok; ++w) {
+            if (!has_job(w)) continue;
+            const int4 v = P.zv[w * P.V + J.v];
+            const int n_flush = (v.w * SPC + P.flush - 1) / P.flush;
+            for (int f = 0; f < n_flush; ++f, ++cg) {
+                if (!wait_bounded(tfull, (uint32_t)cg & 1u, abort_flag, P.err, kTimeoutNs, 300u)) { ok = false; break; }
+                tc_fence_after();
+                if (h * 128 < jn) {
+                    // both loads of a piece go out together; the MMAs wait for this
+#pragma unroll
+                    for (int g = 0; g < 128 / 16; ++g) {
+                        uint32_t acc[16];
+                        tmem_ld16(tl + g * 16, acc);
+                        if (f > 0) {
+                            uint32_t sum[16];
+                            tmem_ld16(trun + g * 16, sum);
+                            tmem_wait_ld16(acc);
+                            tmem_wait_ld16(sum);
+#pragma unroll
+                            for (int i = 0; i < 16; ++i)
+                                acc[i] = __float_as_uint(__uint_as_float(sum[i]) + __uint_as_float(acc[i]));
+                        } else {
+                            tmem_wait_ld16(acc);
+                        }
+                        tmem_st16(trun + g * 16, acc);
+                    }
+                    tmem_wait_st();
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(tempty);
+            }
+            if (!ok || *abort_flag) break;
+            if (h * 128 < jn) {
+                // partial tile, column-major [128][128] (coalesced along rows)
+                const int ks = (w * P.V + J.v) / P.n_inst;
+                float* p = P.partial + (((long long)v.x * P.n_tiles + J.tile[h]) * P.S + ks) * (128 * 128) + q4 * 32 + lane;
+#pragma unroll 1
+                for (int g = 0; g < 8; ++g) {
+                    uint32_t sum[16];
+                    if (n_flush > 0) {
+                        tmem_ld16(trun + g * 16, sum);
+                        tmem_wait_ld16(sum);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) sum[i] = 0u;
+                    }
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) p[(g * 16 + i) * 128] = __uint_as_float(sum[i]);
+                }
+            }
+        }
+    } else if (warp == COUNT_WARP) {
+        // count this SM up for every chunk whose items its Z warps have finished (a
+        // release waits for the SM's stores to reach L2, which would hold up a Z warp)
+        int k = 0;
+        bool ok = true;
+        for (int w = 0; w < P.n_waves && ok; ++w) {
+            const ZShare z = z_share(P, w, Z_WARPS * P.ant_block);
+            if (z.team < 0) continue;
+            const int base = P.wave_base[w], wlen = P.wave_base[w + 1] - base;
+            for (int q = z.team; q < wlen; q += z.teams, ++k) {
+                if (!wait_bounded(zdone(k & 1), (uint32_t)(k >> 1) & 1u, abort_flag, P.err, kTimeoutNs, 100u)) ok = false;
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                if (lane == 0) {
+                    mbar_arrive(zfree(k & 1));  // (seen: the buffer's barrier may start its next phase)
+                    red_release(P.ready + base + q, 1);
+                }
+                __syncwarp();
+            }
+        }
+    } else if (warp == FEED_WARP) {
+        // Feed the Z warps: each chunk's directions and (one beam) WA into one of two
+        // buffers.  And watch the next 32 chunks' done counts and tell the Z warps
+        // through shared memory how far the ring is free (one poller per SM).
+        const int last_base = P.wave_base[P.n_waves - 1], total = P.wave_base[P.n_waves];
+        int next = 0, k = 0, w = -1, q = 0, base = 0, wlen = 0;
+        ZShare z{1, -1, 0, 0};
+        const ZherkGroup* g = nullptr;
+        bool more = true;
+        unsigned long long t0 = gtimer();
+        while (more || next < total - RC) {
+            bool any = false;
+            int d = 0;
+            const int c = next + lane;
+            const bool look = next < total - RC && c < total;
+            if (look) d = ld_relaxed(P.done + c);
+            while (more && q >= wlen) {  // the next wave this SM builds for
+                if (++w >= P.n_waves) {
+                    more = false;
+                    break;
+                }
+                z = z_share(P, w, Z_WARPS * P.ant_block);
+                base = P.wave_base[w];
+                wlen = z.team < 0 ? 0 : P.wave_base[w + 1] - base;
+                q = z.team < 0 ? 0 : z.team;
+                if (z.team >= 0) g = P.groups + P.wave_group0[w] + z.gi;
+            }
+            if (more && (k < 2 || __all_sync(0xffffffffu, mbar_test(zfree(k & 1), ((uint32_t)(k >> 1) & 1u) ^ 1u)))) {
+                any = true;
+                const uint32_t bar = zfull(k & 1), dst = smem_u32(zsm + (k & 1) * Z_BUF);
+                if (q < g->len) {
+                    const int n = ONE ? g->n * NC : 0, src = (g->c0 + q) * kZherkChunk;
+                    if (lane == 0) mbar_expect_tx(bar, (uint32_t)(Z_SRC_B + n * kZherkChunk * 8));
+                    __syncwarp();
+                    if (lane < 6) {
+                        const long long o = ((long long)g->t * 3 + (lane < 3 ? lane : lane - 3)) * P.lt.pitch + src;
+                        bulk_load(dst + lane * (kZherkChunk * 4), lane < 3 ? (const void*)(P.lt.sfix + o) : (const void*)(P.lt.seps + o),
+                                  kZherkChunk * 4, bar);
+                    }
+                    if (lane < n)  // (one beam: the components of successive slots follow each other)
+                        bulk_load(dst + Z_SRC_B + lane * (kZherkChunk * 8), P.wa + ((long long)g->slot * NC + lane) * P.wa_pitch + src,
+                                  kZherkChunk * 8, bar);
+                } else if (lane == 0) {
+                    mbar_arrive(bar);
+                }
+                __syncwarp();
+                q += z.teams;
+                ++k;
+            }
+            if (next < total - RC) {
+                const unsigned m = __ballot_sync(0xffffffffu, look && d >= (c >= last_base ? P.n_jobs_last : P.n_jobs));
+                const int adv = m == 0xffffffffu ? 32 : __ffs(~(int)m) - 1;  // chunks done in a row
+                if (adv > 0) {
+                    any = true;
+                    next += adv;
+                    if (lane == 0) *freed = next;
+                }
+            }
+            if (any) {
+                t0 = gtimer();
+            } else {
+                if (__any_sync(0xffffffffu, *abort_flag || gtimer() - t0 > 2 * kTimeoutNs)) break;
+                __nanosleep(20);
+            }
+        }
+    } else {
+        if (warp == 0) {
+            // The whole warp looks at the next 32 chunks' ready counts with one load, and one
+            // lane issues the copies.  While it waits it counts the chunks that have landed
+            // in this SM (done), ahead of their MMAs, so that their place in the ring is
+            // free about two chunks earlier.
+            int it = 0, landed = 0;  // stages issued, stages seen landed
+            bool ok = true;
+            const int nbox = J.nbox, jv = J.v;
+            for (int w = 0; w < P.n_waves && ok; ++w) {
+                if (!has_job(w)) continue;
+                const int len = P.zv[w * P.V + jv].w;
+                const int base = P.wave_base[w], wlen = P.wave_base[w + 1] - base;
+                const int items = P.wave_items[w] * ((P.m.n_ant + Z_WARPS * P.ant_block - 1) / (Z_WARPS * P.ant_block));
+                if (lane == 0)  // (chunks past this job's sources)
+                    for (int q = len; q < wlen; ++q) red_add(P.done + base + q, 1);
+                int y[MAX_BOX], pl[MAX_BOX];
+#pragma unroll
+                for (int b = 0; b < MAX_BOX; ++b) {
+                    y[b] = jv * P.map_rows + J.row[b];
+                    pl[b] = J.plane[b];
+                }
+                int lq = 0, li = 0;  // chunk of the wave and stage of it that lands next
+                auto land = [&]() {
+                    if (landed >= it) return false;
+                    if (!__all_sync(0xffffffffu, mbar_test(full(landed % STAGES), (uint32_t)(landed / STAGES) & 1u))) return false;
+                    ++landed;
+                    if (++li == SPC) {
+                        if (lane == 0) red_add(P.done + base + lq, 1);
+                        li = 0;
+                        ++lq;
+                    }
+                    return true;
+                };
+                // spin on `ready` (warp-uniform) with the landings in between; false on a timeout
+                auto wait_for = [&](auto ready) {
+                    unsigned long long t0 = 0;
+                    for (unsigned n = 0; !ready(); ++n) {
+                        if (land()) continue;
+                        if ((n & 15u) == 15u) {  // (the clock is read now and then)
+                            const unsigned long long t = gtimer();
+                            if (t0 == 0) t0 = t;
+                            const bool late = t - t0 > kTimeoutNs;
+                            if (late && lane == 0) {
+                                *abort_flag = 1;
+                                atomicCAS(P.err, 0, (int)kDevTimeout);
+                            }
+                            if (__any_sync(0xffffffffu, late || *abort_flag)) return false;
+                        }
+                    }
+                    return true;
+                };
+                int have = 0;  // chunks of the wave known to be ready
+                for (int q = 0; q < len && ok; ++q) {
+                    if (q >= have) {
+                        ok = wait_for([&]() {
+                            const int c = q + lane;
+                            const int r = c < len ? ld_relaxed(P.ready + base + c) : 0;
+                            const unsigned m = __ballot_sync(0xffffffffu, r >= items);
+                            have = q + (m == 0xffffffffu ? 32 : __ffs(~(int)m) - 1);
+                            return have > q;
+                        });
+                        if (!ok) break;
+                        // the items' stores were released before they were counted; the
+                        // copies below read them from L2, never from this SM's L1
+                        asm volatile("fence.proxy.async.global;" ::: "memory");
+                    }
+                    const int x0 = ((base + q) % RC) * SPC * 64;
+#pragma unroll
+                    for (int i = 0; i < SPC; ++i) {
+                        const int s = it % STAGES;
+                        const uint32_t ph = ((uint32_t)(it / STAGES) & 1u) ^ 1u;
+                        ok = wait_for([&]() { return __all_sync(0xffffffffu, mbar_test(empty(s), ph)) != 0; });
+                        if (!ok) break;
+                        while (landed <= it - STAGES && land()) {}  // (the stage was consumed, so it has landed)
+                        if (elect_one()) {
+                            mbar_expect_tx(full(s), (uint32_t)(nbox * BOX));
+#pragma unroll
+                            for (int b = 0; b < MAX_BOX; ++b)
+                                if (b < nbox) tma_load_3d(sbase + s * STAGE + b * BOX, &map, x0 + i * 64, pl[b], y[b], full(s));
+                        }
+                        __syncwarp();
+                        ++it;
+                    }
+                }
+                if (ok) ok = wait_for([&]() { return landed >= it; });
+            }
+        } else if (warp == 1) {
+            // MMA: the whole warp walks the loop (so that descriptors and barriers stay
+            // in uniform registers), one elected lane issues.  With a single-lane loop an
+            // MMA took 72-83 cycles to issue, more than the 64 of an N = 128 one.
+            int it = 0, cg = 0;
+            bool ok = true;
+            const uint64_t da = sdesc(sbase + J.a * BOX), db = sdesc(sbase + J.b * BOX);
+            const uint32_t id = idesc_f16(true, 128, 128) + ((uint32_t)(jn > 128 ? 16 : 0) << 17);
+            const int jv = J.v, flush = P.flush;
+            for (int w = 0; w < P.n_waves && ok; ++w) {
+                if (!has_job(w)) continue;
+                const int len = P.zv[w * P.V + jv].w;
+                int ls = 0;
+                const uint32_t d = tmem_base;
+                for (int q = 0; q < len && ok; ++q) {
+#pragma unroll
+                    for (int i = 0; i < SPC; ++i) {
+                        if (ls == 0) {  // the epilogue has drained the accumulator
+                            if (!wait_bounded_spin(tempty, ((uint32_t)cg & 1u) ^ 1u, abort_flag, P.err)) ok = false;
+                            tc_fence_after();
+                        }
+                        const int s = it % STAGES;
+                        if (ok && !wait_bounded(full(s), (uint32_t)(it / STAGES) & 1u, abort_flag, P.err)) ok = false;
+                        ok = __all_sync(0xffffffffu, ok);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint32_t so = (uint32_t)s * (STAGE >> 4);
+                        const bool last = ls + 1 == flush || (q == len - 1 && i == SPC - 1);
+                        if (elect_one()) {
+#pragma unroll
+                            for (int kk = 0; kk < 2; ++kk) {
+                                // even blocks hold hi then lo, odd ones lo then hi
+                                const uint32_t oh = so + (i & 1 ? 4 : 0) + 2 * kk, ol = so + (i & 1 ? 0 : 4) + 2 * kk;
+                                const uint64_t ah = da + oh, al = da + ol, bh = db + oh, bl = db + ol;
+                                tc_mma_shared_a<true>(d, ah, bh, id, kk > 0 || ls > 0 ? 1u : 0u);
+                                tc_mma_shared_a<false>(d, ah, bl, id, 1);
+                                tc_mma(d, al, bh, id, 1);
+                            }
+                            tc_commit(empty(s));
+                            if (last) tc_commit(tfull);
+                        }
+                        __syncwarp();
+                        ++it;
+                        if (last) {
+                            ++cg;
+                            ls = 0;
+                        } else {
+                            ++ls;
+                        }
+                    }
+                }
+            }
+        } else {
+            // Z build
+            const int zi = warp - FIRST_Z;
+            AntPhase* const tab = reinterpret_cast<AntPhase*>(zsm + 2 * Z_BUF + zi * Z_APH_B);
+            ZOut o;
+            o.inst_b = (unsigned)(P.rows * zherk_row_bytes(NAX));
+            o.wa_pitch = P.wa_pitch;
+            o.wa_slot = (long long)P.m.n_beam * NC * P.wa_pitch;
+            // this lane's columns: even blocks of 32 hold hi then lo, odd ones lo then hi,
+            // so that the half warps of a store meet different banks
+            const int col = 2 * lane * NAX;
+            const unsigned blk_b = (unsigned)((col >> 5) * 128 + (col & 31) * 2);
+            const unsigned hi_b = blk_b + ((col >> 5) & 1) * 64, lo_b = blk_b + (((col >> 5) & 1) ^ 1) * 64;
+            int k = 0, owed = -1;  // owed: the buffer of the last item, whose barrier waits for this warp
+            bool ok = true;
+            for (int w = 0; w < P.n_waves && ok; ++w) {
+                const ZShare z = z_share(P, w, Z_WARPS * P.ant_block);
+                if (z.team < 0) continue;
+                const int base = P.wave_base[w], wlen = P.wave_base[w + 1] - base;
+                const ZherkGroup g = P.groups[P.wave_group0[w] + z.gi];
+                const int a0 = z.a0 + zi * P.ant_block, a1 = min(P.m.n_ant, a0 + P.ant_block);
+                o.scale = P.scale[g.slot];
+                const int per_e = g.uniform && g.n > 1 ? Z_BLOCK / 2 : Z_BLOCK;
+                __syncwarp();
+                {   // the antennas' phase factors, once per wave
+                    const AntPhase* t = P.aph + (long long)g.aph * P.n_phase * P.m.n_ant + a0;
+                    const int n16 = (a1 - a0) * 3;
+                    for (int i = lane; i < n16; i += 32) cp_async16(smem_u32(tab) + i * 16, (const uint4*)t + i);
+                    if (per_e < Z_BLOCK)
+                        for (int i = lane; i < n16; i += 32)
+                            cp_async16(smem_u32(tab + per_e) + i * 16, (const uint4*)(t + P.m.n_ant) + i);
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+                __syncwarp();
+                for (int q = z.team; q < wlen; q += z.teams, ++k) {
+                    const int cq = base + q, buf = k & 1;
+                    if (!wait_bounded(zfull(buf), (uint32_t)(k >> 1) & 1u, abort_flag, P.err)) ok = false;
+                    // the last item's stores have had the time since to drain
+                    if (owed >= 0 && lane == 0) mbar_arrive(zdone(owed));
+                    owed = -1;
+                    // the chunk whose place in the ring this one takes has been read by all
+                    if (__shfl_sync(0xffffffffu, *freed, 0) <= cq - RC) {
+                        const unsigned long long t0 = gtimer();
+                        while (__shfl_sync(0xffffffffu, *freed, 0) <= cq - RC) {
+                            __nanosleep(20);
+                            const bool late = gtimer() - t0 > kTimeoutNs;
+                            if (late && lane == 0) {
+                                *abort_flag = 1;
+                                atomicCAS(P.err, 0, (int)kDevTimeout);
+                            }
+                            if (__any_sync(0xffffffffu, *abort_flag || late)) { ok = false; break; }
+                        }
+                    }
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    if (q < g.len && a0 < a1) {
+                        const uint8_t* sm = zsm + buf * Z_BUF;
+                        unsigned S0[3], S1[3];
+                        float E0[3], E1[3];
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            const uint2 qv = *reinterpret_cast<const uint2*>(sm + c * (kZherkChunk * 4) + lane * 8);
+                            const float2 r2 = *reinterpret_cast<const float2*>(sm + (3 + c) * (kZherkChunk * 4) + lane * 8);
+                            S0[c] = qv.x; S1[c] = qv.y;
+                            E0[c] = r2.x; E1[c] = r2.y;
+                        }
+                        uint8_t* at = P.ring + (unsigned long long)(unsigned)g.v0 * o.inst_b + (unsigned)((cq % RC) * (kZherkChunk * NAX * 4));
+                        o.hi = at + hi_b;
+                        o.lo = at + lo_b;
+                        o.wa = P.wa + (long long)g.slot * o.wa_slot + (g.c0 + q) * kZherkChunk + 2 * lane;
+                        o.ws = reinterpret_cast<const float4*>(sm + Z_SRC_B) + lane;
+                        for (int a = a0; a < a1; ++a)
+                            z_ant<FORM, NAX, NFD, ONE>(P, g, o, tab + (a - a0), per_e, a, S0, S1, E0, E1);
+                    }
+                    __syncwarp();
+                    owed = buf;
+                }
+            }
+            if (owed >= 0 && lane == 0) mbar_arrive(zdone(owed));
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    if (*abort_flag) {
+        // let copies and MMAs already issued land before TMEM and smem go away
+        const unsigned long long t0 = gtimer();
+        while (gtimer() - t0 < 2000000ull) {}
+    }
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS));
+    }
+}
+
+// Per launch: the order of the instances (by_length: by decreasing live count),
+// the FP16 scale of every instance (one power of two for all instances of one
+// time, from the largest |WA| among them), the source range of every virtual
+// instance and group, and the chunk ranges of the waves.
+__global__ void __launch_bounds__(1024) k_zherk_prep(ZherkArgs P, const float* __restrict__ amax_in,
+                                                     float* __restrict__ amax_out, float* __restrict__ scale,
+                                                     int4* __restrict__ zv, int* __restrict__ wave_base,
+                                                     ZherkGroup* __restrict__ groups, int n_groups, int by_length) {
+    extern __shared__ int sm[];  // t, live count and max |WA| of each instance, then the waves' lengths
+    int *st = sm, *sk = sm + P.n_inst, *order = sm + 3 * P.n_inst, *len = sm + 4 * P.n_inst;
+    float* sa = reinterpret_cast<float*>(sm + 2 * P.n_inst);
+    for (int w = threadIdx.x; w < P.n_waves; w += blockDim.x) len[w] = 0;
+    for (int i = threadIdx.x; i < P.n_inst; i += blockDim.x) {
+        st[i] = P.inst[P.inst0 + i].t;
+        sk[i] = P.lt.n_live[st[i]];
+        sa[i] = amax_in[i];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < P.n_inst; i += blockDim.x) {
+        const int ti = st[i], ki = sk[i];
+        int rank = 0;
+        float mx = 0.f;
+        for (int j = 0; j < P.n_inst; ++j) {
+            rank += (sk[j] > ki) || (sk[j] == ki && j < i);
+            if (st[j] == ti) mx = fmaxf(mx, sa[j]);
+        }
+        if (by_length) order[rank] = i;
+        else order[i] = i;
+        amax_out[i] = mx;
+        scale[i] = ldexpf(1.f, fp16_scale_exp(mx));
+    }
+    __syncthreads();
+    const int total = P.n_inst * P.S;
+    for (int vi = threadIdx.x; vi < total; vi += blockDim.x) {
+        const int ks = vi / P.n_inst, slot = order[vi - ks * P.n_inst];
+        const int nch = (sk[slot] + kZherkChunk - 1) / kZherkChunk;
+        const int c0 = (int)((long long)nch * ks / P.S), c1 = (int)((long long)nch * (ks + 1) / P.S);
+        zv[vi] = make_int4(slot, st[slot], c0, c1 - c0);
+        atomicMax(&len[vi / P.V], c1 - c0);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < n_groups; i += blockDim.x) {
+        ZherkGroup g = groups[i];
+        const int4 v = zv[g.vi];
+        g.slot = v.x;
+        g.t = v.y;
+        g.c0 = v.z;
+        g.len = v.w;
+        if (by_length) g.aph = v.x;
+        groups[i] = g;
+    }
+    if (threadIdx.x == 0) {
+        int acc = 0;
+        for (int w = 0; w < P.n_waves; ++w) {
+            wave_base[w] = acc;
+            acc += len[w];
+        }
+        wave_base[P.n_waves] = acc;
+    }
+}
+
+// Sum of the S partial tiles at p (stride 128 x 128), element i.
+__device__ __forceinline__ float sum_parts(const float* p, int S, int i) {
+    float v = p[i];
+    for (int k = 1; k < S; ++k) v += p[(long long)k * (128 * 128) + i];
+    return v;
+}
+
+// V from the partial tiles of the real form: one block per 64 x 64 piece of a
+// tile (32 x 32 antenna-feeds), read along the tile's rows and written along
+// the rows of V through shared memory.
+__global__ void __launch_bounds__(256) k_zherk_final_real(ZherkFinalArgs a) {
+    __shared__ float G[64][65];  // [column][row]
+    const int slot = blockIdx.x / a.n_tiles, tile = blockIdx.x - slot * a.n_tiles;
+    const ZherkTile t = a.tiles[tile];
+    const int br = (blockIdx.y & 1) * 64, bc = (blockIdx.y >> 1) * 64;
+    const float* p = a.partial + ((long long)slot * a.n_tiles + tile) * a.S * (128 * 128);
+    // the product's rows and columns this piece stands for
+    const int pr = t.r0 + (t.trans ? bc : br), pc = t.c0 + (t.trans ? br : bc);
+    int rlim = 2 * a.N, clim = 2 * a.N;
+    if (a.limits) {
+        rlim = min(rlim, a.limits[tile].x);
+        clim = min(clim, a.limits[tile].y);
+    }
+    if (pr >= rlim || pc >= clim || (!a.ho.uidx && pr + 63 < pc)) return;
+    for (int i = threadIdx.x; i < 64 * 64; i += 256) {
+        const int r = i & 63, c = i >> 6;
+        G[c][r] = sum_parts(p, a.S, (bc + c) * 128 + br + r);
+    }
+    __syncthreads();
+    const float us = ldexpf(1.f, -fp16_scale_exp(a.amax[slot]));
+    float2* Vb = a.V + a.inst[a.inst0 + slot].v_off;
+    auto entry = [&](int i, int j) {  // product entry (row, column) of the piece
+        return t.trans ? G[i][j] : G[j][i];
+    };
+    const bool diag = t.r0 == t.c0;
+    for (int pass = 0; pass < (a.ho.uidx ? 1 : 2); ++pass)
+        for (int k = threadIdx.x; k < 32 * 32; k += 256) {
+            // pass 0: along the rows of V; pass 1: the mirror image, along its rows
+            const int x = k & 31, y = k >> 5;
+            const int ia = pass ? x : y, ib = pass ? y : x;
+            const int A = (pr >> 1) + ia, B = (pc >> 1) + ib;
+            if (2 * A >= rlim || 2 * B >= clim) continue;
+            const float g00 = entry(2 * ia, 2 * ib), g01 = entry(2 * ia, 2 * ib + 1);
+            const float g10 = entry(2 * ia + 1, 2 * ib), g11 = entry(2 * ia + 1, 2 * ib + 1);
+            const float re = ((g00 + g11) * us) * us;
+            const float im = A == B ? 0.f : ((g10 - g01) * us) * us;
+            if (a.ho.uidx) {
+                const int nf = a.ho.n_feed;
+                const int aa = A / nf, pa = A - aa * nf, bb = B / nf, pb = B - bb * nf;
+                const int e = a.ho.uidx[aa * a.ho.n_ant + bb];
+                if (e < 0) continue;
+                const int grp = e >> 1;
+                const bool cj = (e & 1) != 0;
+                Vb[((long long)grp * nf + (cj ? pb : pa)) * nf + (cj ? pa : pb)] = make_float2(re, cj ? -im : im);
+                continue;
+            }
+            if (diag && A < B) continue;  // a diagonal tile's upper half is the mirror
+            if (pass == 0) Vb[(long long)A * a.N + B] = make_float2(re, im);
+            else if (A != B) Vb[(long long)B * a.N + A] = make_float2(re, -im);
+        }
+}
+
+// V from the partial tiles of the gauss form: one block per 32 x 32 piece of a
+// 128 x 128 block (i, j), i >= j, of V.
+__global__ void __launch_bounds__(256) k_zherk_final_gauss(ZherkFinalArgs a) {
+    __shared__ float M[3][32][33];  // F_ab, F_ba, H_ab at [row of a][row of b]
+    const int nb = a.np * (a.np + 1) / 2;
+    const int slot = blockIdx.x / nb;
+    int i = 0, j = blockIdx.x - slot * nb;
+    while (j > i) j -= ++i;
+    const int ar = (blockIdx.y & 3) * 32, bc = (blockIdx.y >> 2) * 32;
+    const int A0 = i * 128 + ar, B0 = j * 128 + bc;
+    if (A0 >= a.N || B0 >= a.N || A0 + 31 < B0) return;
+    const float* base = a.partial + (long long)slot * a.n_tiles * a.S * (128 * 128);
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+        const int tile = m == 0 ? a.tile_of[i * a.np + j] : m == 1 ? a.tile_of[j * a.np + i] : a.tile_of[(a.np + i) * a.np + j];
+        const ZherkTile t = a.tiles[tile];
+        const float* p = base + (long long)tile * a.S * (128 * 128);
+        // the tile's rows run along a (M = F_ab, H_ab) unless it is F_ba or transposed
+        const bool row_is_a = (m != 1) == (t.trans == 0);
+        for (int k = threadIdx.x; k < 32 * 32; k += 256) {
+            const int r = k & 31, c = k >> 5;
+            const float v = sum_parts(p, a.S, row_is_a ? (bc + c) * 128 + ar + r : (ar + c) * 128 + bc + r);
+            if (row_is_a) M[m][r][c] = v;
+            else M[m][c][r] = v;
+        }
+    }
+    __syncthreads();
+    const float us = ldexpf(1.f, -fp16_scale_exp(a.amax[slot]));
+    float2* Vb = a.V + a.inst[a.inst0 + slot].v_off;
+    for (int pass = 0; pass < 2; ++pass)
+        for (int k = threadIdx.x; k < 32 * 32; k += 256) {
+            const int x = k & 31, y = k >> 5;
+            const int ia = pass ? x : y, ib = pass ? y : x;
+            const int A = A0 + ia, B = B0 + ib;
+            if (A >= a.N || B >= a.N || A < B) continue;
+            const float f = M[0][ia][ib], ft = M[1][ia][ib];
+            const float re = ((M[2][ia][ib] - (f + ft)) * us) * us;
+            const float im = A == B ? 0.f : ((ft - f) * us) * us;
+            if (pass == 0) Vb[(long long)A * a.N + B] = make_float2(re, im);
+            else if (A != B) Vb[(long long)B * a.N + A] = make_float2(re, -im);
+        }
+}
+
+// The ring as [rows][planes][columns]: one plane of 2N-row instances (real), or
+// the planes X, Y and S of every antenna-feed (gauss).
+bool ring_map(CUtensorMap* map, const void* ring, int row_b, int planes, long long rows) {
+    EncodeTiledFn enc = get_encode();
+    if (!enc) return false;
+    cuuint64_t dims[3] = {(cuuint64_t)row_b / 2, (cuuint64_t)planes, (cuuint64_t)rows};
+    cuuint64_t strides[2] = {(cuuint64_t)row_b, (cuuint64_t)row_b * planes};
+    cuuint32_t box[3] = {64, 1, 128};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(ring), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+}  // namespace
+
+cudaError_t zherk_init() {
+    cudaError_t e = cudaSuccess;
+    auto set = [&](auto* k, int nc) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_for(nc));
+    };
+#define MV_SET(F, A, D) set(k_zherk<F, A, D, false>, A * D), set(k_zherk<F, A, D, true>, A * D)
+    MV_SET(kZherkReal, 1, 1);
+    MV_SET(kZherkReal, 1, 2);
+    MV_SET(kZherkReal, 2, 1);
+    MV_SET(kZherkReal, 2, 2);
+    MV_SET(kZherkGauss, 1, 1);
+    MV_SET(kZherkGauss, 1, 2);
+    MV_SET(kZherkGauss, 2, 1);
+    MV_SET(kZherkGauss, 2, 2);
+#undef MV_SET
+    return e;
+}
+
+cudaError_t launch_zherk_prep(const ZherkArgs& P, const float* amax_in, float* amax_out, float* scale, int4* zv,
+                              int* wave_base, ZherkGroup* groups, int n_groups, bool by_length, cudaStream_t st,
+                              long long* launches) {
+    k_zherk_prep<<<1, 1024, sizeof(int) * (size_t)(P.n_waves + 4 * P.n_inst), st>>>(P, amax_in, amax_out, scale, zv,
+                                                                                   wave_base, groups, n_groups, by_length);
+    *launches += 1;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_zherk(const ZherkArgs& P, int form, int n_ctas, cudaStream_t st, long long* launches) {
+    CUtensorMap map;
+    if (!ring_map(&map, P.ring, zherk_row_bytes(P.m.n_ax), P.rows / P.map_rows, (long long)P.V * P.map_rows)) return cudaErrorInvalidValue;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)n_ctas);
+    const int nc = P.m.n_ax * P.m.n_feed;
+    cfg.blockDim = dim3((unsigned)threads_for(nc));
+    cfg.dynamicSmemBytes = (size_t)smem_for(nc);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    *launches += 1;
+#define MV_ZK(F, A, D)                                                                       \
+    if (form == F && P.m.n_ax == A && P.m.n_feed == D)                                       \
+        return P.m.n_beam == 1 ? cudaLaunchKernelEx(&cfg, k_zherk<F, A, D, true>, map, P)    \
+                               : cudaLaunchKernelEx(&cfg, k_zherk<F, A, D, false>, map, P)
+    MV_ZK(kZherkReal, 1, 1);
+    MV_ZK(kZherkReal, 1, 2);
+    MV_ZK(kZherkReal, 2, 1);
+    MV_ZK(kZherkReal, 2, 2);
+    MV_ZK(kZherkGauss, 1, 1);
+    MV_ZK(kZherkGauss, 1, 2);
+    MV_ZK(kZherkGauss, 2, 1);
+    MV_ZK(kZherkGauss, 2, 2);
+#undef MV_ZK
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_zherk_final(const ZherkFinalArgs& a, int form, cudaStream_t st, long long* launches) {
+    if (form == kZherkReal)
+        k_zherk_final_real<<<dim3((unsigned)(a.n_inst * a.n_tiles), 4), 256, 0, st>>>(a);
+    else
+        k_zherk_final_gauss<<<dim3((unsigned)(a.n_inst * (a.np * (a.np + 1) / 2)), 16), 256, 0, st>>>(a);
+    *launches += 1;
+    return cudaGetLastError();
+}
+
+// ------------------------------------------------------------ host planning
+std::vector<ZherkTile> zherk_triangle(int rows) {
+    std::vector<ZherkTile> t;
+    for (int r = 0; r < rows; r += 128)
+        for (int k = 0; k <= r; k += 128) t.push_back(ZherkTile{r, k, r, k, 0, 0});
+    return t;
+}
+
+namespace {
+
+// Pair up products that share a panel: that panel is A, the other two B (N =
+// 256).  The products are edges between panels (loops on the diagonal); in a
+// depth-first walk every vertex pairs the edges it has not handed on and gives
+// an odd one the edge to its parent, so at most one product per connected
+// component stays alone.
+void make_jobs(std::vector<ZherkTile>& tiles, int plane_rows, std::vector<ZherkJob>& out) {
+    std::vector<int> rows;  // vertices: first rows of panels
+    auto vertex = [&](int row) {
+        for (size_t i = 0; i < rows.size(); ++i)
+            if (rows[i] == row) return (int)i;
+        rows.push_back(row);
+        return (int)rows.size() - 1;
+    };
+    const int T = (int)tiles.size();
+    std::vector<int> u(T), v(T);
+    for (int i = 0; i < T; ++i) {
+        u[i] = vertex(tiles[i].ra);
+        v[i] = vertex(tiles[i].rb);
+    }
+    const int n = (int)rows.size();
+    std::vector<std::vector<int>> inc(n);
+    for (int i = 0; i < T; ++i) {
+        inc[u[i]].push_back(i);
+        if (v[i] != u[i]) inc[v[i]].push_back(i);
+    }
+    std::vector<char> seen(n, 0), used(T, 0);
+    auto emit = [&](int at, int e0, int e1) {  // products e0 and e1 (or -1) with A = panel `at`
+        ZherkJob J{};
+        auto box = [&](int row) {
+            J.row[J.nbox] = row % plane_rows;
+            J.plane[J.nbox] = row / plane_rows;
+            return J.nbox++;
+        };
+        auto other = [&](int e) {  // the B panel of product e; turns it round if A was its B
+            if (u[e] != at) {
+                std::swap(tiles[e].ra, tiles[e].rb);
+                std::swap(u[e], v[e]);
+                tiles[e].trans = 1;
+            }
+            used[e] = 1;
+            return v[e];
+        };
+        const int b0 = other(e0), b1 = e1 >= 0 ? other(e1) : -1;
+        J.b = box(rows[b0]);
+        J.tile[0] = e0;
+        J.n = 128;
+        if (b1 >= 0) {
+            box(rows[b1]);
+            J.tile[1] = e1;
+            J.n = 256;
+        }
+        J.a = b0 == at ? 0 : b1 == at ? 1 : box(rows[at]);
+        out.push_back(J);
+    };
+    // depth-first order with parents
+    std::vector<int> order, parent_edge(n, -1);
+    for (int s = 0; s < n; ++s) {
+        if (seen[s]) continue;
+        std::vector<int> stack{s};
+        seen[s] = 1;
+        while (!stack.empty()) {
+            const int x = stack.back();
+            stack.pop_back();
+            order.push_back(x);
+            for (int e : inc[x]) {
+                const int y = u[e] == x ? v[e] : u[e];
+                if (!seen[y]) {
+                    seen[y] = 1;
+                    parent_edge[y] = e;
+                    stack.push_back(y);
+                }
+            }
+        }
+    }
+    for (int k = n - 1; k >= 0; --k) {
+        const int x = order[k];
+        std::vector<int> free;
+        for (int e : inc[x])
+            if (!used[e] && e != parent_edge[x]) free.push_back(e);
+        if (free.size() % 2 && parent_edge[x] >= 0 && !used[parent_edge[x]]) free.push_back(parent_edge[x]);
+        for (size_t i = 0; i < free.size(); i += 2) emit(x, free[i], i + 1 < free.size() ? free[i + 1] : -1);
+    }
+}
+
+}  // namespace
+
+bool zherk_plan(int N, const std::vector<ZherkTile>& cover, int n_ax, int n_inst, double est_live, int n_sms,
+                long long ring_budget, ZherkPlan& out) {
+    if (n_inst < 1) return false;
+    const double chunks = std::max(1.0, std::ceil(est_live / kZherkChunk));
+    double best = 1e300;
+    for (int form = kZherkReal; form <= (cover.empty() ? kZherkGauss : kZherkReal); ++form) {
+        ZherkPlan z;
+        z.form = form;
+        z.n_ax = n_ax;
+        if (form == kZherkReal) {
+            z.rows = 2 * N;
+            z.tiles = cover.empty() ? zherk_triangle(z.rows) : cover;
+        } else {
+            z.rows = 3 * N;
+            for (int i = 0; i < N; i += 128)
+                for (int j = 0; j < N; j += 128) z.tiles.push_back(ZherkTile{i, N + j, i, j, 0, 0});
+            for (int i = 0; i < N; i += 128)
+                for (int j = 0; j <= i; j += 128) z.tiles.push_back(ZherkTile{2 * N + i, 2 * N + j, i, j, 1, 0});
+        }
+        if ((int)z.tiles.size() > 2 * n_sms) continue;
+        std::vector<ZherkJob> one;  // the jobs of one instance
+        make_jobs(z.tiles, form == kZherkReal ? z.rows : N, one);
+        const int nj = (int)one.size(), T = (int)z.tiles.size();
+        const int vcap = (int)std::min<long long>(n_sms / nj, ring_budget / ((long long)zherk_row_bytes(n_ax) * z.rows));
+        if (vcap < 1) continue;
+        for (int S = 1; S <= 64 && (S == 1 || chunks / S >= 4); ++S) {
+            const int total = n_inst * S, V = std::min(vcap, total), waves = (total + V - 1) / V;
+            if (waves > kZherkMaxWaves) continue;
+            // us: a chunk of a job (its MMAs at about 80 % of the tensor rate; the Z build
+            // where a wave has few products), a wave's ramp, and the partial tiles written and read once
+            const double t = waves * (chunks / S * n_ax * 0.95 + 6.0) + total * (double)T * 131072.0 / 4e6;
+            if (t < best) {
+                best = t;
+                out = z;
+                out.V = V;
+                out.S = S;
+                out.waves = waves;
+                out.jobs.clear();
+                for (int v = 0; v < V; ++v)
+                    for (ZherkJob J : one) {
+                        J.v = v;
+                        out.jobs.push_back(J);
+                    }
+                out.n_jobs = nj * V;
+                out.n_jobs_last = nj * (total - (waves - 1) * V);
+            }
+        }
+    }
+    if (best == 1e300) return false;
+    out.jobs.resize(n_sms, ZherkJob{});
+    return true;
+}
+
+int zherk_ant_block(const ZherkPlan& z, int n_ant, int nc, int groups, int chan, int n_sms) {
+    const int most = chan > 1 ? Z_BLOCK / 2 : Z_BLOCK;
+    const int ring_chunks = zherk_ring_chunks(z.n_ax);
+    int best = 0;
+    double t_best = 1e300;
+    for (int ab = 1; ab <= most; ++ab) {
+        const int ants = z_warps(nc) * ab, teams = n_sms / (groups * ((n_ant + ants - 1) / ants));
+        if (teams < 1) continue;
+        // cycles per chunk: an item's fixed part and its antennas, over the chunks in
+        // flight, which have to leave the tensor side a few chunks of the ring
+        double t = (800.0 + ab * (250.0 + 110.0 * chan)) / teams;
+        if (teams > ring_chunks / 2) t *= 1.0 + 0.5 * (teams - ring_chunks / 2);
+        if (t < t_best) {
+            t_best = t;
+            best = ab;
+        }
+    }
+    return best;
+}
+
+}  // namespace mv
