@@ -417,12 +417,33 @@ struct Prepared {
     HerkOut ho{};             // unique output: group lookup and tile lists (ho.tl set per tile width)
     bool stream = false;      // the streamed schedule (zherk_tc.cu)
     std::vector<StreamBatch> sb;
+    Fp32Plan f32;             // (FP32) form, products and split of the HERK
+    size_t f32_tiles = 0, f32_tile_of = 0;  // its tables in ztab
+    int f32_slots = 0;        // instances per HERK launch (its partial tiles stay within kPartialBytes)
     int sflush = 8;           // (stream) 32-column stages per TMEM flush
 };
 
 // Bytes the ring of Z may take: it has to stay in L2 (129 MB over two dies) beside
 // the WA tables in flight.
 constexpr long long kRingBytes = 96ll << 20;
+
+// Partial tiles of one FP32 HERK launch (at least one instance's).
+constexpr long long kPartialBytes = 1ll << 30;
+
+// Where the product of panels (i, j) of F (kind 0) and H (kind 1) is in a gauss tile list.
+std::vector<int> gauss_tile_of(const std::vector<ZherkTile>& tiles, int np) {
+    std::vector<int> of(2 * np * np, 0);
+    for (size_t k = 0; k < tiles.size(); ++k) of[(tiles[k].kind * np + tiles[k].r0 / 128) * np + tiles[k].c0 / 128] = (int)k;
+    return of;
+}
+
+// Appends d to a table buffer at a 16-byte boundary; its offset.
+size_t put_table(std::vector<uint8_t>& tab, const void* d, size_t bytes) {
+    const size_t at = (tab.size() + 15) / 16 * 16;
+    tab.resize(at + bytes);
+    std::memcpy(tab.data() + at, d, bytes);
+    return at;
+}
 
 // Plan the streamed schedule: batches of consecutive instances (whose WA tables
 // fit the budget), and for each the jobs, channel groups and Z items of its
@@ -457,12 +478,7 @@ bool plan_stream(mv_ctx* c, Plan& P, Prepared& p, std::vector<uint8_t>& tab) {
     P.batches.clear();
     p.sb.clear();
     p.max_slots = 0;
-    auto put = [&](const void* d, size_t bytes) {
-        const size_t at = (tab.size() + 15) / 16 * 16;
-        tab.resize(at + bytes);
-        std::memcpy(tab.data() + at, d, bytes);
-        return at;
-    };
+    auto put = [&](const void* d, size_t bytes) { return put_table(tab, d, bytes); };
     for (int i0 = 0; i0 < p.n_inst; i0 += B) {
         const int n = std::min(B, p.n_inst - i0);
         const ZherkPlan* z = plan_for(n);
@@ -514,11 +530,7 @@ bool plan_stream(mv_ctx* c, Plan& P, Prepared& p, std::vector<uint8_t>& tab) {
         b.tiles = put(z->tiles.data(), z->tiles.size() * sizeof(ZherkTile));
         b.np = (p.N + 127) / 128;
         if (z->form == kZherkGauss) {
-            std::vector<int> of(2 * b.np * b.np, 0);
-            for (size_t k = 0; k < z->tiles.size(); ++k) {
-                const ZherkTile& t = z->tiles[k];
-                of[(t.kind * b.np + t.r0 / 128) * b.np + t.c0 / 128] = (int)k;
-            }
+            const std::vector<int> of = gauss_tile_of(z->tiles, b.np);
             b.tile_of = put(of.data(), of.size() * sizeof(int));
         }
         if (covered) {
@@ -735,7 +747,19 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
         if ((s = ensure(c, c->zamax, sizeof(float) * max_slots))) return s;
         if ((s = ensure(c, c->zorder, sizeof(int4) * vinsts))) return s;
     }
-    const size_t plane_elems = (size_t)p.rows * p.k_pitch * max_slots;
+    if (p.zprec == 0) {
+        p.f32 = herk_fp32_plan(p.N, m.n_ax, max_slots, 0.5 * (double)m.n_src, c->n_sms);
+        const size_t slot = sizeof(float) * 128 * 128 * p.f32.tiles.size() * p.f32.split;
+        p.f32_slots = (int)std::max(1ll, std::min<long long>(max_slots, kPartialBytes / (long long)slot));
+        p.f32_tiles = put_table(ztab, p.f32.tiles.data(), p.f32.tiles.size() * sizeof(ZherkTile));
+        if (p.f32.form == kZherkGauss) {
+            const std::vector<int> of = gauss_tile_of(p.f32.tiles, (p.N + 127) / 128);
+            p.f32_tile_of = put_table(ztab, of.data(), of.size() * sizeof(int));
+        }
+        if ((s = upload(c, c->ztab, ztab.data(), ztab.size(), st))) return s;
+        if ((s = ensure(c, c->partial, slot * p.f32_slots))) return s;
+    }
+    const size_t plane_elems = (size_t)(p.zprec == 0 ? p.f32.rows : p.rows) * p.k_pitch * max_slots;
     for (int k = 0; k < p.nbuf && !p.stream; ++k) {
         if (p.zprec == 0) {
             if ((s = ensure(c, c->u[k], sizeof(float) * plane_elems))) return s;
@@ -792,9 +816,32 @@ cudaError_t enqueue_herk(mv_ctx* c, const Prepared& p, const Plan::Batch& b, con
         ho.tl = c->red.kind == 0 ? nullptr : (const TileDesc*)c->red_tl[w].p;
         ho.n_tl = c->red.kind == 0 ? 0 : c->red_ntl[w];
     }
-    if (p.zprec == 0)
-        return launch_herk_fp32(d_inst, b.inst0, b.n, p.lt, c->model.n_ax, (const float*)c->u[k].p, p.rows,
-                                p.k_pitch, p.Vout, p.N, 256, st, L);
+    if (p.zprec == 0) {
+        const uint8_t* tab = (const uint8_t*)c->ztab.p;
+        const ZherkTile* tiles = (const ZherkTile*)(tab + p.f32_tiles);
+        const int n_tiles = (int)p.f32.tiles.size();
+        cudaError_t e = cudaSuccess;
+        for (int i = 0; i < b.n && e == cudaSuccess; i += p.f32_slots) {
+            ZherkFinalArgs f{};
+            f.inst = d_inst;
+            f.inst0 = b.inst0 + i;
+            f.n_inst = std::min(p.f32_slots, b.n - i);
+            f.partial = (const float*)c->partial.p;
+            f.tiles = tiles;
+            f.tile_of = (const int*)(tab + p.f32_tile_of);
+            f.n_tiles = n_tiles;
+            f.S = p.f32.split;
+            f.N = p.N;
+            f.np = (p.N + 127) / 128;
+            f.V = p.Vout;
+            e = launch_herk_fp32(d_inst, f.inst0, f.n_inst, p.lt, c->model.n_ax,
+                                 (const float*)c->u[k].p + (size_t)i * p.f32.rows * p.k_pitch, p.f32.rows,
+                                 p.f32.plane_rows, p.k_pitch, tiles, n_tiles, p.f32.split, (float*)c->partial.p,
+                                 (int*)c->err.p, st, L);
+            if (e == cudaSuccess) e = launch_zherk_final(f, p.f32.form, st, L);
+        }
+        return e;
+    }
     return launch_herk_tc(d_inst, b.inst0, b.n, p.lt, c->model.n_ax, (const __nv_bfloat16*)c->u[k].p,
                           (const __nv_bfloat16*)c->ulo[k].p, p.rows, p.k_pitch, p.max_slots, p.zprec == 2 ? 1 : 0,
                           (const float*)c->amax[kw].p, p.Vout, p.N, h.flush, h.split, h.bn, c->n_sms, (int*)c->sched.p,
@@ -863,7 +910,8 @@ mv_status enqueue_zside(mv_ctx* c, const Prepared& p, const Plan::Batch& b, int 
     Timed tz(c, MV_KERNEL_ZBUILD, st);
     cudaError_t e = launch_zbuild(m, d_inst, (const Chan*)c->chan.p, (const ZGroup*)c->groups.p, b.g0, b.ng, p.lt,
                       (const float2*)c->wa[k].p, p.pitch, (float*)c->amax[k].p, c->u[k].p, c->ulo[k].p,
-                      p.zprec, p.rows, p.k_pitch, p.nbuf == 2 && !p.fuse ? 4 * c->n_sms : 0, (AntPhase*)c->aph[k].p,
+                      p.zprec == 0 && p.f32.form == kZherkGauss ? 1 : p.zprec, p.zprec == 0 ? p.f32.rows : p.rows,
+                      p.k_pitch, p.nbuf == 2 && !p.fuse ? 4 * c->n_sms : 0, (AntPhase*)c->aph[k].p,
                       p.n_phase, st, L);
     tz.end();
     return launched(e, "Z build", st);
@@ -1111,6 +1159,9 @@ std::vector<long long> graph_key(mv_ctx* c, const Plan& P, const Prepared& p, co
         k.push_back(b.ng);
     }
     k.push_back(p.stream ? p.sflush : 0);
+    for (long long x : {(long long)p.f32.form, (long long)p.f32.rows, (long long)p.f32.split, (long long)p.f32.tiles.size(),
+                        (long long)p.f32_slots, (long long)p.f32_tiles, (long long)p.f32_tile_of})
+        k.push_back(x);
     k.push_back(P.pairs ? 1 : 0);
     k.push_back(p.n_phase);
     for (const StreamBatch& b : p.sb)
@@ -1397,7 +1448,7 @@ mv_status mv_create(mv_ctx** out, int device, const mv_options* opt) {
     mv_ctx* c = new mv_ctx();
     c->device = device;
     c->n_sms = pr.multiProcessorCount;
-    if (herk_tc_init() != cudaSuccess || zherk_init() != cudaSuccess || mlp_tc_init() != cudaSuccess || gemm_tc_init() != cudaSuccess ||
+    if (herk_tc_init() != cudaSuccess || zherk_init() != cudaSuccess || herk_fp32_init() != cudaSuccess || mlp_tc_init() != cudaSuccess || gemm_tc_init() != cudaSuccess ||
         mlp_chain_init() != cudaSuccess || wgrad_tc_init() != cudaSuccess) {
         cudaGetLastError();
         delete c;

@@ -185,9 +185,6 @@ cudaError_t launch_zbuild(const Model& m, const Inst* d_inst, const Chan* d_chan
                           float* d_amax, void* d_u, void* d_u_lo, int prec, int rows,
                           long long k_pitch, int max_blocks, AntPhase* d_aph, int n_phase, cudaStream_t st,
                           long long* launches);
-cudaError_t launch_herk_fp32(const Inst* d_inst, int inst0, int n_inst, LiveTables lt, int n_ax,
-                             const float* d_u, int rows, long long k_pitch, float2* d_v, int N,
-                             int flush_k, cudaStream_t st, long long* launches);
 // Persistent tensor-core HERK over n_inst instance slots: tiles 128 x bn
 // (bn = 128 or 256), the source axis split `split` ways (split > 1 writes
 // 128 x bn FP32 partial tiles, summed by a finalize kernel), TMEM flushed into

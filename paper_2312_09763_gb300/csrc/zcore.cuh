@@ -110,9 +110,11 @@ __device__ __forceinline__ void put_row(void* pu, void* pl, const float* v) {
 // channels are loaded together.
 constexpr int kAnchor = 8, kPrefetch = 4;
 
-// Element type of the U planes.
-template <int PREC> struct Plane { using T = uint16_t; };
-template <> struct Plane<0> { using T = float; };
+// PREC: 0 FP32, rows Re and Im of every antenna-feed in turn; 1 FP32, the
+// planes X = Re Z, Y = Im Z and X + Y of N rows each; 2 FP16 hi and lo planes,
+// rows as with 0.  Element type of the U planes.
+template <int PREC> struct Plane { using T = float; };
+template <> struct Plane<2> { using T = uint16_t; };
 
 // One work item (bx, by, group g) of nthr threads: thread tid builds the two
 // adjacent sources 2 (bx nthr + tid) and +1 (columns 2 n_ax wide) for antennas
@@ -152,14 +154,14 @@ __device__ __forceinline__ void zbuild_item(const Model& m, const Inst* __restri
     }
     const long long col = (long long)s0 * NAX;
     T* const ub = static_cast<T*>(u) + g.slot0 * slot_stride + col;
-    T* const lb = PREC != 0 ? static_cast<T*>(ulo) + g.slot0 * slot_stride + col : nullptr;
+    T* const lb = PREC == 2 ? static_cast<T*>(ulo) + g.slot0 * slot_stride + col : nullptr;
     const float2* const wb = wa + g.slot0 * wa_slot + s0;
     const bool step = g.uniform && g.n > 1;
     const float sc = PREC == 2 ? scale[0] : 1.f;
     for (int a = a_begin; a < a_end; ++a) {
         const float2* w = wb + (long long)m.beam_idx[a] * (NFD * NAX) * wa_pitch;
-        T* ur = ub + 2ll * a * NFD * k_pitch;
-        T* lr = PREC != 0 ? lb + 2ll * a * NFD * k_pitch : nullptr;
+        T* ur = ub + (PREC == 1 ? 1ll : 2ll) * a * NFD * k_pitch;
+        T* lr = PREC == 2 ? lb + 2ll * a * NFD * k_pitch : nullptr;
         // WA of the two sources for the group's instance w + jrel: one 16-byte load
         // per component (s0 is even)
         constexpr int NC = NFD * NAX;
@@ -183,12 +185,22 @@ __device__ __forceinline__ void zbuild_item(const Model& m, const Inst* __restri
                     re[NAX + k] = fmaf(a4.y, c1, a4.w * sn1);
                     im[NAX + k] = fmaf(a4.w, c1, -a4.y * sn1);
                 }
-                const long long r0 = 2ll * p * k_pitch;
-                put_row<PREC, NAX>(ur + r0, PREC != 0 ? lr + r0 : nullptr, re);
-                put_row<PREC, NAX>(ur + r0 + k_pitch, PREC != 0 ? lr + r0 + k_pitch : nullptr, im);
+                if constexpr (PREC == 1) {
+                    const long long r0 = p * k_pitch, plane = (long long)m.n_ant * NFD * k_pitch;
+                    float sum[2 * NAX];
+#pragma unroll
+                    for (int k = 0; k < 2 * NAX; ++k) sum[k] = re[k] + im[k];
+                    put_row<0, NAX>(ur + r0, nullptr, re);
+                    put_row<0, NAX>(ur + r0 + plane, nullptr, im);
+                    put_row<0, NAX>(ur + r0 + 2 * plane, nullptr, sum);
+                } else {
+                    const long long r0 = 2ll * p * k_pitch;
+                    put_row<PREC, NAX>(ur + r0, PREC == 2 ? lr + r0 : nullptr, re);
+                    put_row<PREC, NAX>(ur + r0 + k_pitch, PREC == 2 ? lr + r0 + k_pitch : nullptr, im);
+                }
             }
             ur += slot_stride;
-            if (PREC != 0) lr += slot_stride;
+            if (PREC == 2) lr += slot_stride;
         };
         if (step) {
             // equally spaced channels: exact fixed-point phase every kAnchor

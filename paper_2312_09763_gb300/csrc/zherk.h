@@ -95,7 +95,7 @@ struct ZherkArgs {
 struct ZherkFinalArgs {
     const Inst* inst;
     int inst0, n_inst;
-    const float* amax;               // [n_inst]
+    const float* amax;               // [n_inst] max |WA| behind the FP16 scale (NULL: no scale)
     const float* partial;
     const ZherkTile* tiles;
     const int* tile_of;              // gauss: [2][np][np] tile of F_ij and of H_ij (i >= j), np panels
@@ -105,8 +105,11 @@ struct ZherkFinalArgs {
     const int2* limits;              // unique: row and column limits of every tile
 };
 
-// Products of one instance in the real form: the lower triangle of 2N rows.
+// Products of one instance: in the real form the lower triangle of 2N rows,
 std::vector<ZherkTile> zherk_triangle(int rows);
+
+// and in the gauss form of N antenna-feeds.
+std::vector<ZherkTile> zherk_gauss_tiles(int N);
 
 // Plan for n_inst instances; cover: the real-form tiles to compute (empty: the
 // whole V of N antenna-feeds, in either form).  est_live: live sources
@@ -123,5 +126,19 @@ cudaError_t launch_zherk_prep(const ZherkArgs& P, const float* amax_in, float* a
                               long long* launches);
 cudaError_t launch_zherk(const ZherkArgs& P, int form, int n_ctas, cudaStream_t st, long long* launches);
 cudaError_t launch_zherk_final(const ZherkFinalArgs& a, int form, cudaStream_t st, long long* launches);
+
+// FP32 HERK on the CUDA cores (herk_fp32.cu): the form of Z (with the gauss form
+// plane_rows = N and the planes X, Y and S one after another), its products and
+// the source ranges each is split into.
+struct Fp32Plan {
+    int form = kZherkReal, rows = 0, plane_rows = 0, split = 1;
+    std::vector<ZherkTile> tiles;
+};
+Fp32Plan herk_fp32_plan(int N, int n_ax, int n_inst, double est_live, int n_sms);
+cudaError_t herk_fp32_init();
+// Partial tiles [n_inst][n_tiles][split][128][128] of U's products.
+cudaError_t launch_herk_fp32(const Inst* d_inst, int inst0, int n_inst, LiveTables lt, int n_ax, const float* d_u,
+                             int rows, int plane_rows, long long k_pitch, const ZherkTile* d_tiles, int n_tiles,
+                             int split, float* d_partial, int* d_err, cudaStream_t st, long long* launches);
 
 }  // namespace mv

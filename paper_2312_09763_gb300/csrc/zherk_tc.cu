@@ -829,7 +829,7 @@ __global__ void __launch_bounds__(256) k_zherk_final_real(ZherkFinalArgs a) {
         G[c][r] = sum_parts(p, a.S, (bc + c) * 128 + br + r);
     }
     __syncthreads();
-    const float us = ldexpf(1.f, -fp16_scale_exp(a.amax[slot]));
+    const float us = a.amax ? ldexpf(1.f, -fp16_scale_exp(a.amax[slot])) : 1.f;
     float2* Vb = a.V + a.inst[a.inst0 + slot].v_off;
     auto entry = [&](int i, int j) {  // product entry (row, column) of the piece
         return t.trans ? G[i][j] : G[j][i];
@@ -889,7 +889,7 @@ __global__ void __launch_bounds__(256) k_zherk_final_gauss(ZherkFinalArgs a) {
         }
     }
     __syncthreads();
-    const float us = ldexpf(1.f, -fp16_scale_exp(a.amax[slot]));
+    const float us = a.amax ? ldexpf(1.f, -fp16_scale_exp(a.amax[slot])) : 1.f;
     float2* Vb = a.V + a.inst[a.inst0 + slot].v_off;
     for (int pass = 0; pass < 2; ++pass)
         for (int k = threadIdx.x; k < 32 * 32; k += 256) {
@@ -996,6 +996,15 @@ std::vector<ZherkTile> zherk_triangle(int rows) {
     return t;
 }
 
+std::vector<ZherkTile> zherk_gauss_tiles(int N) {
+    std::vector<ZherkTile> t;
+    for (int i = 0; i < N; i += 128)
+        for (int j = 0; j < N; j += 128) t.push_back(ZherkTile{i, N + j, i, j, 0, 0});
+    for (int i = 0; i < N; i += 128)
+        for (int j = 0; j <= i; j += 128) t.push_back(ZherkTile{2 * N + i, 2 * N + j, i, j, 1, 0});
+    return t;
+}
+
 namespace {
 
 // Pair up products that share a panel: that panel is A, the other two B (N =
@@ -1098,10 +1107,7 @@ bool zherk_plan(int N, const std::vector<ZherkTile>& cover, int n_ax, int n_inst
             z.tiles = cover.empty() ? zherk_triangle(z.rows) : cover;
         } else {
             z.rows = 3 * N;
-            for (int i = 0; i < N; i += 128)
-                for (int j = 0; j < N; j += 128) z.tiles.push_back(ZherkTile{i, N + j, i, j, 0, 0});
-            for (int i = 0; i < N; i += 128)
-                for (int j = 0; j <= i; j += 128) z.tiles.push_back(ZherkTile{2 * N + i, 2 * N + j, i, j, 1, 0});
+            z.tiles = zherk_gauss_tiles(N);
         }
         if ((int)z.tiles.size() > 2 * n_sms) continue;
         std::vector<ZherkJob> one;  // the jobs of one instance
