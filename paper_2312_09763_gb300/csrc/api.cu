@@ -307,7 +307,7 @@ struct StreamBatch {
     int inst0, n, g0, ng;  // groups [g0, g0 + ng) of the plan: entries of the antenna phase table
     const ZherkPlan* plan;
     size_t jobs, groups, items, group0, tiles, tile_of, limits;
-    int n_groups, ant_block, np;
+    int n_groups, ant_block, z_buf_b, np;
     long long max_chunks;
 };
 
@@ -521,6 +521,7 @@ bool plan_stream(mv_ctx* c, Plan& P, Prepared& p, std::vector<uint8_t>& tab) {
         for (const ZherkGroup& g : groups) chan = std::max(chan, g.n);
         b.ant_block = zherk_ant_block(*z, m.n_ant, m.n_ax * m.n_feed, most, chan, c->n_sms);
         if (b.ant_block < 1) return false;
+        b.z_buf_b = zherk_input_bytes(chan, m.n_ax * m.n_feed, m.n_beam);
         b.ng = (int)P.groups.size() - b.g0;
         b.n_groups = (int)groups.size();
         b.jobs = put(z->jobs.data(), z->jobs.size() * sizeof(ZherkJob));
@@ -953,6 +954,8 @@ mv_status enqueue_stream(mv_ctx* c, const Prepared& p, size_t i, cudaStream_t st
     z.n_jobs = b.plan->n_jobs;
     z.n_jobs_last = b.plan->n_jobs_last;
     z.ant_block = b.ant_block;
+    z.z_buf_b = b.z_buf_b;
+    z.z_shift = zherk_input_shift(b.z_buf_b);
     z.flush = p.sflush;
     z.n_tiles = (int)b.plan->tiles.size();
     z.ready = (int*)c->zcount.p;
@@ -1170,7 +1173,7 @@ std::vector<long long> graph_key(mv_ctx* c, const Plan& P, const Prepared& p, co
                             (long long)b.plan->tiles.size(),
                             (long long)b.jobs, (long long)b.groups, (long long)b.items, (long long)b.group0,
                             (long long)b.tiles, (long long)b.tile_of, (long long)b.limits, (long long)b.n_groups,
-                            (long long)b.ant_block, b.max_chunks})
+                            (long long)b.ant_block, (long long)b.z_buf_b, b.max_chunks})
             k.push_back(x);
     return k;
 }

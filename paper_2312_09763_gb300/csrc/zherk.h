@@ -84,6 +84,7 @@ struct ZherkArgs {
     const ZherkJob* jobs;
     int n_jobs, n_jobs_last;
     int ant_block;                   // antennas per Z warp
+    int z_shift, z_buf_b;            // 1 << z_shift input buffers of the Z warps, bytes of each
     int flush;                       // 32-column stages per TMEM flush
     int n_tiles;
     int *ready, *done;               // per chunk: SMs that finished building it, that loaded it
@@ -120,6 +121,9 @@ bool zherk_plan(int N, const std::vector<ZherkTile>& cover, int n_ax, int n_inst
 // Antennas per Z warp for groups of up to `chan` channels, `groups` of them in
 // a wave (0: no choice fits); nc: feeds x axes.
 int zherk_ant_block(const ZherkPlan& z, int n_ant, int nc, int groups, int chan, int n_sms);
+// Bytes of an input buffer of the Z warps (groups of up to chan channels), and the log2 of their number.
+int zherk_input_bytes(int chan, int nc, int n_beam);
+int zherk_input_shift(int bytes);
 cudaError_t zherk_init();
 cudaError_t launch_zherk_prep(const ZherkArgs& P, const float* amax_in, float* amax_out, float* scale, int4* zv,
                               int* wave_base, ZherkGroup* groups, int n_groups, bool by_length, cudaStream_t st,

@@ -67,12 +67,16 @@ constexpr int Z_APH_B = Z_BLOCK * (int)sizeof(AntPhase);  // their phase factors
 constexpr int Z_SRC_B = 6 * kZherkChunk * 4;              // a chunk's directions: 3 x S, 3 x eps
 constexpr int Z_CHAN = kZherkChan;        // channels x components of a chunk's WA in shared memory
 constexpr int Z_WA_B = Z_CHAN * kZherkChunk * 8;
-constexpr int Z_BUF = Z_SRC_B + Z_WA_B;   // one of two buffers
+// The Z warps' inputs: two buffers of the most channels, four or eight of fewer:
+// with two, a chunk of one channel waits for the latency of a fill (12 antennas,
+// 84 pairs of 70,000 sources: 704 us, with eight buffers 505).
+constexpr int Z_BUF = Z_SRC_B + Z_WA_B, MAX_BUF = 8;
+constexpr int Z_BARS_B = (2 * STAGES + 2 + 3 * MAX_BUF) * 8 + 16;
 // Z-build warps per SM: as many as the registers allow (24 warps of 80
 // registers in all with one component, 20 of 96 with several).
 __host__ __device__ constexpr int z_warps(int nc) { return nc == 1 ? 12 : 8; }
 constexpr int threads_for(int nc) { return (FIRST_Z + z_warps(nc)) * 32; }
-constexpr int smem_for(int nc) { return STAGES * STAGE + 2 * Z_BUF + z_warps(nc) * Z_APH_B + 1024 + 256; }
+constexpr int smem_for(int nc) { return STAGES * STAGE + 2 * Z_BUF + z_warps(nc) * Z_APH_B + 1024 + Z_BARS_B; }
 static_assert(smem_for(1) <= 232448 && smem_for(2) <= 232448, "227 KB of shared memory");
 static_assert(Z_BUF % 16 == 0 && Z_SRC_B % 16 == 0 && Z_APH_B % 16 == 0, "16-byte copies");
 
@@ -321,10 +325,10 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     constexpr int Z_WARPS = z_warps(NAX * NFD), NC = NAX * NFD;
-    uint8_t* zsm = smem + STAGES * STAGE;      // two buffers, then the Z warps' phase factors
-    // barriers: full[STAGES], empty[STAGES], tfull, tempty, zfull[2], zdone[2], zfree[2]
+    uint8_t* zsm = smem + STAGES * STAGE;      // input buffers, then the Z warps' phase factors
+    // barriers: full[STAGES], empty[STAGES], tfull, tempty, zfull, zdone and zfree [MAX_BUF] each
     uint64_t* bars = reinterpret_cast<uint64_t*>(zsm + 2 * Z_BUF + Z_WARPS * Z_APH_B);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 8);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 2 + 3 * MAX_BUF);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     volatile int* freed = reinterpret_cast<volatile int*>(tmem_slot + 2);  // chunks every SM has loaded, in a row
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -332,15 +336,18 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
     auto empty = [&](int s) { return smem_u32(&bars[STAGES + s]); };
     const uint32_t tfull = smem_u32(&bars[2 * STAGES]), tempty = smem_u32(&bars[2 * STAGES + 1]);
     auto zfull = [&](int b) { return smem_u32(&bars[2 * STAGES + 2 + b]); };
-    auto zdone = [&](int b) { return smem_u32(&bars[2 * STAGES + 4 + b]); };
-    auto zfree = [&](int b) { return smem_u32(&bars[2 * STAGES + 6 + b]); };
+    auto zdone = [&](int b) { return smem_u32(&bars[2 * STAGES + 2 + MAX_BUF + b]); };
+    auto zfree = [&](int b) { return smem_u32(&bars[2 * STAGES + 2 + 2 * MAX_BUF + b]); };
+    // input k of the Z warps: buffer k & zmask, its barriers' phase
+    const int zmask = (1 << P.z_shift) - 1;
+    auto zphase = [&](int k) { return (uint32_t)(k >> P.z_shift) & 1u; };
     constexpr int SPC = kZherkChunk * NAX / 32, RC = zherk_ring_chunks(NAX);  // stages per chunk, chunks in the ring
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
         mbar_init(tfull, 1);
         mbar_init(tempty, EPI_WARPS);
-        for (int b = 0; b < 2; ++b) { mbar_init(zfull(b), 1); mbar_init(zdone(b), Z_WARPS); mbar_init(zfree(b), 1); }
+        for (int b = 0; b < MAX_BUF; ++b) { mbar_init(zfull(b), 1); mbar_init(zdone(b), Z_WARPS); mbar_init(zfree(b), 1); }
         *abort_flag = 0;
         *freed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -430,19 +437,19 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
             if (z.team < 0) continue;
             const int base = P.wave_base[w], wlen = P.wave_base[w + 1] - base;
             for (int q = z.team; q < wlen; q += z.teams, ++k) {
-                if (!wait_bounded(zdone(k & 1), (uint32_t)(k >> 1) & 1u, abort_flag, P.err, kTimeoutNs, 100u)) ok = false;
+                if (!wait_bounded(zdone(k & zmask), zphase(k), abort_flag, P.err, kTimeoutNs, 100u)) ok = false;
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 if (lane == 0) {
-                    mbar_arrive(zfree(k & 1));  // (seen: the buffer's barrier may start its next phase)
+                    mbar_arrive(zfree(k & zmask));  // (seen: the buffer's barrier may start its next phase)
                     red_release(P.ready + base + q, 1);
                 }
                 __syncwarp();
             }
         }
     } else if (warp == FEED_WARP) {
-        // Feed the Z warps: each chunk's directions and (one beam) WA into one of two
-        // buffers.  And watch the next 32 chunks' done counts and tell the Z warps
+        // Feed the Z warps: each chunk's directions and (one beam) WA into the next
+        // buffer.  And watch the next 32 chunks' done counts and tell the Z warps
         // through shared memory how far the ring is free (one poller per SM).
         const int last_base = P.wave_base[P.n_waves - 1], total = P.wave_base[P.n_waves];
         int next = 0, k = 0, w = -1, q = 0, base = 0, wlen = 0;
@@ -467,9 +474,9 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                 q = z.team < 0 ? 0 : z.team;
                 if (z.team >= 0) g = P.groups + P.wave_group0[w] + z.gi;
             }
-            if (more && (k < 2 || __all_sync(0xffffffffu, mbar_test(zfree(k & 1), ((uint32_t)(k >> 1) & 1u) ^ 1u)))) {
+            if (more && (k <= zmask || __all_sync(0xffffffffu, mbar_test(zfree(k & zmask), zphase(k) ^ 1u)))) {
                 any = true;
-                const uint32_t bar = zfull(k & 1), dst = smem_u32(zsm + (k & 1) * Z_BUF);
+                const uint32_t bar = zfull(k & zmask), dst = smem_u32(zsm + (k & zmask) * P.z_buf_b);
                 if (q < g->len) {
                     const int n = ONE ? g->n * NC : 0, src = (g->c0 + q) * kZherkChunk;
                     if (lane == 0) mbar_expect_tx(bar, (uint32_t)(Z_SRC_B + n * kZherkChunk * 8));
@@ -657,7 +664,7 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
             const int col = 2 * lane * NAX;
             const unsigned blk_b = (unsigned)((col >> 5) * 128 + (col & 31) * 2);
             const unsigned hi_b = blk_b + ((col >> 5) & 1) * 64, lo_b = blk_b + (((col >> 5) & 1) ^ 1) * 64;
-            int k = 0, owed = -1;  // owed: the buffer of the last item, whose barrier waits for this warp
+            int k = 0;
             bool ok = true;
             for (int w = 0; w < P.n_waves && ok; ++w) {
                 const ZShare z = z_share(P, w, Z_WARPS * P.ant_block);
@@ -680,11 +687,8 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                 asm volatile("cp.async.wait_group 0;" ::: "memory");
                 __syncwarp();
                 for (int q = z.team; q < wlen; q += z.teams, ++k) {
-                    const int cq = base + q, buf = k & 1;
-                    if (!wait_bounded(zfull(buf), (uint32_t)(k >> 1) & 1u, abort_flag, P.err)) ok = false;
-                    // the last item's stores have had the time since to drain
-                    if (owed >= 0 && lane == 0) mbar_arrive(zdone(owed));
-                    owed = -1;
+                    const int cq = base + q;
+                    if (!wait_bounded(zfull(k & zmask), zphase(k), abort_flag, P.err)) ok = false;
                     // the chunk whose place in the ring this one takes has been read by all
                     if (__shfl_sync(0xffffffffu, *freed, 0) <= cq - RC) {
                         const unsigned long long t0 = gtimer();
@@ -701,7 +705,7 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     if (q < g.len && a0 < a1) {
-                        const uint8_t* sm = zsm + buf * Z_BUF;
+                        const uint8_t* sm = zsm + (k & zmask) * P.z_buf_b;
                         unsigned S0[3], S1[3];
                         float E0[3], E1[3];
 #pragma unroll
@@ -720,10 +724,9 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                             z_ant<FORM, NAX, NFD, ONE>(P, g, o, tab + (a - a0), per_e, a, S0, S1, E0, E1);
                     }
                     __syncwarp();
-                    owed = buf;
+                    if (lane == 0) mbar_arrive(zdone(k & zmask));
                 }
             }
-            if (owed >= 0 && lane == 0) mbar_arrive(zdone(owed));
             __syncwarp();
         }
     }
@@ -800,21 +803,32 @@ __global__ void __launch_bounds__(1024) k_zherk_prep(ZherkArgs P, const float* _
     }
 }
 
-// Sum of the S partial tiles at p (stride 128 x 128), element i.
-__device__ __forceinline__ float sum_parts(const float* p, int S, int i) {
-    float v = p[i];
-    for (int k = 1; k < S; ++k) v += p[(long long)k * (128 * 128) + i];
+// Rows [r, r + 4) of column c of the sum of the S partial tiles at p (128 x
+// 128 floats each): what bounds the sums is the loads' latency, so eight go out
+// together (one instance in 64 ranges: 32 us with 64 x 64 pieces and a load at a
+// time, 6 us with 32 x 32 pieces of four rows a thread).
+__device__ __forceinline__ float4 sum_parts(const float* p, int S, int r, int c) {
+    const float4* q = reinterpret_cast<const float4*>(p + c * 128 + r);
+    float4 v = *q;
+#pragma unroll 8
+    for (int k = 1; k < S; ++k) {
+        const float4 x = q[(long long)k * (128 * 128 / 4)];
+        v.x += x.x;
+        v.y += x.y;
+        v.z += x.z;
+        v.w += x.w;
+    }
     return v;
 }
 
-// V from the partial tiles of the real form: one block per 64 x 64 piece of a
-// tile (32 x 32 antenna-feeds), read along the tile's rows and written along
+// V from the partial tiles of the real form: one block per 32 x 32 piece of a
+// tile (16 x 16 antenna-feeds), read along the tile's rows and written along
 // the rows of V through shared memory.
 __global__ void __launch_bounds__(256) k_zherk_final_real(ZherkFinalArgs a) {
-    __shared__ float G[64][65];  // [column][row]
+    __shared__ float G[32][33];  // [column][row]
     const int slot = blockIdx.x / a.n_tiles, tile = blockIdx.x - slot * a.n_tiles;
     const ZherkTile t = a.tiles[tile];
-    const int br = (blockIdx.y & 1) * 64, bc = (blockIdx.y >> 1) * 64;
+    const int br = (blockIdx.y & 3) * 32, bc = (blockIdx.y >> 2) * 32;
     const float* p = a.partial + ((long long)slot * a.n_tiles + tile) * a.S * (128 * 128);
     // the product's rows and columns this piece stands for
     const int pr = t.r0 + (t.trans ? bc : br), pc = t.c0 + (t.trans ? br : bc);
@@ -823,10 +837,14 @@ __global__ void __launch_bounds__(256) k_zherk_final_real(ZherkFinalArgs a) {
         rlim = min(rlim, a.limits[tile].x);
         clim = min(clim, a.limits[tile].y);
     }
-    if (pr >= rlim || pc >= clim || (!a.ho.uidx && pr + 63 < pc)) return;
-    for (int i = threadIdx.x; i < 64 * 64; i += 256) {
-        const int r = i & 63, c = i >> 6;
-        G[c][r] = sum_parts(p, a.S, (bc + c) * 128 + br + r);
+    if (pr >= rlim || pc >= clim || (!a.ho.uidx && pr + 31 < pc)) return;
+    {
+        const int r = (threadIdx.x & 7) * 4, c = threadIdx.x >> 3;
+        const float4 v = sum_parts(p, a.S, br + r, bc + c);
+        G[c][r] = v.x;
+        G[c][r + 1] = v.y;
+        G[c][r + 2] = v.z;
+        G[c][r + 3] = v.w;
     }
     __syncthreads();
     const float us = a.amax ? ldexpf(1.f, -fp16_scale_exp(a.amax[slot])) : 1.f;
@@ -835,31 +853,30 @@ __global__ void __launch_bounds__(256) k_zherk_final_real(ZherkFinalArgs a) {
         return t.trans ? G[i][j] : G[j][i];
     };
     const bool diag = t.r0 == t.c0;
-    for (int pass = 0; pass < (a.ho.uidx ? 1 : 2); ++pass)
-        for (int k = threadIdx.x; k < 32 * 32; k += 256) {
-            // pass 0: along the rows of V; pass 1: the mirror image, along its rows
-            const int x = k & 31, y = k >> 5;
-            const int ia = pass ? x : y, ib = pass ? y : x;
-            const int A = (pr >> 1) + ia, B = (pc >> 1) + ib;
-            if (2 * A >= rlim || 2 * B >= clim) continue;
-            const float g00 = entry(2 * ia, 2 * ib), g01 = entry(2 * ia, 2 * ib + 1);
-            const float g10 = entry(2 * ia + 1, 2 * ib), g11 = entry(2 * ia + 1, 2 * ib + 1);
-            const float re = ((g00 + g11) * us) * us;
-            const float im = A == B ? 0.f : ((g10 - g01) * us) * us;
-            if (a.ho.uidx) {
-                const int nf = a.ho.n_feed;
-                const int aa = A / nf, pa = A - aa * nf, bb = B / nf, pb = B - bb * nf;
-                const int e = a.ho.uidx[aa * a.ho.n_ant + bb];
-                if (e < 0) continue;
-                const int grp = e >> 1;
-                const bool cj = (e & 1) != 0;
-                Vb[((long long)grp * nf + (cj ? pb : pa)) * nf + (cj ? pa : pb)] = make_float2(re, cj ? -im : im);
-                continue;
-            }
-            if (diag && A < B) continue;  // a diagonal tile's upper half is the mirror
-            if (pass == 0) Vb[(long long)A * a.N + B] = make_float2(re, im);
-            else if (A != B) Vb[(long long)B * a.N + A] = make_float2(re, -im);
+    const int x = threadIdx.x & 15, y = threadIdx.x >> 4;
+    for (int pass = 0; pass < (a.ho.uidx ? 1 : 2); ++pass) {
+        // pass 0: along the rows of V; pass 1: the mirror image, along its rows
+        const int ia = pass ? x : y, ib = pass ? y : x;
+        const int A = (pr >> 1) + ia, B = (pc >> 1) + ib;
+        if (2 * A >= rlim || 2 * B >= clim) continue;
+        const float g00 = entry(2 * ia, 2 * ib), g01 = entry(2 * ia, 2 * ib + 1);
+        const float g10 = entry(2 * ia + 1, 2 * ib), g11 = entry(2 * ia + 1, 2 * ib + 1);
+        const float re = ((g00 + g11) * us) * us;
+        const float im = A == B ? 0.f : ((g10 - g01) * us) * us;
+        if (a.ho.uidx) {
+            const int nf = a.ho.n_feed;
+            const int aa = A / nf, pa = A - aa * nf, bb = B / nf, pb = B - bb * nf;
+            const int e = a.ho.uidx[aa * a.ho.n_ant + bb];
+            if (e < 0) continue;
+            const int grp = e >> 1;
+            const bool cj = (e & 1) != 0;
+            Vb[((long long)grp * nf + (cj ? pb : pa)) * nf + (cj ? pa : pb)] = make_float2(re, cj ? -im : im);
+            continue;
         }
+        if (diag && A < B) continue;  // a diagonal tile's upper half is the mirror
+        if (pass == 0) Vb[(long long)A * a.N + B] = make_float2(re, im);
+        else if (A != B) Vb[(long long)B * a.N + A] = make_float2(re, -im);
+    }
 }
 
 // V from the partial tiles of the gauss form: one block per 32 x 32 piece of a
@@ -881,11 +898,13 @@ __global__ void __launch_bounds__(256) k_zherk_final_gauss(ZherkFinalArgs a) {
         const float* p = base + (long long)tile * a.S * (128 * 128);
         // the tile's rows run along a (M = F_ab, H_ab) unless it is F_ba or transposed
         const bool row_is_a = (m != 1) == (t.trans == 0);
-        for (int k = threadIdx.x; k < 32 * 32; k += 256) {
-            const int r = k & 31, c = k >> 5;
-            const float v = sum_parts(p, a.S, row_is_a ? (bc + c) * 128 + ar + r : (ar + c) * 128 + bc + r);
-            if (row_is_a) M[m][r][c] = v;
-            else M[m][c][r] = v;
+        const int r = (threadIdx.x & 7) * 4, c = threadIdx.x >> 3;
+        const float4 v = row_is_a ? sum_parts(p, a.S, ar + r, bc + c) : sum_parts(p, a.S, bc + r, ar + c);
+        const float f[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (row_is_a) M[m][r + k][c] = f[k];
+            else M[m][c][r + k] = f[k];
         }
     }
     __syncthreads();
@@ -948,6 +967,9 @@ cudaError_t launch_zherk_prep(const ZherkArgs& P, const float* amax_in, float* a
     return cudaGetLastError();
 }
 
+int zherk_input_bytes(int chan, int nc, int n_beam) { return Z_SRC_B + (n_beam == 1 ? chan * nc * kZherkChunk * 8 : 0); }
+int zherk_input_shift(int bytes) { return bytes * 8 <= 2 * Z_BUF ? 3 : bytes * 4 <= 2 * Z_BUF ? 2 : 1; }
+
 cudaError_t launch_zherk(const ZherkArgs& P, int form, int n_ctas, cudaStream_t st, long long* launches) {
     CUtensorMap map;
     if (!ring_map(&map, P.ring, zherk_row_bytes(P.m.n_ax), P.rows / P.map_rows, (long long)P.V * P.map_rows)) return cudaErrorInvalidValue;
@@ -981,7 +1003,7 @@ cudaError_t launch_zherk(const ZherkArgs& P, int form, int n_ctas, cudaStream_t 
 
 cudaError_t launch_zherk_final(const ZherkFinalArgs& a, int form, cudaStream_t st, long long* launches) {
     if (form == kZherkReal)
-        k_zherk_final_real<<<dim3((unsigned)(a.n_inst * a.n_tiles), 4), 256, 0, st>>>(a);
+        k_zherk_final_real<<<dim3((unsigned)(a.n_inst * a.n_tiles), 16), 256, 0, st>>>(a);
     else
         k_zherk_final_gauss<<<dim3((unsigned)(a.n_inst * (a.np * (a.np + 1) / 2)), 16), 256, 0, st>>>(a);
     *launches += 1;
