@@ -77,7 +77,12 @@ struct mv_ctx {
     std::vector<double> h_flux;  // I at nu_ref (host copy, for the polarised sky's coherency)
     Buf xeq, sqrt_flux, half_alpha, pol_m, ant_e, ant_n, ant_u, bidx, grid;
     // workspace
-    Buf R, counts, offsets, le, ln, lu, lsfix, lseps, lidx, lazza, nlive, chan, inst, groups, planes, vdev, err, partial, sched;
+    // tables of the call in progress (in ztab)
+    const double* d_R = nullptr;
+    const Chan* d_chan = nullptr;
+    const Inst* d_inst = nullptr;
+    const ZGroup* d_groups = nullptr;
+    Buf counts, offsets, masks, lsfix, lseps, lidx, lazza, nlive, planes, vdev, err, partial, sched;
     // per-batch workspace, double-buffered so that the beam evaluation and Z
     // build of one batch (on zstream) overlap the HERK of the previous one
     Buf wa[3], amax[3], u[2], ulo[2], aph[2];  // wa/amax: a third set when the beam runs two batches ahead
@@ -690,15 +695,31 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
     const long long pitch = p.pitch;
 
     mv_status s;
-    if ((s = upload(c, c->R, R.data(), R.size() * sizeof(double), st))) return s;
-    if ((s = upload(c, c->chan, chan.data(), chan.size() * sizeof(Chan), st))) return s;
-    if ((s = upload(c, c->inst, P.inst.data(), P.inst.size() * sizeof(Inst), st))) return s;
-    if ((s = upload(c, c->groups, P.groups.data(), P.groups.size() * sizeof(ZGroup), st))) return s;
+    if (p.zprec == 0) {
+        p.f32 = herk_fp32_plan(p.N, m.n_ax, max_slots, 0.5 * (double)m.n_src, c->n_sms);
+        const size_t slot = sizeof(float) * 128 * 128 * p.f32.tiles.size() * p.f32.split;
+        p.f32_slots = (int)std::max(1ll, std::min<long long>(max_slots, kPartialBytes / (long long)slot));
+        p.f32_tiles = put_table(ztab, p.f32.tiles.data(), p.f32.tiles.size() * sizeof(ZherkTile));
+        if (p.f32.form == kZherkGauss) {
+            const std::vector<int> of = gauss_tile_of(p.f32.tiles, (p.N + 127) / 128);
+            p.f32_tile_of = put_table(ztab, of.data(), of.size() * sizeof(int));
+        }
+        if ((s = ensure(c, c->partial, slot * p.f32_slots))) return s;
+    }
+    // everything the call's kernels read from the host goes up in one copy
+    const size_t at_R = put_table(ztab, R.data(), R.size() * sizeof(double));
+    const size_t at_chan = put_table(ztab, chan.data(), chan.size() * sizeof(Chan));
+    const size_t at_inst = put_table(ztab, P.inst.data(), P.inst.size() * sizeof(Inst));
+    const size_t at_groups = put_table(ztab, P.groups.data(), P.groups.size() * sizeof(ZGroup));
+    if ((s = upload(c, c->ztab, ztab.data(), ztab.size(), st))) return s;
+    const uint8_t* tab = (const uint8_t*)c->ztab.p;
+    c->d_R = (const double*)(tab + at_R);
+    c->d_chan = (const Chan*)(tab + at_chan);
+    c->d_inst = (const Inst*)(tab + at_inst);
+    c->d_groups = (const ZGroup*)(tab + at_groups);
     if ((s = ensure(c, c->counts, sizeof(int) * (size_t)p.bpt * n_times))) return s;
     if ((s = ensure(c, c->offsets, sizeof(int) * (size_t)p.bpt * n_times))) return s;
-    if ((s = ensure(c, c->le, sizeof(double) * (size_t)pitch * n_times))) return s;
-    if ((s = ensure(c, c->ln, sizeof(double) * (size_t)pitch * n_times))) return s;
-    if ((s = ensure(c, c->lu, sizeof(double) * (size_t)pitch * n_times))) return s;
+    if ((s = ensure(c, c->masks, sizeof(unsigned) * 8 * (size_t)p.bpt * n_times))) return s;
     if ((s = ensure(c, c->lsfix, sizeof(unsigned) * 3 * (size_t)pitch * n_times))) return s;
     if ((s = ensure(c, c->lseps, sizeof(float) * 3 * (size_t)pitch * n_times))) return s;
     if ((s = ensure(c, c->lidx, sizeof(int) * (size_t)pitch * n_times))) return s;
@@ -739,7 +760,6 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
             chunks = std::max(chunks, (size_t)b.max_chunks);
             vinsts = std::max(vinsts, (size_t)b.n * b.plan->S);
         }
-        if ((s = upload(c, c->ztab, ztab.data(), ztab.size(), st))) return s;
         if ((s = ensure(c, c->ring, ring))) return s;
         if ((s = ensure(c, c->partial, part))) return s;
         if ((s = ensure(c, c->zwave, sizeof(int) * waves))) return s;
@@ -747,18 +767,6 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
         if ((s = ensure(c, c->zscale, sizeof(float) * max_slots))) return s;
         if ((s = ensure(c, c->zamax, sizeof(float) * max_slots))) return s;
         if ((s = ensure(c, c->zorder, sizeof(int4) * vinsts))) return s;
-    }
-    if (p.zprec == 0) {
-        p.f32 = herk_fp32_plan(p.N, m.n_ax, max_slots, 0.5 * (double)m.n_src, c->n_sms);
-        const size_t slot = sizeof(float) * 128 * 128 * p.f32.tiles.size() * p.f32.split;
-        p.f32_slots = (int)std::max(1ll, std::min<long long>(max_slots, kPartialBytes / (long long)slot));
-        p.f32_tiles = put_table(ztab, p.f32.tiles.data(), p.f32.tiles.size() * sizeof(ZherkTile));
-        if (p.f32.form == kZherkGauss) {
-            const std::vector<int> of = gauss_tile_of(p.f32.tiles, (p.N + 127) / 128);
-            p.f32_tile_of = put_table(ztab, of.data(), of.size() * sizeof(int));
-        }
-        if ((s = upload(c, c->ztab, ztab.data(), ztab.size(), st))) return s;
-        if ((s = ensure(c, c->partial, slot * p.f32_slots))) return s;
     }
     const size_t plane_elems = (size_t)(p.zprec == 0 ? p.f32.rows : p.rows) * p.k_pitch * max_slots;
     for (int k = 0; k < p.nbuf && !p.stream; ++k) {
@@ -793,9 +801,6 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
         cudaGetLastError();
     }
     LiveTables& lt = p.lt;
-    lt.e = (double*)c->le.p;
-    lt.n = (double*)c->ln.p;
-    lt.u = (double*)c->lu.p;
     lt.sfix = (unsigned*)c->lsfix.p;
     lt.seps = (float*)c->lseps.p;
     lt.idx = (int*)c->lidx.p;
@@ -810,7 +815,7 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
 cudaError_t enqueue_herk(mv_ctx* c, const Prepared& p, const Plan::Batch& b, const HerkCfg& h, int k,
                          cudaStream_t st, long long* L, const ZJob* zj = nullptr, int kw = -1) {
     if (kw < 0) kw = k;
-    const Inst* d_inst = (const Inst*)c->inst.p;
+    const Inst* d_inst = c->d_inst;
     HerkOut ho = p.ho;
     if (ho.uidx) {
         const int w = h.bn == 128 ? 0 : 1;
@@ -849,13 +854,40 @@ cudaError_t enqueue_herk(mv_ctx* c, const Prepared& p, const Plan::Batch& b, con
                           (float*)c->partial.p, (int*)c->err.p, zj, p.zprec, p.ho.uidx ? &ho : nullptr, st, L);
 }
 
+// The start of a call: cull, beam planes and, with a streamed schedule, the phase
+// table of the first batch into workspace set 0.
+cudaError_t enqueue_front(mv_ctx* c, const Prepared& p, cudaStream_t st, long long* L) {
+    FrontArgs f{};
+    f.m = c->model;
+    f.R = c->d_R;
+    f.w = CullWork{(int*)c->counts.p, (int*)c->offsets.p, (unsigned*)c->masks.p};
+    f.bpt = p.bpt;
+    f.chan = c->d_chan;
+    if (c->model.beam_kind == 2 && !c->use_sur) {
+        f.grid = (const float2*)c->grid.p;
+        f.n_chan = p.n_chan;
+        f.planes = (float2*)c->planes.p;
+    }
+    if (p.stream && !p.sb.empty()) {
+        f.inst = c->d_inst;
+        f.groups = c->d_groups;
+        f.g_first = p.sb[0].g0;
+        f.n_groups = p.sb[0].ng;
+        f.n_phase = p.n_phase;
+        f.aph = (AntPhase*)c->aph[0].p;
+        f.amax = (float*)c->amax[0].p;
+        f.n_amax = p.sb[0].n;
+    }
+    return launch_front(f, p.n_times, p.lt, st, L);
+}
+
 // The Z build of batch b into workspace set k, for the HERK of the batch before.
 ZJob make_zjob(mv_ctx* c, const Prepared& p, const Plan::Batch& b, int k, int kw = -1) {
     if (kw < 0) kw = k;
     ZJob z{};
     z.m = c->model;
-    z.inst = (const Inst*)c->inst.p;
-    z.groups = (const ZGroup*)c->groups.p;
+    z.inst = c->d_inst;
+    z.groups = c->d_groups;
     z.g_first = b.g0;
     z.n_groups = b.ng;
     z.lt = p.lt;
@@ -872,32 +904,34 @@ ZJob make_zjob(mv_ctx* c, const Prepared& p, const Plan::Batch& b, int k, int kw
 }
 
 // Beam evaluation of one batch into workspace set k.
-mv_status enqueue_wa(mv_ctx* c, const Prepared& p, const Plan::Batch& b, int k, cudaStream_t st, long long* L) {
+mv_status enqueue_wa(mv_ctx* c, const Prepared& p, const Plan::Batch& b, int k, cudaStream_t st, long long* L,
+                     bool amax_zeroed = false) {
     mv_status s;
     const Model& m = c->model;
-    const Inst* d_inst = (const Inst*)c->inst.p;
-    if ((s = cuda_check(cudaMemsetAsync(c->amax[k].p, 0, sizeof(float) * b.n, st), "amax reset"))) return s;
+    const Inst* d_inst = c->d_inst;
+    if (!amax_zeroed && (s = cuda_check(cudaMemsetAsync(c->amax[k].p, 0, sizeof(float) * b.n, st), "amax reset"))) return s;
     Timed tw(c, MV_KERNEL_BEAM, st);
     cudaError_t e;
     if (c->use_sur)
         e = surrogate_wa(c->sur, m, p.plan->inst, b.inst0, b.n, p.h_nlive, p.plan->nu, c->nu_ref, p.lt,
                          (float2*)c->wa[k].p, p.pitch, (float*)c->amax[k].p, (int*)c->err.p, c->n_sms, st, L);
     else
-        e = launch_wa(m, (const float2*)c->planes.p, (const Chan*)c->chan.p, d_inst, b.inst0, b.n, p.lt,
+        e = launch_wa(m, (const float2*)c->planes.p, c->d_chan, d_inst, b.inst0, b.n, p.lt,
                       (float2*)c->wa[k].p, p.pitch, (float*)c->amax[k].p, st, L);
     tw.end();
     return launched(e, "beam evaluation", st);
 }
 
-// Antenna phase table of one batch into workspace set k (fused Z build, which
-// also wants one max |WA| per Z group, and the streamed schedule).
+// Antenna phase table of one batch into workspace set k, and its max |WA| folded
+// per Z group (fused Z build, after the beam evaluation) or zeroed (streamed
+// schedule, before it).
 mv_status enqueue_ant_phase(mv_ctx* c, const Prepared& p, const Plan::Batch& b, int k, cudaStream_t st,
                             long long* L, int kw = -1, bool group_max = true) {
     if (kw < 0) kw = k;
     Timed tz(c, MV_KERNEL_ZBUILD, st);
-    cudaError_t e = launch_ant_phase(c->model, (const Inst*)c->inst.p, (const Chan*)c->chan.p,
-                                     (const ZGroup*)c->groups.p, b.g0, b.ng, (AntPhase*)c->aph[k].p, p.n_phase,
-                                     p.zprec == 2 && group_max ? (float*)c->amax[kw].p : nullptr, st, L);
+    cudaError_t e = launch_ant_phase(c->model, c->d_inst, c->d_chan,
+                                     c->d_groups, b.g0, b.ng, (AntPhase*)c->aph[k].p, p.n_phase,
+                                     p.zprec == 2 ? (float*)c->amax[kw].p : nullptr, !group_max, st, L);
     tz.end();
     return launched(e, "phase table", st);
 }
@@ -906,10 +940,10 @@ mv_status enqueue_ant_phase(mv_ctx* c, const Prepared& p, const Plan::Batch& b, 
 mv_status enqueue_zside(mv_ctx* c, const Prepared& p, const Plan::Batch& b, int k, cudaStream_t st, long long* L) {
     mv_status s;
     const Model& m = c->model;
-    const Inst* d_inst = (const Inst*)c->inst.p;
+    const Inst* d_inst = c->d_inst;
     if ((s = enqueue_wa(c, p, b, k, st, L))) return s;
     Timed tz(c, MV_KERNEL_ZBUILD, st);
-    cudaError_t e = launch_zbuild(m, d_inst, (const Chan*)c->chan.p, (const ZGroup*)c->groups.p, b.g0, b.ng, p.lt,
+    cudaError_t e = launch_zbuild(m, d_inst, c->d_chan, c->d_groups, b.g0, b.ng, p.lt,
                       (const float2*)c->wa[k].p, p.pitch, (float*)c->amax[k].p, c->u[k].p, c->ulo[k].p,
                       p.zprec == 0 && p.f32.form == kZherkGauss ? 1 : p.zprec, p.zprec == 0 ? p.f32.rows : p.rows,
                       p.k_pitch, p.nbuf == 2 && !p.fuse ? 4 * c->n_sms : 0, (AntPhase*)c->aph[k].p,
@@ -918,18 +952,19 @@ mv_status enqueue_zside(mv_ctx* c, const Prepared& p, const Plan::Batch& b, int 
     return launched(e, "Z build", st);
 }
 
-// One batch of the streamed schedule: beam evaluation, phase table, then the
-// launch that builds Z and expands it, and the sum of its partial tiles into V.
-mv_status enqueue_stream(mv_ctx* c, const Prepared& p, size_t i, cudaStream_t st, long long* L) {
+// One batch of the streamed schedule: phase table (unless enqueue_front made it),
+// beam evaluation, then the launch that builds Z and expands it, and the sum of
+// its partial tiles into V.
+mv_status enqueue_stream(mv_ctx* c, const Prepared& p, size_t i, bool have_phase, cudaStream_t st, long long* L) {
     mv_status s;
     const StreamBatch& b = p.sb[i];
     const Plan::Batch pb{b.inst0, b.n, b.g0, b.ng};
-    if ((s = enqueue_wa(c, p, pb, 0, st, L))) return s;
-    if ((s = enqueue_ant_phase(c, p, pb, 0, st, L, -1, false))) return s;
+    if (!have_phase && (s = enqueue_ant_phase(c, p, pb, 0, st, L, -1, false))) return s;
+    if ((s = enqueue_wa(c, p, pb, 0, st, L, true))) return s;
     const uint8_t* tab = (const uint8_t*)c->ztab.p;
     ZherkArgs z{};
     z.m = c->model;
-    z.inst = (const Inst*)c->inst.p;
+    z.inst = c->d_inst;
     z.inst0 = b.inst0;
     z.n_inst = b.n;
     z.lt = p.lt;
@@ -963,10 +998,9 @@ mv_status enqueue_stream(mv_ctx* c, const Prepared& p, size_t i, cudaStream_t st
     z.partial = (float*)c->partial.p;
     z.err = (int*)c->err.p;
     Timed th(c, MV_KERNEL_HERK, st);
-    if ((s = cuda_check(cudaMemsetAsync(c->zcount.p, 0, sizeof(int) * 2 * b.max_chunks, st), "chunk counters"))) return s;
     cudaError_t e = launch_zherk_prep(z, (const float*)c->amax[0].p, (float*)c->zamax.p, (float*)c->zscale.p,
                                       (int4*)c->zorder.p, (int*)c->zwave.p, (ZherkGroup*)((uint8_t*)c->ztab.p + b.groups),
-                                      b.n_groups, p.plan->pairs, st, L);
+                                      b.n_groups, p.plan->pairs, 2 * b.max_chunks, st, L);
     if (e == cudaSuccess) e = launch_zherk(z, b.plan->form, c->n_sms, st, L);
     ZherkFinalArgs f{};
     f.inst = z.inst;
@@ -1013,8 +1047,7 @@ mv_status enqueue_all(mv_ctx* c, Plan& P, Prepared& p, const HerkCfg& h, cudaStr
         return cuda_check(cudaStreamWaitEvent(st, c->ev_cdone, 0), "event wait");
     };
     Timed tc0(c, MV_KERNEL_CULL, st);
-    cudaError_t e = launch_cull(m, (const double*)c->R.p, p.n_times, p.lt, (int*)c->counts.p, (int*)c->offsets.p,
-                                p.bpt, st, L);
+    cudaError_t e = enqueue_front(c, p, st, L);
     tc0.end();
     if ((s = launched(e, "cull", st))) return s;
     if (c->use_sur) {
@@ -1024,16 +1057,10 @@ mv_status enqueue_all(mv_ctx* c, Plan& P, Prepared& p, const HerkCfg& h, cudaStr
                                             cudaMemcpyDeviceToHost, st), "live counts")))
             return s;
         if ((s = cuda_check(cudaStreamSynchronize(st), "synchronize"))) return s;
-    } else if (m.beam_kind == 2) {
-        Timed tb(c, MV_KERNEL_BEAM, st);
-        e = launch_beam_planes(m, (const float2*)c->grid.p, (const Chan*)c->chan.p, p.n_chan, (float2*)c->planes.p,
-                               st, L);
-        tb.end();
-        if ((s = launched(e, "beam planes", st))) return s;
     }
     if (p.stream) {
         for (size_t i = 0; i < p.sb.size(); ++i) {
-            if ((s = enqueue_stream(c, p, i, st, L))) return s;
+            if ((s = enqueue_stream(c, p, i, i == 0, st, L))) return s;
             if ((s = copy_out(P.batches[i]))) return s;
         }
         return join_copies();
@@ -1148,13 +1175,15 @@ std::vector<long long> graph_key(mv_ctx* c, const Plan& P, const Prepared& p, co
                                 (long long)(uintptr_t)m.ant_u, (long long)(uintptr_t)m.beam_idx, m.beam_kind,
                                 bits(m.gauss_c), m.n_beam, m.n_feed, m.n_ax, m.n_nu, m.n_za, m.n_az, bits(m.dza),
                                 bits(m.daz), m.interp};
-    const Buf* bufs[] = {&c->R, &c->chan, &c->inst, &c->groups, &c->counts, &c->offsets, &c->le, &c->ln, &c->lu,
+    const Buf* bufs[] = {&c->counts, &c->offsets, &c->masks,
                          &c->lidx, &c->lazza, &c->nlive, &c->wa[0], &c->amax[0], &c->sched, &c->u[0], &c->ulo[0],
                          &c->wa[1], &c->amax[1], &c->u[1], &c->ulo[1], &c->wa[2], &c->amax[2], &c->partial,
                          &c->planes, &c->grid, &c->err,
                          &c->lsfix, &c->lseps, &c->aph[0], &c->aph[1], &c->pol_m, &c->red_uidx, &c->red_tl[0],
                          &c->red_tl[1], &c->ring, &c->ztab, &c->zcount, &c->zscale, &c->zorder, &c->zwave, &c->zamax};
     for (const Buf* b : bufs) k.push_back((long long)(uintptr_t)b->p);
+    for (const void* d : {(const void*)c->d_R, (const void*)c->d_chan, (const void*)c->d_inst, (const void*)c->d_groups})
+        k.push_back((long long)(uintptr_t)d);
     for (const auto& b : P.batches) {
         k.push_back(b.inst0);
         k.push_back(b.n);
@@ -1310,14 +1339,7 @@ mv_status autotune(mv_ctx* c, Plan& P, mv_precision prec, cudaStream_t st, mv_tu
     if ((s = ensure(c, c->partial, need))) return s;
     long long L = 0;
     const Model& m = c->model;
-    cudaError_t e = launch_cull(m, (const double*)c->R.p, p.n_times, p.lt, (int*)c->counts.p, (int*)c->offsets.p,
-                                p.bpt, st, &L);
-    if ((s = cuda_check(e, "cull"))) return s;
-    if (m.beam_kind == 2) {
-        e = launch_beam_planes(m, (const float2*)c->grid.p, (const Chan*)c->chan.p, p.n_chan, (float2*)c->planes.p,
-                               st, &L);
-        if ((s = cuda_check(e, "beam planes"))) return s;
-    }
+    if ((s = cuda_check(enqueue_front(c, p, st, &L), "cull"))) return s;
     if ((s = enqueue_zside(c, p, b0, 0, st, &L))) return s;
     ZJob zj{};
     if (p.fuse) {
@@ -1372,14 +1394,12 @@ mv_status autotune(mv_ctx* c, Plan& P, mv_precision prec, cudaStream_t st, mv_tu
         if ((s = prepare(c, P2, prec, c->vdev.p, 0, st, p2, true, true))) return s;
         if (p2.stream) {
             ++n_cands;
-            if ((s = cuda_check(launch_cull(m, (const double*)c->R.p, p2.n_times, p2.lt, (int*)c->counts.p,
-                                            (int*)c->offsets.p, p2.bpt, st, &L), "cull")))
-                return s;
+            if ((s = cuda_check(enqueue_front(c, p2, st, &L), "cull"))) return s;
             double sms = 1e300;
             for (int r = 0; r <= reps; ++r) {  // the first run warms up
                 cudaEventRecord(e0, st);
                 for (size_t i = 0; i < p2.sb.size(); ++i)
-                    if ((s = enqueue_stream(c, p2, i, st, &L))) return s;
+                    if ((s = enqueue_stream(c, p2, i, false, st, &L))) return s;
                 cudaEventRecord(e1, st);
                 if ((s = cuda_check(cudaEventSynchronize(e1), "trial timing"))) return s;
                 float ms = 0.f;
@@ -1492,10 +1512,12 @@ void mv_destroy(mv_ctx* c) {
     DeviceGuard g(c->device);
     cudaDeviceSynchronize();
     Buf* all[] = {&c->xeq, &c->sqrt_flux, &c->half_alpha, &c->ant_e, &c->ant_n, &c->ant_u, &c->bidx, &c->grid,
-                  &c->R, &c->counts, &c->offsets, &c->le, &c->ln, &c->lu, &c->lidx, &c->lazza, &c->nlive,
-                  &c->chan, &c->inst, &c->groups, &c->planes, &c->wa[0], &c->amax[0], &c->u[0], &c->ulo[0],
+                  &c->counts, &c->offsets, &c->masks, &c->lidx, &c->lazza, &c->nlive,
+                  &c->planes, &c->wa[0], &c->amax[0], &c->u[0], &c->ulo[0],
                   &c->wa[1], &c->amax[1], &c->u[1], &c->ulo[1], &c->wa[2], &c->amax[2], &c->vdev, &c->err,
-                  &c->partial, &c->sched, &c->lsfix, &c->lseps, &c->aph[0], &c->aph[1], &c->pol_m};
+                  &c->partial, &c->sched, &c->lsfix, &c->lseps, &c->aph[0], &c->aph[1], &c->pol_m, &c->ring, &c->ztab,
+                  &c->zcount, &c->zscale, &c->zorder, &c->zwave, &c->zamax, &c->red_e, &c->red_n, &c->red_u, &c->red_b,
+                  &c->red_uidx, &c->red_tl[0], &c->red_tl[1]};
     for (Buf* b : all) buf_free(c, *b);
     surrogate_destroy(c->sur);
     harvest(c);

@@ -95,13 +95,31 @@ struct HerkOut {
     int n_ant, n_feed;
 };
 
+// The short kernels of a call start while the one before them ends (programmatic
+// dependent launch): each lets the next one start at once and waits itself, before
+// it touches memory, until the one before has ended (64 antennas x 8192 sources x
+// 16 channels: 54 us without, 45 with the tables of a call in one copy as well).
+__device__ __forceinline__ void kernel_chain() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // ------------------------------------------------------------ host launchers
 // (defined in the .cu files; all enqueue on `st` and return the CUDA error)
-cudaError_t launch_cull(const Model& m, const double* d_R, int n_times, LiveTables lt,
-                        int* d_counts, int* d_offsets, int blocks_per_time, cudaStream_t st,
-                        long long* launches);
-cudaError_t launch_beam_planes(const Model& m, const float2* d_grid, const Chan* d_chan, int n_chan,
-                               float2* d_planes, cudaStream_t st, long long* launches);
 // Z-side source factor of a polarised sky (eq. "fullz"): the two axis
 // components a0, a1 of one (beam, feed) times M = [[m00, 0], [m10, m11]] and
 // the spectral factor w: z0 = w (a0 m00 + a1 m10), z1 = w a1 m11.
@@ -176,7 +194,36 @@ struct ZJob {
 // max |WA|, so that one FP16 scale serves the whole group.
 cudaError_t launch_ant_phase(const Model& m, const Inst* d_inst, const Chan* d_chan, const ZGroup* d_groups,
                              int g_first, int n_groups, AntPhase* d_aph, int n_phase, float* d_amax,
-                             cudaStream_t st, long long* launches);
+                             bool zero_amax, cudaStream_t st, long long* launches);
+
+// What the cull keeps per block of 256 sources: [time][block] counts, and their
+// scan where there are more than 2048 blocks; a bit per source of who is live
+// (eight words a block; NULL: decided again).
+struct CullWork {
+    int *counts, *offsets;
+    unsigned* masks;
+};
+// The independent start of a call (prep.cu): cull, beam planes (planes NULL:
+// none) and the phase table of one batch with its n_amax max |WA| zeroed (aph
+// NULL: neither).  The live tables follow in lt.
+struct FrontArgs {
+    Model m;
+    const double* R;
+    CullWork w;
+    int bpt;
+    const float2* grid;
+    const Chan* chan;
+    int n_chan;
+    float2* planes;
+    const Inst* inst;
+    const ZGroup* groups;
+    int g_first, n_groups, n_phase;
+    AntPhase* aph;
+    float* amax;
+    int n_amax;
+    long long cull_blocks, plane_blocks;  // (set by the launch)
+};
+cudaError_t launch_front(const FrontArgs& a, int n_times, LiveTables lt, cudaStream_t st, long long* launches);
 
 // d_aph: workspace for n_groups x n_phase x n_ant AntPhase entries, n_phase
 // >= max(2, largest group of the batch).

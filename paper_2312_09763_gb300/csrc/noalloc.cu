@@ -107,7 +107,12 @@ extern "C" mv_status mv_horizon_cull_static(int64_t n_src, const double* xeq_dev
     lt.pitch = n_src;
     const int bpt = (int)((n_src + 255) / 256);
     long long launches = 0;
-    cudaError_t e = mv::launch_cull(m, rot, 1, lt, scratch, scratch + kMaxCullBlocks, bpt, st, &launches);
+    mv::FrontArgs f{};
+    f.m = m;
+    f.R = rot;
+    f.w = mv::CullWork{scratch, scratch + kMaxCullBlocks, nullptr};
+    f.bpt = bpt;
+    cudaError_t e = mv::launch_front(f, 1, lt, st, &launches);
     if (e != cudaSuccess) return fail(MV_ERR_CUDA, "mv_horizon_cull_static: launch failed");
     return MV_OK;
 }

@@ -3,11 +3,15 @@
 // (Sec. 2.3), the horizon cut with stable stream compaction, and the beam
 // evaluation at the live sources (Sec. 2.4), fused with sqrt(I_s(nu)).
 #include "common.cuh"
+#include "zcore.cuh"
 
 namespace mv {
 namespace {
 
 constexpr int kCullThreads = 256;
+// Blocks of one time up to which a scatter block sums the counts before it
+// itself (at most eight loads a thread); beyond, a scan kernel does it.
+constexpr int kScanBlocks = 2048;
 
 // One component of X_hrz = R X_eq, evaluated as (R0 x + R1 y) + R2 z with
 // every product and sum rounded on its own (no FMA contraction), so the
@@ -16,23 +20,76 @@ __device__ __forceinline__ double rot_row(const double* r, double x, double y, d
     return __dadd_rn(__dadd_rn(__dmul_rn(r[0], x), __dmul_rn(r[1], y)), __dmul_rn(r[2], z));
 }
 
-__global__ void __launch_bounds__(kCullThreads)
-k_cull_count(Model m, const double* __restrict__ R, int* __restrict__ counts, int bpt) {
-    const int t = blockIdx.y;
-    const long long s = (long long)blockIdx.x * kCullThreads + threadIdx.x;
-    int live = 0;
-    if (s < m.n_src) {
-        const double* r = R + 9 * t;
-        double up = rot_row(r + 6, m.xeq[s], m.xeq[m.n_src + s], m.xeq[2 * m.n_src + s]);
-        live = up > 0.0;
+__device__ __forceinline__ bool above(const Model& m, const double* __restrict__ R, int t, long long s) {
+    return s < m.n_src && rot_row(R + 9 * t + 6, m.xeq[s], m.xeq[m.n_src + s], m.xeq[2 * m.n_src + s]) > 0.0;
+}
+
+// The live sources of block blk of time t: their count and, a bit each, which.
+__device__ __forceinline__ void cull_count(const Model& m, const double* __restrict__ R, const CullWork& w, int bpt, int t,
+                                           int blk) {
+    const long long b = (long long)t * bpt + blk;
+    const bool live = above(m, R, t, (long long)blk * kCullThreads + threadIdx.x);
+    if (w.masks) {
+        const unsigned mask = __ballot_sync(0xffffffffu, live);
+        if ((threadIdx.x & 31) == 0) w.masks[b * (kCullThreads / 32) + (threadIdx.x >> 5)] = mask;
     }
-    int c = __syncthreads_count(live);
-    if (threadIdx.x == 0) counts[(long long)t * bpt + blockIdx.x] = c;
+    const int c = __syncthreads_count(live);
+    if (threadIdx.x == 0) w.counts[b] = c;
+}
+
+// Per-channel beam planes: P[c][b][p][k][za][az] = sum_m w_m(c) G[b][p][k][m0(c)+m][za][az]
+// (the frequency axis of the gridded beam interpolated once per channel); comp:
+// (b, p, k) flattened.
+__device__ __forceinline__ void beam_plane(const Model& m, const float2* __restrict__ grid, const Chan* __restrict__ chan,
+                                           float2* __restrict__ planes, int n_comp, int c, int comp, long long i) {
+    const long long plane = (long long)m.n_za * m.n_az;
+    if (i >= plane) return;
+    const Chan ch = chan[c];
+    const float2* g = grid + (long long)comp * m.n_nu * plane;
+    float re = 0.f, im = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        float2 v = g[(long long)(ch.m0 + j) * plane + i];
+        re = fmaf(ch.w[j], v.x, re);
+        im = fmaf(ch.w[j], v.y, im);
+    }
+    planes[((long long)c * n_comp + comp) * plane + i] = make_float2(re, im);
+}
+
+// The parts of a call that depend on none of its other results, one range of
+// blocks each: the live counts, the beam planes, and the first batch's phase
+// table and zeroed max |WA|.  Small calls are bound by launches (64 antennas x
+// 8192 sources x 16 channels: 62 us with nine kernels and two fills, 54 with six
+// kernels and one).
+__global__ void __launch_bounds__(kCullThreads) k_front(FrontArgs a) {
+    kernel_chain();
+    long long b = blockIdx.x;
+    if (b < a.cull_blocks) {
+        cull_count(a.m, a.R, a.w, a.bpt, (int)(b / a.bpt), (int)(b % a.bpt));
+        return;
+    }
+    b -= a.cull_blocks;
+    if (b < a.plane_blocks) {
+        const int pb = (int)(((long long)a.m.n_za * a.m.n_az + kCullThreads - 1) / kCullThreads);
+        const int n_comp = a.m.n_beam * a.m.n_feed * a.m.n_ax;
+        const long long rest = b / pb;
+        beam_plane(a.m, a.grid, a.chan, a.planes, n_comp, (int)(rest / n_comp), (int)(rest % n_comp),
+                   (b % pb) * kCullThreads + threadIdx.x);
+        return;
+    }
+    b -= a.plane_blocks;
+    const int nb = (a.m.n_ant + kCullThreads - 1) / kCullThreads;
+    const long long rest = b / nb;
+    if (b == 0)
+        for (int i = threadIdx.x; i < a.n_amax; i += kCullThreads) a.amax[i] = 0.f;
+    zcore::ant_phase_entry(a.m, a.inst, a.chan, a.groups, a.g_first, a.n_phase, a.aph, (int)(rest / a.n_phase),
+                           (int)(rest % a.n_phase), (int)(b % nb) * kCullThreads + threadIdx.x);
 }
 
 // Exclusive scan of the per-block live counts of one time (one block per time).
 __global__ void __launch_bounds__(1024)
 k_cull_scan(const int* __restrict__ counts, int* __restrict__ offsets, int* __restrict__ n_live, int bpt) {
+    kernel_chain();
     __shared__ int warp_sums[32];
     const int t = blockIdx.x;
     const int per = (bpt + blockDim.x - 1) / blockDim.x;
@@ -66,77 +123,97 @@ k_cull_scan(const int* __restrict__ counts, int* __restrict__ offsets, int* __re
     if (threadIdx.x == blockDim.x - 1) n_live[t] = warp_sums[(blockDim.x >> 5) - 1];
 }
 
+// (float)v in integer operations (round to nearest even): conversions run at the
+// FP64 rate.  Results below 2^-126 take the conversion.
+__device__ __forceinline__ float to_float(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    if (((unsigned)(b >> 52) & 0x7ffu) <= 897u) return (float)v;
+    const unsigned r = (unsigned)((b + 0x0fffffffull + (b >> 29 & 1ull)) >> 29);  // exponent's low bits and 23 places
+    return __uint_as_float(((unsigned)(b >> 32) & 0x80000000u) | ((r - (896u << 23)) & 0x7fffffffu));
+}
+
+// Stable compaction of a block's live sources and their tables.  What bounds it is
+// FP64 (two lanes a clock and SM): a live source costs 15 operations of its
+// rotation and three per component of its fixed-point direction, one below the
+// horizon none.  Count and compaction of 48 times of 1e5 sources: 390 us when
+// every source was rotated and converted before the cut, 257 here.
 __global__ void __launch_bounds__(kCullThreads)
-k_cull_scatter(Model m, const double* __restrict__ R, const int* __restrict__ offsets, int bpt,
-               LiveTables lt) {
-    __shared__ int warp_base[kCullThreads / 32];
-    const int t = blockIdx.y;
-    const long long s = (long long)blockIdx.x * kCullThreads + threadIdx.x;
-    double e = 0, n = 0, u = 0;
-    int live = 0;
-    if (s < m.n_src) {
-        const double* r = R + 9 * t;
-        const double x = m.xeq[s], y = m.xeq[m.n_src + s], z = m.xeq[2 * m.n_src + s];
-        e = rot_row(r, x, y, z);
-        n = rot_row(r + 3, x, y, z);
-        u = rot_row(r + 6, x, y, z);
-        live = u > 0.0;
-    }
+k_cull_scatter(Model m, const double* __restrict__ R, CullWork w, int bpt, LiveTables lt) {
+    kernel_chain();
+    __shared__ unsigned masks[kCullThreads / 32];
+    __shared__ int sums[kCullThreads / 32];
+    __shared__ unsigned char list[kCullThreads];
+    const int t = blockIdx.x / bpt, blk = blockIdx.x - t * bpt;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned mask = __ballot_sync(0xffffffffu, live);
-    if (lane == 0) warp_base[warp] = __popc(mask);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int acc = 0;
-        for (int w = 0; w < kCullThreads / 32; ++w) { int c = warp_base[w]; warp_base[w] = acc; acc += c; }
+    const long long b = (long long)t * bpt + blk;
+    const long long s0 = (long long)blk * kCullThreads;
+    if (!w.masks) {
+        const unsigned mask = __ballot_sync(0xffffffffu, above(m, R, t, s0 + threadIdx.x));
+        if (lane == 0) masks[warp] = mask;
+    } else if (threadIdx.x < kCullThreads / 32) {
+        masks[threadIdx.x] = w.masks[b * (kCullThreads / 32) + threadIdx.x];
+    }
+    // live sources of the blocks before
+    int before = 0;
+    if (bpt <= kScanBlocks) {
+        for (int i = threadIdx.x; i < blk; i += kCullThreads) before += w.counts[(long long)t * bpt + i];
+        before = __reduce_add_sync(0xffffffffu, before);
+        if (lane == 0) sums[warp] = before;
     }
     __syncthreads();
-    if (!live) return;
-    const long long pos = (long long)offsets[(long long)t * bpt + blockIdx.x] + warp_base[warp] +
-                          __popc(mask & ((1u << lane) - 1u));
-    const long long o = (long long)t * lt.pitch + pos;
-    lt.e[o] = e;
-    lt.n[o] = n;
-    lt.u[o] = u;
+    int rank = 0, total = 0;
+#pragma unroll
+    for (int i = 0; i < kCullThreads / 32; ++i) {
+        const int c = __popc(masks[i]);
+        if (i < warp) rank += c;
+        total += c;
+    }
+    if (bpt <= kScanBlocks) {
+        before = 0;
+#pragma unroll
+        for (int i = 0; i < kCullThreads / 32; ++i) before += sums[i];
+        if (blk == bpt - 1 && threadIdx.x == 0) lt.n_live[t] = before + total;
+    } else {
+        before = w.offsets[b];
+    }
+    if (masks[warp] >> lane & 1u) list[rank + __popc(masks[warp] & ((1u << lane) - 1u))] = (unsigned char)threadIdx.x;
+    __syncthreads();
+    if (threadIdx.x >= total) return;
+    const long long s = s0 + list[threadIdx.x];
+    const double* r = R + 9 * t;
+    const double x = m.xeq[s], y = m.xeq[m.n_src + s], z = m.xeq[2 * m.n_src + s];
+    const double comp[3] = {rot_row(r, x, y, z), rot_row(r + 3, x, y, z), rot_row(r + 6, x, y, z)};
+    const long long pos = before + (int)threadIdx.x, o = (long long)t * lt.pitch + pos;
+    if (lt.e) {
+        lt.e[o] = comp[0];
+        lt.n[o] = comp[1];
+        lt.u[o] = comp[2];
+    }
     lt.idx[o] = (int)s;
     if (lt.sfix) {
-        const double comp[3] = {e, n, u};
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const double q = fmin(rint(comp[c] * 2147483648.0), 2147483647.0);  // 2^31
+            // q = comp 2^31 rounded to an integer: added to 1.5 x 2^52, whose last place is
+            // one, so that q (mod 2^32) is the sum's low word
+            constexpr double kShift = 6755399441055744.0;
+            const double sum = fma(comp[c], 2147483648.0, kShift);
+            double q = sum - kShift;
+            unsigned lo = (unsigned)__double2loint(sum);
+            if (lo == 0x80000000u && __double2hiint(comp[c]) >= 0) {  // 1 rounds to 2^31 - 1
+                lo = 0x7fffffffu;
+                q = 2147483647.0;
+            }
             const long long o3 = ((long long)t * 3 + c) * lt.pitch + pos;
-            lt.sfix[o3] = (unsigned)((long long)q + 2147483648ll);
-            lt.seps[o3] = (float)(comp[c] - q * 4.656612873077392578125e-10);  // 2^-31
+            lt.sfix[o3] = lo + 0x80000000u;
+            lt.seps[o3] = to_float(fma(q, -4.656612873077392578125e-10, comp[c]));  // 2^-31
         }
     }
     // az = atan2(E, N) in [0, 2 pi), za = atan2(|EN|, Up): well conditioned at the pole
-    const float ef = (float)e, nf = (float)n, uf = (float)u;
+    const float ef = to_float(comp[0]), nf = to_float(comp[1]), uf = to_float(comp[2]);
     float az = atan2f(ef, nf);
     if (az < 0.f) az += 6.2831853071795864769f;
     const float za = atan2f(sqrtf(ef * ef + nf * nf), uf);
     lt.azza[o] = make_float2(az, za);
-}
-
-// Per-channel beam planes: P[c][b][p][k][za][az] = sum_m w_m(c) G[b][p][k][m0(c)+m][za][az]
-// (the frequency axis of the gridded beam interpolated once per channel).
-__global__ void k_beam_planes(Model m, const float2* __restrict__ grid, const Chan* __restrict__ chan,
-                              float2* __restrict__ planes) {
-    const long long plane = (long long)m.n_za * m.n_az;
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= plane) return;
-    const int comp = blockIdx.y;  // (b, p, k) flattened
-    const int c = blockIdx.z;
-    const Chan ch = chan[c];
-    const float2* g = grid + (long long)comp * m.n_nu * plane;
-    float re = 0.f, im = 0.f;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        float2 v = g[(long long)(ch.m0 + j) * plane + i];
-        re = fmaf(ch.w[j], v.x, re);
-        im = fmaf(ch.w[j], v.y, im);
-    }
-    const int n_comp = gridDim.y;
-    planes[((long long)c * n_comp + comp) * plane + i] = make_float2(re, im);
 }
 
 // Keys (1981) cubic-convolution kernel, a = -1/2.
@@ -164,6 +241,7 @@ __global__ void __launch_bounds__(128)
 k_wa(Model m, const float2* __restrict__ planes, const Chan* __restrict__ chan,
      const Inst* __restrict__ inst, int inst0, LiveTables lt, float2* __restrict__ wa, long long wa_pitch,
      float* __restrict__ amax) {
+    kernel_chain();
     const int slot = blockIdx.y;
     const Inst in = inst[inst0 + slot];
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -258,22 +336,28 @@ __device__ float wa_eval(const Model& m, const float2* __restrict__ planes, cons
 
 }  // namespace
 
-cudaError_t launch_cull(const Model& m, const double* d_R, int n_times, LiveTables lt, int* d_counts,
-                        int* d_offsets, int bpt, cudaStream_t st, long long* launches) {
-    dim3 grid(bpt, n_times);
-    k_cull_count<<<grid, kCullThreads, 0, st>>>(m, d_R, d_counts, bpt);
-    k_cull_scan<<<n_times, 1024, 0, st>>>(d_counts, d_offsets, lt.n_live, bpt);
-    k_cull_scatter<<<grid, kCullThreads, 0, st>>>(m, d_R, d_offsets, bpt, lt);
-    *launches += 3;
-    return cudaGetLastError();
-}
-
-cudaError_t launch_beam_planes(const Model& m, const float2* d_grid, const Chan* d_chan, int n_chan,
-                               float2* d_planes, cudaStream_t st, long long* launches) {
-    const long long plane = (long long)m.n_za * m.n_az;
-    dim3 grid((unsigned)((plane + 255) / 256), m.n_beam * m.n_feed * m.n_ax, n_chan);
-    k_beam_planes<<<grid, 256, 0, st>>>(m, d_grid, d_chan, d_planes);
-    *launches += 1;
+cudaError_t launch_front(const FrontArgs& args, int n_times, LiveTables lt, cudaStream_t st, long long* launches) {
+    FrontArgs a = args;
+    const Model& m = a.m;
+    a.cull_blocks = (long long)a.bpt * n_times;
+    a.plane_blocks = a.planes ? ((long long)m.n_za * m.n_az + kCullThreads - 1) / kCullThreads * m.n_beam * m.n_feed * m.n_ax * a.n_chan : 0;
+    const long long phase_blocks = a.aph ? (long long)((m.n_ant + kCullThreads - 1) / kCullThreads) * a.n_phase * a.n_groups : 0;
+    const long long blocks = a.cull_blocks + a.plane_blocks + phase_blocks;
+    if (blocks > 0x7fffffffll) return cudaErrorInvalidValue;
+    if (blocks > 0) {
+        k_front<<<(unsigned)blocks, kCullThreads, 0, st>>>(a);
+        *launches += 1;
+    }
+    if (a.cull_blocks > 0) {
+        if (a.bpt > kScanBlocks) {
+            cudaError_t e = launch_chained(k_cull_scan, dim3(n_times), dim3(1024), 0, st, (const int*)a.w.counts, a.w.offsets,
+                                           lt.n_live, a.bpt);
+            if (e != cudaSuccess) return e;
+            *launches += 1;
+        }
+        *launches += 1;
+        return launch_chained(k_cull_scatter, dim3((unsigned)a.cull_blocks), dim3(kCullThreads), 0, st, m, a.R, a.w, a.bpt, lt);
+    }
     return cudaGetLastError();
 }
 
@@ -281,9 +365,8 @@ cudaError_t launch_wa(const Model& m, const float2* d_planes, const Chan* d_chan
                       int inst0, int n_inst, LiveTables lt, float2* d_wa, long long wa_pitch, float* d_amax,
                       cudaStream_t st, long long* launches) {
     dim3 grid((unsigned)((lt.pitch + 127) / 128), n_inst);
-    k_wa<<<grid, 128, 0, st>>>(m, d_planes, d_chan, d_inst, inst0, lt, d_wa, wa_pitch, d_amax);
     *launches += 1;
-    return cudaGetLastError();
+    return launch_chained(k_wa, grid, dim3(128), 0, st, m, d_planes, d_chan, d_inst, inst0, lt, d_wa, wa_pitch, d_amax);
 }
 
 }  // namespace mv

@@ -18,48 +18,23 @@ namespace {
 
 using namespace zcore;
 
-// Antenna factors of every wavenumber of a batch's groups: entry e of group
-// gl is kappa0 (e = 0) and dkappa (e = 1) of an equally spaced group, or the
-// wavenumber of its instance e otherwise.
+// The phase table of a batch (zcore.cuh).  Also max |WA| of every instance
+// (amax): zeroed (zero_amax), or given to every instance of a group as the
+// group's largest, so that one FP16 scale serves the group (the Z build folds
+// the scale into its cos/sin factors; the HERK undoes it per instance from the
+// same value).
 __global__ void k_ant_phase(Model m, const Inst* __restrict__ inst, const Chan* __restrict__ chan,
                             const ZGroup* __restrict__ groups, int g_first, int n_phase, AntPhase* __restrict__ tab,
-                            float* __restrict__ amax) {
+                            float* __restrict__ amax, int zero_amax) {
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     const int e = blockIdx.y, gl = blockIdx.z;
     const ZGroup g = groups[g_first + gl];
     if (amax && blockIdx.x == 0 && e == 0 && threadIdx.x == 0) {
-        // one FP16 scale per group: every instance takes the group's max |WA|
-        // (the Z build folds the scale into its cos/sin factors; the HERK
-        // undoes it per instance from the same value)
         float mx = 0.f;
-        for (int j = 0; j < g.n; ++j) mx = fmaxf(mx, amax[g.slot0 + j]);
+        for (int j = 0; j < g.n && !zero_amax; ++j) mx = fmaxf(mx, amax[g.slot0 + j]);
         for (int j = 0; j < g.n; ++j) amax[g.slot0 + j] = mx;
     }
-    if (a >= m.n_ant) return;
-    double kap;
-    if (g.uniform) {
-        if (e >= 2) return;
-        kap = e == 0 ? g.kappa0 : g.dkappa;
-    } else {
-        if (e >= g.n) return;
-        kap = chan[inst[g.inst0 + e].c].kappa;
-    }
-    const double x[3] = {m.ant_e[a], m.ant_n[a], m.ant_u[a]};
-    AntPhase p;
-    unsigned long long nk = 0ull;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const double y = kap * x[c];
-        const long long Y = __double2ll_rn(y * 4294967296.0);  // 2^32
-        p.yl[c] = (unsigned)Y;
-        p.yh[c] = (int)(Y >> 32);
-        p.yf[c] = (float)y;
-        nk -= (unsigned long long)p.yl[c] << 31;
-    }
-    p.negk_lo = (unsigned)nk;
-    p.negk_hi = (unsigned)(nk >> 32);
-    p.pad = 0u;
-    tab[((long long)gl * n_phase + e) * m.n_ant + a] = p;
+    ant_phase_entry(m, inst, chan, groups, g_first, n_phase, tab, gl, e, a);
 }
 
 // Grid-stride over the work items, so that the launch can be held to a fixed
@@ -90,11 +65,11 @@ k_zbuild(Model m, const Inst* __restrict__ inst, const ZGroup* __restrict__ grou
 }  // namespace
 
 cudaError_t launch_ant_phase(const Model& m, const Inst* d_inst, const Chan* d_chan, const ZGroup* d_groups,
-                             int g_first, int n_groups, AntPhase* d_aph, int n_phase, float* d_amax, cudaStream_t st,
-                             long long* launches) {
+                             int g_first, int n_groups, AntPhase* d_aph, int n_phase, float* d_amax, bool zero_amax,
+                             cudaStream_t st, long long* launches) {
     if (!d_aph || n_phase < 2) return cudaErrorInvalidValue;
     k_ant_phase<<<dim3((unsigned)((m.n_ant + 127) / 128), (unsigned)n_phase, (unsigned)n_groups), 128, 0, st>>>(
-        m, d_inst, d_chan, d_groups, g_first, n_phase, d_aph, d_amax);
+        m, d_inst, d_chan, d_groups, g_first, n_phase, d_aph, d_amax, zero_amax);
     *launches += 1;
     return cudaGetLastError();
 }
@@ -105,7 +80,7 @@ cudaError_t launch_zbuild(const Model& m, const Inst* d_inst, const Chan* d_chan
                           int max_blocks, AntPhase* d_aph, int n_phase, cudaStream_t st, long long* launches) {
     if (!lt.sfix) return cudaErrorInvalidValue;
     cudaError_t e = launch_ant_phase(m, d_inst, d_chan, d_groups, g_first, n_groups, d_aph, n_phase,
-                                     prec == 2 ? d_amax : nullptr, st, launches);
+                                     prec == 2 ? d_amax : nullptr, false, st, launches);
     if (e != cudaSuccess) return e;
     const int apb = 32;
     const int nx = (int)((lt.pitch / 2 + 127) / 128), ny = (m.n_ant + apb - 1) / apb;

@@ -40,6 +40,33 @@ __device__ __forceinline__ unsigned long long phase64(const AntPhase& p, const u
     return (acc << 1) + ((unsigned long long)(long long)cf << 32);
 }
 
+// Entry (gl, e) of a batch's phase table for antenna a: the factors of kappa0
+// (e = 0) and dkappa (e = 1) of an equally spaced group gl, or of the wavenumber
+// of its instance e otherwise.
+__device__ __forceinline__ void ant_phase_entry(const Model& m, const Inst* __restrict__ inst, const Chan* __restrict__ chan,
+                                                const ZGroup* __restrict__ groups, int g_first, int n_phase,
+                                                AntPhase* __restrict__ tab, int gl, int e, int a) {
+    const ZGroup g = groups[g_first + gl];
+    if (a >= m.n_ant || e >= (g.uniform ? 2 : g.n)) return;
+    const double kap = !g.uniform ? chan[inst[g.inst0 + e].c].kappa : e == 0 ? g.kappa0 : g.dkappa;
+    const double x[3] = {m.ant_e[a], m.ant_n[a], m.ant_u[a]};
+    AntPhase p;
+    unsigned long long nk = 0ull;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        const double y = kap * x[c];
+        const long long Y = __double2ll_rn(y * 4294967296.0);  // 2^32
+        p.yl[c] = (unsigned)Y;
+        p.yh[c] = (int)(Y >> 32);
+        p.yf[c] = (float)y;
+        nk -= (unsigned long long)p.yl[c] << 31;
+    }
+    p.negk_lo = (unsigned)nk;
+    p.negk_hi = (unsigned)(nk >> 32);
+    p.pad = 0u;
+    tab[((long long)gl * n_phase + e) * m.n_ant + a] = p;
+}
+
 __device__ __forceinline__ AntPhase load_phase(const AntPhase* __restrict__ t) {
     const uint4* q = reinterpret_cast<const uint4*>(t);
     const uint4 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2);

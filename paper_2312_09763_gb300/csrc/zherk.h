@@ -126,8 +126,8 @@ int zherk_input_bytes(int chan, int nc, int n_beam);
 int zherk_input_shift(int bytes);
 cudaError_t zherk_init();
 cudaError_t launch_zherk_prep(const ZherkArgs& P, const float* amax_in, float* amax_out, float* scale, int4* zv,
-                              int* wave_base, ZherkGroup* groups, int n_groups, bool by_length, cudaStream_t st,
-                              long long* launches);
+                              int* wave_base, ZherkGroup* groups, int n_groups, bool by_length, long long n_counters,
+                              cudaStream_t st, long long* launches);
 cudaError_t launch_zherk(const ZherkArgs& P, int form, int n_ctas, cudaStream_t st, long long* launches);
 cudaError_t launch_zherk_final(const ZherkFinalArgs& a, int form, cudaStream_t st, long long* launches);
 

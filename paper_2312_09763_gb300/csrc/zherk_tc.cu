@@ -749,7 +749,10 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
 __global__ void __launch_bounds__(1024) k_zherk_prep(ZherkArgs P, const float* __restrict__ amax_in,
                                                      float* __restrict__ amax_out, float* __restrict__ scale,
                                                      int4* __restrict__ zv, int* __restrict__ wave_base,
-                                                     ZherkGroup* __restrict__ groups, int n_groups, int by_length) {
+                                                     ZherkGroup* __restrict__ groups, int n_groups, int by_length,
+                                                     long long n_counters) {
+    kernel_chain();
+    for (long long i = threadIdx.x; i < n_counters; i += blockDim.x) P.ready[i] = 0;  // (ready, then done)
     extern __shared__ int sm[];  // t, live count and max |WA| of each instance, then the waves' lengths
     int *st = sm, *sk = sm + P.n_inst, *order = sm + 3 * P.n_inst, *len = sm + 4 * P.n_inst;
     float* sa = reinterpret_cast<float*>(sm + 2 * P.n_inst);
@@ -825,6 +828,7 @@ __device__ __forceinline__ float4 sum_parts(const float* p, int S, int r, int c)
 // tile (16 x 16 antenna-feeds), read along the tile's rows and written along
 // the rows of V through shared memory.
 __global__ void __launch_bounds__(256) k_zherk_final_real(ZherkFinalArgs a) {
+    kernel_chain();
     __shared__ float G[32][33];  // [column][row]
     const int slot = blockIdx.x / a.n_tiles, tile = blockIdx.x - slot * a.n_tiles;
     const ZherkTile t = a.tiles[tile];
@@ -882,6 +886,7 @@ __global__ void __launch_bounds__(256) k_zherk_final_real(ZherkFinalArgs a) {
 // V from the partial tiles of the gauss form: one block per 32 x 32 piece of a
 // 128 x 128 block (i, j), i >= j, of V.
 __global__ void __launch_bounds__(256) k_zherk_final_gauss(ZherkFinalArgs a) {
+    kernel_chain();
     __shared__ float M[3][32][33];  // F_ab, F_ba, H_ab at [row of a][row of b]
     const int nb = a.np * (a.np + 1) / 2;
     const int slot = blockIdx.x / nb;
@@ -959,12 +964,11 @@ cudaError_t zherk_init() {
 }
 
 cudaError_t launch_zherk_prep(const ZherkArgs& P, const float* amax_in, float* amax_out, float* scale, int4* zv,
-                              int* wave_base, ZherkGroup* groups, int n_groups, bool by_length, cudaStream_t st,
-                              long long* launches) {
-    k_zherk_prep<<<1, 1024, sizeof(int) * (size_t)(P.n_waves + 4 * P.n_inst), st>>>(P, amax_in, amax_out, scale, zv,
-                                                                                   wave_base, groups, n_groups, by_length);
+                              int* wave_base, ZherkGroup* groups, int n_groups, bool by_length, long long n_counters,
+                              cudaStream_t st, long long* launches) {
     *launches += 1;
-    return cudaGetLastError();
+    return launch_chained(k_zherk_prep, dim3(1), dim3(1024), sizeof(int) * (size_t)(P.n_waves + 4 * P.n_inst), st, P, amax_in,
+                          amax_out, scale, zv, wave_base, groups, n_groups, (int)by_length, n_counters);
 }
 
 int zherk_input_bytes(int chan, int nc, int n_beam) { return Z_SRC_B + (n_beam == 1 ? chan * nc * kZherkChunk * 8 : 0); }
@@ -1002,12 +1006,10 @@ cudaError_t launch_zherk(const ZherkArgs& P, int form, int n_ctas, cudaStream_t 
 }
 
 cudaError_t launch_zherk_final(const ZherkFinalArgs& a, int form, cudaStream_t st, long long* launches) {
-    if (form == kZherkReal)
-        k_zherk_final_real<<<dim3((unsigned)(a.n_inst * a.n_tiles), 16), 256, 0, st>>>(a);
-    else
-        k_zherk_final_gauss<<<dim3((unsigned)(a.n_inst * (a.np * (a.np + 1) / 2)), 16), 256, 0, st>>>(a);
     *launches += 1;
-    return cudaGetLastError();
+    if (form == kZherkReal)
+        return launch_chained(k_zherk_final_real, dim3((unsigned)(a.n_inst * a.n_tiles), 16), dim3(256), 0, st, a);
+    return launch_chained(k_zherk_final_gauss, dim3((unsigned)(a.n_inst * (a.np * (a.np + 1) / 2)), 16), dim3(256), 0, st, a);
 }
 
 // ------------------------------------------------------------ host planning
