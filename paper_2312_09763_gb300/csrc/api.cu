@@ -465,9 +465,10 @@ constexpr long long kRingBytes = 96ll << 20;
 constexpr long long kPartialBytes = 1ll << 30;
 
 // Where the product of panels (i, j) of F (kind 0) and H (kind 1) is in a gauss tile list.
-std::vector<int> gauss_tile_of(const std::vector<ZherkTile>& tiles, int np) {
+std::vector<int> gauss_tile_of(const std::vector<ZherkTile>& tiles, int np, int panel) {
     std::vector<int> of(2 * np * np, 0);
-    for (size_t k = 0; k < tiles.size(); ++k) of[(tiles[k].kind * np + tiles[k].r0 / 128) * np + tiles[k].c0 / 128] = (int)k;
+    for (size_t k = 0; k < tiles.size(); ++k)
+        of[(tiles[k].kind * np + tiles[k].r0 / panel) * np + tiles[k].c0 / panel] = (int)k;
     return of;
 }
 
@@ -487,7 +488,7 @@ bool plan_stream(mv_ctx* c, Plan& P, Prepared& p, std::vector<uint8_t>& tab) {
     const Model& m = c->model;
     static const std::vector<ZherkTile> whole_v;
     const bool covered = P.unique && c->red.kind != 0;
-    const std::vector<ZherkTile> cover = covered ? c->red_tiles : P.unique ? zherk_triangle(p.rows) : whole_v;
+    const std::vector<ZherkTile> cover = covered ? c->red_tiles : P.unique ? zherk_triangle(p.rows, 128) : whole_v;
     const long long wa_slot = 8ll * p.ncomp * p.pitch;
     const long long budget = 8ll << 30;
     int B = (int)std::max(1ll, std::min<long long>(kMaxBatch, budget / wa_slot));
@@ -563,9 +564,9 @@ bool plan_stream(mv_ctx* c, Plan& P, Prepared& p, std::vector<uint8_t>& tab) {
         b.items = put(items.data(), items.size() * sizeof(int));
         b.group0 = put(group0.data(), group0.size() * sizeof(int));
         b.tiles = put(z->tiles.data(), z->tiles.size() * sizeof(ZherkTile));
-        b.np = (p.N + 127) / 128;
+        b.np = (p.N + z->panel - 1) / z->panel;
         if (z->form == kZherkGauss) {
-            const std::vector<int> of = gauss_tile_of(z->tiles, b.np);
+            const std::vector<int> of = gauss_tile_of(z->tiles, b.np, z->panel);
             b.tile_of = put(of.data(), of.size() * sizeof(int));
         }
         if (covered) {
@@ -730,7 +731,7 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
         p.f32_slots = (int)std::max(1ll, std::min<long long>(max_slots, kPartialBytes / (long long)slot));
         p.f32_tiles = put_table(ztab, p.f32.tiles.data(), p.f32.tiles.size() * sizeof(ZherkTile));
         if (p.f32.form == kZherkGauss) {
-            const std::vector<int> of = gauss_tile_of(p.f32.tiles, (p.N + 127) / 128);
+            const std::vector<int> of = gauss_tile_of(p.f32.tiles, (p.N + 127) / 128, 128);
             p.f32_tile_of = put_table(ztab, of.data(), of.size() * sizeof(int));
         }
         if ((s = ensure(c, c->partial, slot * p.f32_slots))) return s;
@@ -868,6 +869,7 @@ cudaError_t enqueue_herk(mv_ctx* c, const Prepared& p, const Plan::Batch& b, con
             f.S = p.f32.split;
             f.N = p.N;
             f.np = (p.N + 127) / 128;
+            f.panel = 128;
             f.V = p.Vout;
             e = launch_herk_fp32(d_inst, f.inst0, f.n_inst, p.lt, c->model.n_ax,
                                  (const float*)c->u[k].p + (size_t)i * p.f32.rows * p.k_pitch, p.f32.rows,
@@ -1005,6 +1007,7 @@ mv_status enqueue_stream(mv_ctx* c, const Prepared& p, size_t i, bool have_phase
     z.zv = (const int4*)c->zorder.p;
     z.ring = (uint8_t*)c->ring.p;
     z.rows = b.plan->rows;
+    z.panel = b.plan->panel;
     z.map_rows = b.plan->form == kZherkReal ? b.plan->rows : p.N;
     z.V = b.plan->V;
     z.S = b.plan->S;
@@ -1043,6 +1046,7 @@ mv_status enqueue_stream(mv_ctx* c, const Prepared& p, size_t i, bool have_phase
     f.S = z.S;
     f.N = p.N;
     f.np = b.np;
+    f.panel = b.plan->panel;
     f.V = p.Vout;
     f.ho = p.ho;
     f.limits = p.ho.uidx && c->red.kind != 0 ? (const int2*)(tab + b.limits) : nullptr;
@@ -1227,7 +1231,7 @@ std::vector<long long> graph_key(mv_ctx* c, const Plan& P, const Prepared& p, co
     k.push_back(p.n_phase);
     for (const StreamBatch& b : p.sb)
         for (long long x : {(long long)b.plan->V, (long long)b.plan->S, (long long)b.plan->waves, (long long)b.plan->form,
-                            (long long)b.plan->n_jobs, (long long)b.plan->n_jobs_last, (long long)b.plan->rows,
+                            (long long)b.plan->n_jobs, (long long)b.plan->n_jobs_last, (long long)b.plan->rows, (long long)b.plan->panel,
                             (long long)b.plan->tiles.size(),
                             (long long)b.jobs, (long long)b.groups, (long long)b.items, (long long)b.group0,
                             (long long)b.tiles, (long long)b.tile_of, (long long)b.limits, (long long)b.n_groups,

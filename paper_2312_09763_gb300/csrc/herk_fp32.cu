@@ -205,7 +205,7 @@ Fp32Plan herk_fp32_plan(int N, int n_ax, int n_inst, double est_live, int n_sms)
     for (int form = kZherkReal; form <= kZherkGauss; ++form) {
         Fp32Plan z;
         z.form = form;
-        z.tiles = form == kZherkReal ? zherk_triangle(2 * N) : zherk_gauss_tiles(N);
+        z.tiles = form == kZherkReal ? zherk_triangle(2 * N, BT) : zherk_gauss_tiles(N, BT);
         z.rows = form == kZherkReal ? 2 * N : 3 * N;
         z.plane_rows = form == kZherkReal ? 2 * N : N;
         double area = 0;

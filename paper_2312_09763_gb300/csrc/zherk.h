@@ -26,22 +26,22 @@ constexpr int kZherkChan = 20;       // channels x components a group may have
 //          Re V_ab = H_ab - (F_ab + F_ba), Im V_ab = F_ba - F_ab.
 enum ZherkForm : int { kZherkReal = 0, kZherkGauss = 1 };
 
-// A 128 x 128 product of ring rows: A rows [ra, ra + 128) of an instance times
-// B rows [rb, rb + 128) (gauss: plane * N + antenna-feed).  r0, c0: the rows and columns of the product it
+// A product of panels of ring rows: A rows [ra, ra + panel) of an instance times
+// B rows [rb, rb + panel) (gauss: plane * N + antenna-feed).  r0, c0: the rows and columns of the product it
 // stands for (antenna-feeds of F or H with the gauss form, rows of U with the
 // real one); trans: its rows hold the product's columns.
 struct ZherkTile {
     int ra, rb, r0, c0, kind, trans;  // kind: 0 G (real) or F, 1 H
 };
 
-// The work of one SM in one wave: one A box of 128 ring rows and one or two B
-// boxes (N = 128 or 256).  n = 0: none.
+// The work of one SM in one wave: one A box of a panel of ring rows (128 rows of MMA,
+// the last ones unused) and one or two B boxes.  n: columns of MMA, 0: none.
 struct ZherkJob {
     int n, nbox;
     int a, b;                        // A's box; B's first box (the second one follows it)
     int row[4], plane[4];            // first row of each box within the instance (and its plane)
     int tile[2];
-    int v, pad;                      // instance within the wave
+    int v, np;                       // instance within the wave, products
 };
 
 // Channels of one time (and one source range) whose Z is built together:
@@ -56,7 +56,7 @@ struct alignas(16) ZherkGroup {
 
 struct ZherkPlan {
     int form = kZherkReal, n_ax = 1;
-    int rows = 0;                    // ring rows per instance
+    int rows = 0, panel = 128;       // ring rows per instance, rows of a panel
     int V = 0, S = 0, waves = 0;     // instances per wave, source ranges per instance
     int n_jobs = 0, n_jobs_last = 0;
     std::vector<ZherkTile> tiles;
@@ -75,7 +75,7 @@ struct ZherkArgs {
     int n_phase;
     const int4* zv;                  // virtual instances: slot, time, first source chunk, chunks
     uint8_t* ring;
-    int rows, map_rows;              // ring rows per instance; rows of one plane
+    int rows, map_rows, panel;       // ring rows per instance; rows of one plane, of a panel
     int V, S, n_waves, v_last;       // v_last: instances of the last wave
     const int* wave_base;            // [n_waves + 1] first chunk of each wave
     const int* wave_items;           // [n_waves] groups
@@ -100,17 +100,21 @@ struct ZherkFinalArgs {
     const float* partial;
     const ZherkTile* tiles;
     const int* tile_of;              // gauss: [2][np][np] tile of F_ij and of H_ij (i >= j), np panels
-    int n_tiles, S, N, np;
+    int n_tiles, S, N, np, panel;    // np: panels of a plane (gauss)
     float2* V;
     HerkOut ho;                      // uidx NULL: the full V
     const int2* limits;              // unique: row and column limits of every tile
 };
 
+// Rows of a panel: those of a plane split evenly over as few panels of at most 128 rows
+// as there can be, in eights (350 rows: three of 120, so that two products side by
+// side are 240 columns of MMAs instead of 256; 131: two of 72).
+int zherk_panel(int rows);
 // Products of one instance: in the real form the lower triangle of 2N rows,
-std::vector<ZherkTile> zherk_triangle(int rows);
+std::vector<ZherkTile> zherk_triangle(int rows, int panel);
 
 // and in the gauss form of N antenna-feeds.
-std::vector<ZherkTile> zherk_gauss_tiles(int N);
+std::vector<ZherkTile> zherk_gauss_tiles(int N, int panel);
 
 // Plan for n_inst instances; cover: the real-form tiles to compute (empty: the
 // whole V of N antenna-feeds, in either form).  est_live: live sources

@@ -54,7 +54,7 @@ namespace {
 using namespace tc;
 using namespace zcore;
 
-constexpr int BOX = 128 * 128;            // bytes of a box: 128 rows x 32 columns, hi and lo
+constexpr int BOX = 128 * 128;            // bytes of the largest box: 128 rows x 32 columns, hi and lo
 constexpr int MAX_BOX = 3;                // boxes of a stage: A and two of B
 constexpr int STAGE = MAX_BOX * BOX;      // 48 KB
 constexpr int STAGES = 4;
@@ -364,7 +364,7 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
     const uint32_t tmem_base = *tmem_slot;
     const uint32_t sbase = smem_u32(smem);
     const ZherkJob& J = P.jobs[blockIdx.x];   // this SM's job, the same in every wave
-    const int jn = J.n;
+    const int jn = J.n, pan = P.panel, box_b = pan * 128;
     // whether the job's instance is in wave w
     auto has_job = [&](int w) { return jn > 0 && (w < P.n_waves - 1 || J.v < P.v_last); };
 
@@ -386,6 +386,7 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                     // both loads of a piece go out together; the MMAs wait for this
 #pragma unroll
                     for (int g = 0; g < 128 / 16; ++g) {
+                        if (h * 128 + g * 16 >= jn) break;
                         uint32_t acc[16];
                         tmem_ld16(tl + g * 16, acc);
                         if (f > 0) {
@@ -409,11 +410,16 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
             }
             if (!ok || *abort_flag) break;
             if (h * 128 < jn) {
-                // partial tile, column-major [128][128] (coalesced along rows)
-                const int ks = (w * P.V + J.v) / P.n_inst;
-                float* p = P.partial + (((long long)v.x * P.n_tiles + J.tile[h]) * P.S + ks) * (128 * 128) + q4 * 32 + lane;
+                // partial tiles, column-major [128][128] (coalesced along rows); the second
+                // product's columns follow the first one's panel
+                const int ks = (w * P.V + J.v) / P.n_inst, cols = J.np * pan;
+                float* const p = P.partial + (long long)v.x * P.n_tiles * P.S * (128 * 128) + (long long)ks * (128 * 128) + q4 * 32 + lane;
+                float* const p0 = p + (long long)J.tile[0] * P.S * (128 * 128);
+                float* const p1 = p + (long long)J.tile[1] * P.S * (128 * 128) - pan * 128;
 #pragma unroll 1
                 for (int g = 0; g < 8; ++g) {
+                    const int c0 = h * 128 + g * 16;
+                    if (c0 >= cols) break;
                     uint32_t sum[16];
                     if (n_flush > 0) {
                         tmem_ld16(trun + g * 16, sum);
@@ -423,7 +429,8 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                         for (int i = 0; i < 16; ++i) sum[i] = 0u;
                     }
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) p[(g * 16 + i) * 128] = __uint_as_float(sum[i]);
+                    for (int i = 0; i < 16; ++i)
+                        if (c0 + i < cols) (c0 + i < pan ? p0 : p1)[(c0 + i) * 128] = __uint_as_float(sum[i]);
                 }
             }
         }
@@ -588,10 +595,10 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                         if (!ok) break;
                         while (landed <= it - STAGES && land()) {}  // (the stage was consumed, so it has landed)
                         if (elect_one()) {
-                            mbar_expect_tx(full(s), (uint32_t)(nbox * BOX));
+                            mbar_expect_tx(full(s), (uint32_t)(nbox * box_b));
 #pragma unroll
                             for (int b = 0; b < MAX_BOX; ++b)
-                                if (b < nbox) tma_load_3d(sbase + s * STAGE + b * BOX, &map, x0 + i * 64, pl[b], y[b], full(s));
+                                if (b < nbox) tma_load_3d(sbase + s * STAGE + b * box_b, &map, x0 + i * 64, pl[b], y[b], full(s));
                         }
                         __syncwarp();
                         ++it;
@@ -605,8 +612,8 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
             // MMA took 72-83 cycles to issue, more than the 64 of an N = 128 one.
             int it = 0, cg = 0;
             bool ok = true;
-            const uint64_t da = sdesc(sbase + J.a * BOX), db = sdesc(sbase + J.b * BOX);
-            const uint32_t id = idesc_f16(true, 128, 128) + ((uint32_t)(jn > 128 ? 16 : 0) << 17);
+            const uint64_t da = sdesc(sbase + J.a * box_b), db = sdesc(sbase + J.b * box_b);
+            const uint32_t id = idesc_f16(true, 128, 0) + ((uint32_t)(jn >> 3) << 17);
             const int jv = J.v, flush = P.flush;
             for (int w = 0; w < P.n_waves && ok; ++w) {
                 if (!has_job(w)) continue;
@@ -836,7 +843,7 @@ __global__ void __launch_bounds__(256) k_zherk_final_real(ZherkFinalArgs a) {
     const float* p = a.partial + ((long long)slot * a.n_tiles + tile) * a.S * (128 * 128);
     // the product's rows and columns this piece stands for
     const int pr = t.r0 + (t.trans ? bc : br), pc = t.c0 + (t.trans ? br : bc);
-    int rlim = 2 * a.N, clim = 2 * a.N;
+    int rlim = min(2 * a.N, t.r0 + a.panel), clim = min(2 * a.N, t.c0 + a.panel);
     if (a.limits) {
         rlim = min(rlim, a.limits[tile].x);
         clim = min(clim, a.limits[tile].y);
@@ -884,7 +891,7 @@ __global__ void __launch_bounds__(256) k_zherk_final_real(ZherkFinalArgs a) {
 }
 
 // V from the partial tiles of the gauss form: one block per 32 x 32 piece of a
-// 128 x 128 block (i, j), i >= j, of V.
+// block of panels (i, j), i >= j, of V.
 __global__ void __launch_bounds__(256) k_zherk_final_gauss(ZherkFinalArgs a) {
     kernel_chain();
     __shared__ float M[3][32][33];  // F_ab, F_ba, H_ab at [row of a][row of b]
@@ -893,8 +900,9 @@ __global__ void __launch_bounds__(256) k_zherk_final_gauss(ZherkFinalArgs a) {
     int i = 0, j = blockIdx.x - slot * nb;
     while (j > i) j -= ++i;
     const int ar = (blockIdx.y & 3) * 32, bc = (blockIdx.y >> 2) * 32;
-    const int A0 = i * 128 + ar, B0 = j * 128 + bc;
-    if (A0 >= a.N || B0 >= a.N || A0 + 31 < B0) return;
+    const int A0 = i * a.panel + ar, B0 = j * a.panel + bc;
+    const int A1 = min(a.N, (i + 1) * a.panel), B1 = min(a.N, (j + 1) * a.panel);
+    if (A0 >= A1 || B0 >= B1 || A0 + 31 < B0) return;
     const float* base = a.partial + (long long)slot * a.n_tiles * a.S * (128 * 128);
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
@@ -920,7 +928,7 @@ __global__ void __launch_bounds__(256) k_zherk_final_gauss(ZherkFinalArgs a) {
             const int x = k & 31, y = k >> 5;
             const int ia = pass ? x : y, ib = pass ? y : x;
             const int A = A0 + ia, B = B0 + ib;
-            if (A >= a.N || B >= a.N || A < B) continue;
+            if (A >= A1 || B >= B1 || A < B) continue;
             const float f = M[0][ia][ib], ft = M[1][ia][ib];
             const float re = ((M[2][ia][ib] - (f + ft)) * us) * us;
             const float im = A == B ? 0.f : ((ft - f) * us) * us;
@@ -931,12 +939,12 @@ __global__ void __launch_bounds__(256) k_zherk_final_gauss(ZherkFinalArgs a) {
 
 // The ring as [rows][planes][columns]: one plane of 2N-row instances (real), or
 // the planes X, Y and S of every antenna-feed (gauss).
-bool ring_map(CUtensorMap* map, const void* ring, int row_b, int planes, long long rows) {
+bool ring_map(CUtensorMap* map, const void* ring, int row_b, int planes, long long rows, int panel) {
     EncodeTiledFn enc = get_encode();
     if (!enc) return false;
     cuuint64_t dims[3] = {(cuuint64_t)row_b / 2, (cuuint64_t)planes, (cuuint64_t)rows};
     cuuint64_t strides[2] = {(cuuint64_t)row_b, (cuuint64_t)row_b * planes};
-    cuuint32_t box[3] = {64, 1, 128};
+    cuuint32_t box[3] = {64, 1, (cuuint32_t)panel};
     cuuint32_t estr[3] = {1, 1, 1};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(ring), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -976,7 +984,8 @@ int zherk_input_shift(int bytes) { return bytes * 8 <= 2 * Z_BUF ? 3 : bytes * 4
 
 cudaError_t launch_zherk(const ZherkArgs& P, int form, int n_ctas, cudaStream_t st, long long* launches) {
     CUtensorMap map;
-    if (!ring_map(&map, P.ring, zherk_row_bytes(P.m.n_ax), P.rows / P.map_rows, (long long)P.V * P.map_rows)) return cudaErrorInvalidValue;
+    if (!ring_map(&map, P.ring, zherk_row_bytes(P.m.n_ax), P.rows / P.map_rows, (long long)P.V * P.map_rows, P.panel))
+        return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)n_ctas);
     const int nc = P.m.n_ax * P.m.n_feed;
@@ -1013,19 +1022,24 @@ cudaError_t launch_zherk_final(const ZherkFinalArgs& a, int form, cudaStream_t s
 }
 
 // ------------------------------------------------------------ host planning
-std::vector<ZherkTile> zherk_triangle(int rows) {
+int zherk_panel(int rows) {
+    const int np = (rows + 127) / 128;
+    return ((rows + np - 1) / np + 7) / 8 * 8;
+}
+
+std::vector<ZherkTile> zherk_triangle(int rows, int panel) {
     std::vector<ZherkTile> t;
-    for (int r = 0; r < rows; r += 128)
-        for (int k = 0; k <= r; k += 128) t.push_back(ZherkTile{r, k, r, k, 0, 0});
+    for (int r = 0; r < rows; r += panel)
+        for (int k = 0; k <= r; k += panel) t.push_back(ZherkTile{r, k, r, k, 0, 0});
     return t;
 }
 
-std::vector<ZherkTile> zherk_gauss_tiles(int N) {
+std::vector<ZherkTile> zherk_gauss_tiles(int N, int panel) {
     std::vector<ZherkTile> t;
-    for (int i = 0; i < N; i += 128)
-        for (int j = 0; j < N; j += 128) t.push_back(ZherkTile{i, N + j, i, j, 0, 0});
-    for (int i = 0; i < N; i += 128)
-        for (int j = 0; j <= i; j += 128) t.push_back(ZherkTile{2 * N + i, 2 * N + j, i, j, 1, 0});
+    for (int i = 0; i < N; i += panel)
+        for (int j = 0; j < N; j += panel) t.push_back(ZherkTile{i, N + j, i, j, 0, 0});
+    for (int i = 0; i < N; i += panel)
+        for (int j = 0; j <= i; j += panel) t.push_back(ZherkTile{2 * N + i, 2 * N + j, i, j, 1, 0});
     return t;
 }
 
@@ -1036,7 +1050,7 @@ namespace {
 // depth-first walk every vertex pairs the edges it has not handed on and gives
 // an odd one the edge to its parent, so at most one product per connected
 // component stays alone.
-void make_jobs(std::vector<ZherkTile>& tiles, int plane_rows, std::vector<ZherkJob>& out) {
+void make_jobs(std::vector<ZherkTile>& tiles, int plane_rows, int panel, std::vector<ZherkJob>& out) {
     std::vector<int> rows;  // vertices: first rows of panels
     auto vertex = [&](int row) {
         for (size_t i = 0; i < rows.size(); ++i)
@@ -1076,11 +1090,13 @@ void make_jobs(std::vector<ZherkTile>& tiles, int plane_rows, std::vector<ZherkJ
         const int b0 = other(e0), b1 = e1 >= 0 ? other(e1) : -1;
         J.b = box(rows[b0]);
         J.tile[0] = e0;
-        J.n = 128;
+        J.np = 1;
+        J.n = (panel + 15) / 16 * 16;
         if (b1 >= 0) {
             box(rows[b1]);
             J.tile[1] = e1;
-            J.n = 256;
+            J.np = 2;
+            J.n = 2 * panel;
         }
         J.a = b0 == at ? 0 : b1 == at ? 1 : box(rows[at]);
         out.push_back(J);
@@ -1128,14 +1144,16 @@ bool zherk_plan(int N, const std::vector<ZherkTile>& cover, int n_ax, int n_inst
         z.n_ax = n_ax;
         if (form == kZherkReal) {
             z.rows = 2 * N;
-            z.tiles = cover.empty() ? zherk_triangle(z.rows) : cover;
+            z.panel = cover.empty() ? zherk_panel(z.rows) : 128;
+            z.tiles = cover.empty() ? zherk_triangle(z.rows, z.panel) : cover;
         } else {
             z.rows = 3 * N;
-            z.tiles = zherk_gauss_tiles(N);
+            z.panel = zherk_panel(N);
+            z.tiles = zherk_gauss_tiles(N, z.panel);
         }
         if ((int)z.tiles.size() > 2 * n_sms) continue;
         std::vector<ZherkJob> one;  // the jobs of one instance
-        make_jobs(z.tiles, form == kZherkReal ? z.rows : N, one);
+        make_jobs(z.tiles, form == kZherkReal ? z.rows : N, z.panel, one);
         const int nj = (int)one.size(), T = (int)z.tiles.size();
         const int vcap = (int)std::min<long long>(n_sms / nj, ring_budget / ((long long)zherk_row_bytes(n_ax) * z.rows));
         if (vcap < 1) continue;
@@ -1144,7 +1162,7 @@ bool zherk_plan(int N, const std::vector<ZherkTile>& cover, int n_ax, int n_inst
             if (waves > kZherkMaxWaves) continue;
             // us: a chunk of a job (its MMAs at about 80 % of the tensor rate; the Z build
             // where a wave has few products), a wave's ramp, and the partial tiles written and read once
-            const double t = waves * (chunks / S * n_ax * 0.95 + 6.0) + total * (double)T * 131072.0 / 4e6;
+            const double t = waves * (chunks / S * n_ax * (0.35 + 0.6 * z.panel / 128.0) + 6.0) + total * (double)T * 131072.0 / 4e6;
             if (t < best) {
                 best = t;
                 out = z;
