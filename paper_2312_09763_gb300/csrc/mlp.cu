@@ -145,12 +145,14 @@ __global__ void k_weight_copies(LayerTab t, const float* __restrict__ p, int H, 
 
 // Weight and bias gradients from the k-split partial products, summed in a
 // fixed order (deterministic).
-// Weight gradient (o, i) of layer l from its k-split partials.
-__device__ __forceinline__ float layer_grad(const LayerTab& t, int l, const float* __restrict__ part, int splits, int o,
-                                            int i) {
+// Weight gradient q (row-major) of layer l from its k-split partials: the loads of
+// eight splits go out together.
+__device__ __forceinline__ float layer_grad(const LayerTab& t, int l, const float* __restrict__ part, int splits, int q) {
     float sum = 0.f;
-    const float* P = part + t.part_off[l] + (long long)o * t.kin[l] + i;
-    for (int s = 0; s < splits; ++s) sum += P[s * t.part_stride[l]];
+    const float* P = part + t.part_off[l] + q;
+    const long long stride = t.part_stride[l];
+#pragma unroll 8
+    for (int s = 0; s < splits; ++s) sum += P[s * stride];
     return sum;
 }
 
@@ -171,10 +173,7 @@ __global__ void k_reduce_grads(LayerTab t, const float* __restrict__ part, int s
     const int kin = t.kin[l], nout = t.nout[l];
     const long long n = (long long)nout * kin;
     const long long q0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
-    for (long long q = q0; q < n; q += step) {
-        const int o = (int)(q / kin), i = (int)(q % kin);
-        g[t.off_w[l] + q] = layer_grad(t, l, part, splits, o, i);
-    }
+    for (long long q = q0; q < n; q += step) g[t.off_w[l] + q] = layer_grad(t, l, part, splits, (int)q);
     // biases: one warp each
     const int lane = threadIdx.x & 31;
     for (long long w = q0 >> 5; w < nout; w += step >> 5) {
@@ -201,45 +200,59 @@ __device__ __forceinline__ float adam_step(float* __restrict__ p, float* __restr
 // One optimiser step of training: the weight and bias gradients summed from
 // the k-split partials (fixed order), Adam on them and on the embedding
 // (whose gradient is in g), and every BF16 copy the products read (W, W^T,
-// the padded output layer).  blockIdx.y: layer, or t.n for the embedding.
-__global__ void k_reduce_adam(LayerTab t, const float* __restrict__ part, int splits, const float* __restrict__ bpart,
-                              int brows, const float* __restrict__ g, long long off_emb, long long n_emb,
-                              float* __restrict__ p, float* __restrict__ am, float* __restrict__ av,
-                              bf16* __restrict__ pb, int H, bf16* __restrict__ wout16, bf16* __restrict__ woutT,
-                              AdamArgs a) {
-    const int l = blockIdx.y;
-    const long long step = (long long)gridDim.x * blockDim.x;
-    const long long q0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// the padded output layer).  blockIdx.y: layer, or t.n for the embedding.  What
+// bounds it is latency: a block takes a 32 x 32 piece of a layer, one weight a
+// thread and 1024 threads, its loads all in flight at once, and writes W^T along
+// its rows through shared memory; the biases have blocks of their own (350 beams,
+// 16,384 samples: 84.4 us a step with the pieces of a layer, its biases and W^T column
+// by column in the same threads, 81.4 so, the fill of the next sums included).
+__global__ void __launch_bounds__(1024)
+k_reduce_adam(LayerTab t, const float* __restrict__ part, int splits, const float* __restrict__ bpart,
+              int brows, float* __restrict__ g, long long off_emb, long long n_emb,
+              float* __restrict__ p, float* __restrict__ am, float* __restrict__ av,
+              bf16* __restrict__ pb, int H, bf16* __restrict__ wout16, bf16* __restrict__ woutT,
+              AdamArgs a) {
+    __shared__ bf16 tile[32][34];
+    const int l = blockIdx.y, x = threadIdx.x & 31, y = threadIdx.x >> 5;
     if (l == t.n) {
-        for (long long q = q0; q < n_emb; q += step) {
+        for (long long q = (long long)blockIdx.x * 1024 + threadIdx.x; q < n_emb; q += (long long)gridDim.x * 1024) {
             const long long i = off_emb + q;
             pb[i] = __float2bfloat16(adam_step(p, am, av, i, g[i], a));
+            g[i] = 0.f;  // the next step's sums start here
         }
         return;
     }
     const bool out = l == t.n - 1;
     const int kin = t.kin[l], nout = t.nout[l];
-    const long long n = (long long)nout * kin;
-    const int lane = threadIdx.x & 31;
-    for (long long w = q0 >> 5; w < nout; w += step >> 5) {  // biases: one warp each
-        const float gb = bias_grad_warp(t, l, bpart, brows, (int)w, lane);
-        if (lane == 0) {
-            const long long ib = t.off_b[l] + w;
-            pb[ib] = __float2bfloat16(adam_step(p, am, av, ib, gb, a));
+    const int pi = (kin + 31) / 32, pieces = pi * ((nout + 31) / 32);
+    for (int b = blockIdx.x; b < pieces + (nout + 31) / 32; b += gridDim.x) {
+        if (b >= pieces) {  // 32 biases, one warp each
+            const int w = (b - pieces) * 32 + y;
+            if (w < nout) {
+                const float gb = bias_grad_warp(t, l, bpart, brows, w, x);
+                if (x == 0) {
+                    const long long ib = t.off_b[l] + w;
+                    pb[ib] = __float2bfloat16(adam_step(p, am, av, ib, gb, a));
+                }
+            }
+            continue;
         }
-    }
-    for (long long q = q0; q < n; q += step) {
-        const int o = (int)(q / kin), i = (int)(q % kin);
-        const float sum = layer_grad(t, l, part, splits, o, i);
-        const long long iw = t.off_w[l] + (long long)o * kin + i;
-        const bf16 w = __float2bfloat16(adam_step(p, am, av, iw, sum, a));
-        pb[iw] = w;
-        if (!out) {
-            t.wt[l][(long long)i * H + o] = w;
-        } else {
-            wout16[(long long)o * H + i] = w;
-            woutT[(long long)i * 64 + o] = w;
+        const int o0 = b / pi * 32, i0 = (b - b / pi * pi) * 32, o = o0 + y, i = i0 + x;
+        if (o < nout && i < kin) {
+            const float sum = layer_grad(t, l, part, splits, o * kin + i);
+            const long long iw = t.off_w[l] + (long long)o * kin + i;
+            const bf16 w = __float2bfloat16(adam_step(p, am, av, iw, sum, a));
+            pb[iw] = w;
+            if (out) wout16[(long long)o * H + i] = w;
+            tile[y][x] = w;
         }
+        __syncthreads();
+        const int ot = o0 + x, it = i0 + y;
+        if (ot < nout && it < kin) {
+            if (out) woutT[(long long)it * 64 + ot] = tile[x][y];
+            else t.wt[l][(long long)it * H + ot] = tile[x][y];
+        }
+        __syncthreads();
     }
 }
 
@@ -584,16 +597,17 @@ cudaError_t weight_grads(Surrogate* S, int rows, bool reduce, int sms, cudaStrea
 // One training pass over the `rows` samples in S->ant / az / za / nu / T; the
 // loss is accumulated into S->loss, which the caller zeroes.  Leaves the
 // gradients of the loss as k-split partials and the embedding gradient in
-// S->g, with `reduce` every gradient summed into S->g.  Where the network's
-// shape allows, the row-local part (features, forward, loss, input gradients,
-// embedding gradient) is one fused launch (mlp_chain_tc.cu); else it runs
-// kernel by kernel.  The weight gradients follow as products over the batch.
+// S->g (which starts from zero: emb_zeroed tells that it is), with `reduce` every
+// gradient summed into S->g.  Where the network's shape allows, the row-local part
+// (features, forward, loss, input gradients, embedding gradient) is one fused
+// launch (mlp_chain_tc.cu); else it runs kernel by kernel.  The weight gradients
+// follow as products over the batch.
 // The tensor-core launches take at most `sms` SMs.
-cudaError_t train_rows(Surrogate* S, int rows, bool reduce, int sms, cudaStream_t st, long long* L) {
+cudaError_t train_rows(Surrogate* S, int rows, bool reduce, bool emb_zeroed, int sms, cudaStream_t st, long long* L) {
     const Dims& d = S->d;
     const int D = d.depth, H = d.H;
     // the embedding gradient accumulates; the rest is written by the reduction
-    cudaError_t e = reduce ? cudaMemsetAsync(S->g, 0, sizeof(float) * (size_t)S->n_par, st)
+    cudaError_t e = emb_zeroed ? cudaSuccess : reduce ? cudaMemsetAsync(S->g, 0, sizeof(float) * (size_t)S->n_par, st)
                            : cudaMemsetAsync(S->g + S->off_emb, 0, sizeof(float) * (size_t)(S->n_par - S->off_emb), st);
     const long long kext = std::max(rows, 64);
     if (e == cudaSuccess && kext > rows) {
@@ -836,7 +850,7 @@ cudaError_t surrogate_grad(Surrogate* S, int n, const int* ant, const float* az,
     if (e == cudaSuccess) e = cudaMemcpyAsync(S->T, T, sizeof(float) * n * d.n_out, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(S->loss, 0, sizeof(double), st);
     if (e != cudaSuccess) return e;
-    e = train_rows(S, n, true, S->n_sms, st, &L);
+    e = train_rows(S, n, true, false, S->n_sms, st, &L);
     if (e == cudaSuccess) e = cudaMemcpyAsync(grads_host, S->g, sizeof(float) * S->n_par, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(loss, S->loss, sizeof(double), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = check_err(S, st);
@@ -965,7 +979,7 @@ cudaError_t surrogate_train(Surrogate* S, const Model& m, const float2* grid, do
         S->T = s_T[k];
         if (it == 0 || it == steps - 1) e = cudaMemsetAsync(S->loss, 0, sizeof(double), st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(st, S->ev_ready[k], 0);
-        if (e == cudaSuccess) e = train_rows(S, batch, false, sms, st, L);
+        if (e == cudaSuccess) e = train_rows(S, batch, false, it > 0, sms, st, L);
         if (e == cudaSuccess) e = cudaEventRecord(S->ev_free[k], st);  // set k read for the last time
         if (e != cudaSuccess) break;
         if (it == 0 || it == steps - 1) {
@@ -986,9 +1000,9 @@ cudaError_t surrogate_train(Surrogate* S, const Model& m, const float2* grid, do
         a.c1 = 1.f - powf(0.9f, (float)S->adam_k);
         a.c2 = 1.f - powf(0.999f, (float)S->adam_k);
         const long long n_emb = S->n_par - S->off_emb;
-        const long long max_layer = (long long)std::max(d.d0p, d.H) * (d.H + 1);
         const int splits = grad_splits(S, batch, sms);
-        k_reduce_adam<<<dim3(gridsz(std::max(max_layer, n_emb), 256), d.depth + 2), 256, 0, st>>>(
+        const int max_pieces = (std::max(d.d0p, d.H) + 31) / 32 * ((d.H + 31) / 32) + (d.H + 31) / 32;
+        k_reduce_adam<<<dim3(std::max((unsigned)max_pieces, gridsz(n_emb, 1024)), d.depth + 2), 1024, 0, st>>>(
             S->tab, S->part, splits, S->bpart, splits, S->g, S->off_emb, n_emb, S->p, S->am, S->av, S->pb, d.H,
             S->wout16, S->woutT, a);
         ++*L;
