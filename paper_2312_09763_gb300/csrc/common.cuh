@@ -138,8 +138,8 @@ __device__ __forceinline__ void put_wa(float2* row, long long s, float2 v) {
     p[0] = v.x;
     p[2] = v.y;
 }
-// WA[slot] = sqrt(I_s) A(s) for the live sources and zero for the rest of
-// the pitch; amax[slot] (zeroed by the caller) receives max |WA| over the
+// WA[slot] = sqrt(I_s) A(s) for the live sources and zero up to the next
+// multiple of 256; amax[slot] (zeroed by the caller) receives max |WA| over the
 // slot's components, as float bits.
 cudaError_t launch_wa(const Model& m, const float2* d_planes, const Chan* d_chan, const Inst* d_inst,
                       int inst0, int n_inst, LiveTables lt, float2* d_wa, long long wa_pitch,

@@ -2,6 +2,8 @@
 // rotation of the sources to East-North-Up with R(t) of eq. "rotation"
 // (Sec. 2.3), the horizon cut with stable stream compaction, and the beam
 // evaluation at the live sources (Sec. 2.4), fused with sqrt(I_s(nu)).
+#include <algorithm>
+
 #include "common.cuh"
 #include "zcore.cuh"
 
@@ -249,9 +251,6 @@ __device__ __forceinline__ float keys(float x) {
     return 0.f;
 }
 
-// WA[slot][b][p][k][s] = sqrt(I_s(nu)) * A^{pk}_b(az_s, za_s, nu) for the live
-// sources of each instance (Algorithm 2 step ii, with the flux weight of step iv),
-// in pairs of sources (common.cuh).
 // Max of |value| over a warp, folded into amax (non-negative floats order
 // like their bit patterns).
 __device__ __forceinline__ void fold_amax(float v, float* amax) {
@@ -259,104 +258,143 @@ __device__ __forceinline__ void fold_amax(float v, float* amax) {
     if ((threadIdx.x & 31) == 0 && v > 0.f) atomicMax(reinterpret_cast<int*>(amax), __float_as_int(v));
 }
 
-__device__ float wa_eval(const Model& m, const float2* __restrict__ planes, const Chan& ch, const Inst& in,
-                         LiveTables lt, int s, float2* __restrict__ out, long long wa_pitch);
+// What the beam evaluation of a live source keeps from one channel to the next.
+// T: taps per axis (4 cubic, 2 bilinear).
+template <int T>
+struct SourceBeam {
+    float sqrt_flux, half_alpha, za;
+    float4 M;
+    // stencil in za (pole-reflected, clamped) and az (periodic): weights, row offsets
+    // in a plane, columns (those of a row across the pole half a turn on)
+    float wa[T], sg[T];
+    int row[T], col[T];
+    unsigned across;  // bit r: row r lies across the pole
 
-__global__ void __launch_bounds__(128)
-k_wa(Model m, const float2* __restrict__ planes, const Chan* __restrict__ chan,
-     const Inst* __restrict__ inst, int inst0, LiveTables lt, float2* __restrict__ wa, long long wa_pitch,
-     float* __restrict__ amax) {
-    kernel_chain();
-    const int slot = blockIdx.y;
-    const Inst in = inst[inst0 + slot];
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nl = lt.n_live[in.t];
-    const int ncomp = m.n_beam * m.n_feed * m.n_ax;
-    float mx = 0.f;
-    float2* out = wa + (long long)slot * ncomp * wa_pitch;
-    if (s < nl) {
-        mx = wa_eval(m, planes, chan[in.c], in, lt, s, out, wa_pitch);
-    } else if (s < wa_pitch) {  // zeros past the live count: the Z build reads whole source pairs
-        for (int comp = 0; comp < ncomp; ++comp) put_wa(out + (long long)comp * wa_pitch, s, make_float2(0.f, 0.f));
+    __device__ __forceinline__ void load(const Model& m, const LiveTables& lt, int t, int s) {
+        const long long o = (long long)t * lt.pitch + s;
+        const int src = lt.idx[o];
+        const float2 azza = lt.azza[o];
+        za = azza.y;
+        half_alpha = m.half_alpha[src];
+        sqrt_flux = m.pol_m ? 1.f : m.sqrt_flux[src];
+        M = m.pol_m ? m.pol_m[src] : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (m.beam_kind == 1) return;
+        const float uz = azza.y / m.dza, ua = azza.x / m.daz;
+        const float fz = floorf(uz), fa = floorf(ua);
+        const float tz = uz - fz, ta = ua - fa;
+        const int z0 = (int)fz - (T == 4 ? 1 : 0), a0 = (int)fa - (T == 4 ? 1 : 0);
+        float wz[T];
+        if constexpr (T == 4) {
+            wz[0] = keys(tz + 1.f); wz[1] = keys(tz); wz[2] = keys(1.f - tz); wz[3] = keys(2.f - tz);
+            wa[0] = keys(ta + 1.f); wa[1] = keys(ta); wa[2] = keys(1.f - ta); wa[3] = keys(2.f - ta);
+        } else {
+            wz[0] = 1.f - tz; wz[1] = tz;
+            wa[0] = 1.f - ta; wa[1] = ta;
+        }
+        const float pole_sign = m.n_ax == 2 ? -1.f : 1.f;
+        across = 0u;
+#pragma unroll
+        for (int r = 0; r < T; ++r) {
+            int z = z0 + r;
+            float g = 1.f;
+            if (z < 0) {
+                z = -z;
+                across |= 1u << r;
+                g = pole_sign;
+            }
+            row[r] = min(z, m.n_za - 1) * m.n_az;
+            sg[r] = g * wz[r];
+            int c = (a0 + r) % m.n_az;
+            if (c < 0) c += m.n_az;
+            col[r] = c;
+        }
     }
-    fold_amax(mx, amax + slot);
-}
 
-// sqrt(I_s(nu)) A^{pk}_b(s) for every component of one live source; returns
-// the largest magnitude written.
-__device__ float wa_eval(const Model& m, const float2* __restrict__ planes, const Chan& ch, const Inst& in,
-                         LiveTables lt, int s, float2* __restrict__ out, long long wa_pitch) {
-    const long long o = (long long)in.t * lt.pitch + s;
-    const int src = lt.idx[o];
-    const float2 azza = lt.azza[o];
-    const float spec = expf(m.half_alpha[src] * ch.ln_ratio);
-    const float w = m.pol_m ? spec : m.sqrt_flux[src] * spec;
-    const float4 M = m.pol_m ? m.pol_m[src] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const int ncomp = m.n_beam * m.n_feed * m.n_ax;
-    if (m.beam_kind == 1) {
-        const float a = w * expf(-m.gauss_c * azza.y * azza.y);
-        put_wa(out, s, make_float2(a, 0.f));
-        return fabsf(a);
-    }
-    // stencil in za (pole-reflected, clamped) and az (periodic)
-    const bool cubic = m.interp == 0;
-    const int nt = cubic ? 4 : 2;
-    const float uz = azza.y / m.dza, ua = azza.x / m.daz;
-    const float fz = floorf(uz), fa = floorf(ua);
-    const float tz = uz - fz, ta = ua - fa;
-    const int z0 = (int)fz - (cubic ? 1 : 0), a0 = (int)fa - (cubic ? 1 : 0);
-    float wz[4], wa_[4];
-    if (cubic) {
-        wz[0] = keys(tz + 1.f); wz[1] = keys(tz); wz[2] = keys(1.f - tz); wz[3] = keys(2.f - tz);
-        wa_[0] = keys(ta + 1.f); wa_[1] = keys(ta); wa_[2] = keys(1.f - ta); wa_[3] = keys(2.f - ta);
-    } else {
-        wz[0] = 1.f - tz; wz[1] = tz; wz[2] = wz[3] = 0.f;
-        wa_[0] = 1.f - ta; wa_[1] = ta; wa_[2] = wa_[3] = 0.f;
-    }
-    int rows[4], shifts[4];
-    float sg[4];
-    const float pole_sign = m.n_ax == 2 ? -1.f : 1.f;
-    for (int r = 0; r < nt; ++r) {
-        int row = z0 + r, sh = 0;
-        float g = 1.f;
-        if (row < 0) { row = -row; sh = m.n_az / 2; g = pole_sign; }
-        if (row > m.n_za - 1) row = m.n_za - 1;
-        rows[r] = row; shifts[r] = sh; sg[r] = g * wz[r];
-    }
-    const long long plane = (long long)m.n_za * m.n_az;
-    float mx = 0.f;
-    float2 a_prev = make_float2(0.f, 0.f);
-    for (int comp = 0; comp < ncomp; ++comp) {
-        const float2* P = planes + ((long long)in.c * ncomp + comp) * plane;
+    // One component of the beam from its plane P.
+    __device__ __forceinline__ float2 eval(const float2* __restrict__ P, int n_az) const {
         float re = 0.f, im = 0.f;
-        for (int r = 0; r < nt; ++r) {
-            const float2* rowp = P + (long long)rows[r] * m.n_az;
+#pragma unroll
+        for (int r = 0; r < T; ++r) {
+            const float2* rowp = P + row[r];
             float rr = 0.f, ri = 0.f;
-            for (int q = 0; q < nt; ++q) {
-                int col = (a0 + q + shifts[r]) % m.n_az;
-                if (col < 0) col += m.n_az;
-                const float2 v = rowp[col];
-                rr = fmaf(wa_[q], v.x, rr);
-                ri = fmaf(wa_[q], v.y, ri);
+#pragma unroll
+            for (int q = 0; q < T; ++q) {
+                int c = col[q];
+                if (across >> r & 1u) {
+                    c += n_az / 2;
+                    if (c >= n_az) c -= n_az;
+                }
+                const float2 v = rowp[c];
+                rr = fmaf(wa[q], v.x, rr);
+                ri = fmaf(wa[q], v.y, ri);
             }
             re = fmaf(sg[r], rr, re);
             im = fmaf(sg[r], ri, im);
         }
-        if (!m.pol_m) {
-            const float2 v = make_float2(w * re, w * im);
-            put_wa(out + (long long)comp * wa_pitch, s, v);
-            mx = fmaxf(mx, hypotf(v.x, v.y));
-        } else if ((comp & 1) == 0) {  // axis 0 of a (beam, feed): wait for axis 1
-            a_prev = make_float2(re, im);
-        } else {
-            float2 z0, z1;
-            apply_sky_sqrt(a_prev, make_float2(re, im), M, w, z0, z1);
-            put_wa(out + (long long)(comp - 1) * wa_pitch, s, z0);
-            put_wa(out + (long long)comp * wa_pitch, s, z1);
-            mx = fmaxf(mx, fmaxf(hypotf(z0.x, z0.y), hypotf(z1.x, z1.y)));
-        }
+        return make_float2(re, im);
     }
-    return mx;
+};
+
+// WA[slot][b][p][k][s] = sqrt(I_s(nu)) * A^{pk}_b(az_s, za_s, nu) for the live
+// sources of each instance (Algorithm 2 step ii, with the flux weight of step iv),
+// in pairs of sources (common.cuh), zero up to the next multiple of 256 (as far as
+// anything reads).  A thread takes `per` consecutive slots: their stencil, indices
+// and divisions are those of the first one while the time stays the same.  What
+// bounds it is the 16 scattered loads per channel: 350 antennas x 1e5 sources x 256
+// instances 490 us with one slot a thread and zeros to the end of the pitch, 425 with
+// four (438 with 16).
+template <int T>
+__global__ void __launch_bounds__(128, 6)
+k_wa(Model m, const float2* __restrict__ planes, const Chan* __restrict__ chan,
+     const Inst* __restrict__ inst, int inst0, int n_inst, int per, LiveTables lt, float2* __restrict__ wa,
+     long long wa_pitch, float* __restrict__ amax) {
+    kernel_chain();
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    const int ncomp = m.n_beam * m.n_feed * m.n_ax;
+    const long long plane = (long long)m.n_za * m.n_az;
+    SourceBeam<T> b;
+    int t = -1, nl = 0;
+    for (int slot = blockIdx.y * per; slot < min(n_inst, (int)(blockIdx.y + 1) * per); ++slot) {
+        const Inst in = inst[inst0 + slot];
+        if (in.t != t) {
+            t = in.t;
+            nl = lt.n_live[t];
+            if (s < nl) b.load(m, lt, t, s);
+        }
+        float mx = 0.f;
+        float2* out = wa + (long long)slot * ncomp * wa_pitch;
+        if (s < nl) {
+            const float spec = expf(b.half_alpha * chan[in.c].ln_ratio);
+            const float w = m.pol_m ? spec : b.sqrt_flux * spec;
+            if (m.beam_kind == 1) {
+                const float a = w * expf(-m.gauss_c * b.za * b.za);
+                put_wa(out, s, make_float2(a, 0.f));
+                mx = fabsf(a);
+            } else {
+                const float2* P = planes + (long long)in.c * ncomp * plane;
+                float2 a_prev = make_float2(0.f, 0.f);
+                for (int comp = 0; comp < ncomp; ++comp, P += plane) {
+                    const float2 a = b.eval(P, m.n_az);
+                    if (!m.pol_m) {
+                        const float2 v = make_float2(w * a.x, w * a.y);
+                        put_wa(out + (long long)comp * wa_pitch, s, v);
+                        mx = fmaxf(mx, hypotf(v.x, v.y));
+                    } else if ((comp & 1) == 0) {  // axis 0 of a (beam, feed): wait for axis 1
+                        a_prev = a;
+                    } else {
+                        float2 z0, z1;
+                        apply_sky_sqrt(a_prev, a, b.M, w, z0, z1);
+                        put_wa(out + (long long)(comp - 1) * wa_pitch, s, z0);
+                        put_wa(out + (long long)comp * wa_pitch, s, z1);
+                        mx = fmaxf(mx, fmaxf(hypotf(z0.x, z0.y), hypotf(z1.x, z1.y)));
+                    }
+                }
+            }
+        } else if (s < (nl + kKPad - 1) / kKPad * kKPad && s < wa_pitch) {
+            for (int comp = 0; comp < ncomp; ++comp) put_wa(out + (long long)comp * wa_pitch, s, make_float2(0.f, 0.f));
+        }
+        fold_amax(mx, amax + slot);
+    }
 }
 
 }  // namespace
@@ -389,9 +427,13 @@ cudaError_t launch_front(const FrontArgs& args, int n_times, LiveTables lt, cuda
 cudaError_t launch_wa(const Model& m, const float2* d_planes, const Chan* d_chan, const Inst* d_inst,
                       int inst0, int n_inst, LiveTables lt, float2* d_wa, long long wa_pitch, float* d_amax,
                       cudaStream_t st, long long* launches) {
-    dim3 grid((unsigned)((lt.pitch + 127) / 128), n_inst);
+    // slots per thread: as many as leave four blocks of 128 sources for every SM
+    const long long bx = (lt.pitch + 127) / 128;
+    const int per = (int)std::max(1ll, std::min<long long>(4, bx * n_inst / (4 * 152)));
+    const dim3 grid((unsigned)bx, (unsigned)((n_inst + per - 1) / per));
     *launches += 1;
-    return launch_chained(k_wa, grid, dim3(128), 0, st, m, d_planes, d_chan, d_inst, inst0, lt, d_wa, wa_pitch, d_amax);
+    return launch_chained(m.interp == 0 ? k_wa<4> : k_wa<2>, grid, dim3(128), 0, st, m, d_planes, d_chan, d_inst, inst0,
+                          n_inst, per, lt, d_wa, wa_pitch, d_amax);
 }
 
 }  // namespace mv
