@@ -113,8 +113,8 @@ typedef struct {
     int split;           /* source-axis split */
     int flush_kblocks;   /* 64-source k-blocks per TMEM flush */
     int candidates;      /* configurations timed */
-    double herk_ms;      /* best time of one batch: the HERK launch (with the next batch's Z build when
-                            fused), or the HERK and the batch's own Z-side launches */
+    double herk_ms;      /* best time of one batch: the HERK launch and the Z-side launches (beam, phase
+                            table, Z build) that run beside it */
     int fused;           /* 1: the launch that computes V also builds Z (streamed through L2, with
                             128-column tiles, or the next batch's Z planes);
                             0: every batch's Z build runs as its own launches */

@@ -1387,19 +1387,26 @@ mv_status autotune(mv_ctx* c, Plan& P, mv_precision prec, cudaStream_t st, mv_tu
     }
     cudaEvent_t e0 = ev_get(c), e1 = ev_get(c);
     const int reps = 2;
-    // the separate schedule's Z side of one batch (beam, phase table, Z build)
-    double zside_ms = 0;
-    if (p.fuse) {
-        if ((s = enqueue_zside(c, p, b0, 1, st, &L))) return s;  // warm-up
+    // the separate schedule's Z side of one batch (beam, phase table, Z build), and the
+    // beam alone
+    double zside_ms = 0, beam_ms = 0;
+    for (double* out : {&zside_ms, &beam_ms}) {
+        const int k = p.fuse ? 1 : 0;
+        auto side = [&]() { return out == &beam_ms ? enqueue_wa(c, p, b0, k, st, &L) : enqueue_zside(c, p, b0, k, st, &L); };
+        if ((s = side())) return s;  // warm-up
         cudaEventRecord(e0, st);
         for (int r = 0; r < reps; ++r)
-            if ((s = enqueue_zside(c, p, b0, 1, st, &L))) return s;
+            if ((s = side())) return s;
         cudaEventRecord(e1, st);
         if ((s = cuda_check(cudaEventSynchronize(e1), "trial timing"))) return s;
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
-        zside_ms = ms / reps;
+        *out = ms / reps;
     }
+    // what a batch of the fused schedule takes beside its launch: the first batch's Z side
+    // runs alone, the other ones' beam evaluation as well unless it runs ahead
+    const double n_b = (double)P.batches.size();
+    const double beside_fused = zside_ms / n_b + (p.ahead ? 0.0 : beam_ms * (n_b - 1) / n_b);
     HerkCfg best;
     bool best_fused = false;
     double best_ms = 1e300;
@@ -1414,7 +1421,7 @@ mv_status autotune(mv_ctx* c, Plan& P, mv_precision prec, cudaStream_t st, mv_tu
         if ((s = cuda_check(cudaEventSynchronize(e1), "trial timing"))) return s;
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
-        const double per_batch = ms / reps + (p.fuse && !fused_trial[i] ? zside_ms : 0.0);
+        const double per_batch = ms / reps + (fused_trial[i] ? beside_fused : zside_ms);
         if (per_batch < best_ms) {
             best_ms = per_batch;
             best = h;
@@ -1444,7 +1451,6 @@ mv_status autotune(mv_ctx* c, Plan& P, mv_precision prec, cudaStream_t st, mv_tu
                 cudaEventElapsedTime(&ms, e0, e1);
                 if (r > 0) sms = std::min(sms, (double)ms);
             }
-            // (a batch's beam evaluation is in every schedule's time here but the fused one's)
             const double per_batch = sms / (double)P2.inst.size() * b0.n;
             if (per_batch < best_ms) {
                 best_ms = per_batch;
