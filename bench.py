@@ -51,6 +51,10 @@ MLP_DRAM_BYTES_PER_LAUNCH = 53.68e6 + 499.97e6
 # read + 43.3 MB written for 16 instances, summarised in
 # profiles/k_herk_tc_redundant_cover_350ant_1e5src_16ch.txt.
 UNIQUE_DRAM_BYTES_PER_INSTANCE = (2.3149e9 + 0.0433e9) / 16
+# k_zherk on the same workload (19 instances: one wave of the streamed schedule):
+# 9.2 MB read + 1.2435 GB written (chunks of the ring that leave L2 before they are
+# overwritten), summarised in profiles/k_zherk_350ant_1e5src_19ch.txt.
+STREAM_DRAM_BYTES_PER_INSTANCE = (0.0092e9 + 1.2435e9) / 19
 METRIC = "vis/s (bl·chan·time) at 350 ant×1e5 src; split-prec TC vs FP32 @1e-5 rel err"
 UNIT = "vis/s"
 
@@ -212,6 +216,16 @@ class Clocks:
         return {"sm_mhz": statistics.median(busy) if busy else None,
                 "sm_max_mhz": max(smax) if smax else None,
                 "samples": len(sm), "reasons": sorted(reasons)}
+
+
+def streams(args, hk, tuning, w, pairs, launches):
+    """Whether the HERK launches of a step ran the streamed schedule: the default
+    without an option that asks for another one; mv_autotune may have timed
+    another one faster, which launches at least once per LST (or 64 pairs)."""
+    if hk or args.overlap or args.no_fuse or args.precision == "fp32":
+        return False
+    least = -(-n_instances(w, pairs) // 64) if pairs else len(w.lsts)
+    return tuning is None or least == 1 or launches < least
 
 
 def peaks():
@@ -453,16 +467,21 @@ def main():
         # with the fused Z build (the schedule the autotuner timed faster, or
         # the default for a forced 128-column tile) the timed HERK launches
         # also write the next batch's U planes
-        fused = not args.no_fuse and args.precision != "fp32" and nf == nax and \
+        # (the streamed schedule keeps Z in L2: no U planes in HBM)
+        streamed = streams(args, hk, tuning, w, pairs, n_h / args.steps)
+        fused = not streamed and not args.no_fuse and args.precision != "fp32" and nf == nax and \
             (bool(tuning.get("fused")) if tuning is not None else hk.get("herk_tile_n") == 128)
         traffic = None
         if args.workload == "hera" and not args.small and args.precision == "fp16x3" and tuning \
-                and tuning.get("tile_n") == 128:
-            per = FUSED_DRAM_BYTES_PER_INSTANCE if fused else HERK_DRAM_BYTES_PER_INSTANCE
+                and tuning.get("tile_n") == 128 and n_unique is None:
+            per = (STREAM_DRAM_BYTES_PER_INSTANCE if streamed else FUSED_DRAM_BYTES_PER_INSTANCE if fused
+                   else HERK_DRAM_BYTES_PER_INSTANCE)
             traffic = per * n_instances(w, pairs) / max(n_h / args.steps, 1)
         roof = {"bound": "tensor", "achieved": achieved, "peak": sustained, "unit": "TFLOP/s",
                 "frac": achieved / sustained, "traffic": traffic, "traffic_unit": "B per launch",
-                "kernel": "k_herk_tc" + (" (fused with the next batch's Z build)" if fused else ""),
+                "kernel": "k_zherk (Z built into a ring in L2 and expanded, with its preparation and the sum of "
+                          "its partial tiles)" if streamed else
+                          "k_herk_tc" + (" (fused with the next batch's Z build)" if fused else ""),
                 "launches": n_h, "avg_launch_ms": ms_h / max(n_h, 1),
                 "peak_source": f"{src} bf16 sustained (kernel timed inside a long step)"}
         if fused:
@@ -514,11 +533,15 @@ def main():
         traffic = None
         if args.workload == "hera" and not args.small and args.precision == "fp16x3":
             traffic = UNIQUE_DRAM_BYTES_PER_INSTANCE * n_instances(w, pairs) / n_launch
-        roof.update({"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
-                     "traffic": traffic, "kernel": "k_herk_tc over the redundant-group cover",
-                     "peak_source": f"{src} HBM copy rate",
-                     "algorithmic_bytes_per_launch": u_bytes / n_launch,
-                     "tensor_achieved_tflops": tflops, "tensor_frac": tflops / sustained})
+        if streamed:  # Z stays in L2: the sub-matrix products against the tensor rate
+            roof.update({"achieved": tflops, "frac": tflops / sustained, "traffic": None,
+                         "kernel": "k_zherk over the redundant-group cover"})
+        else:
+            roof.update({"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
+                         "traffic": traffic, "kernel": "k_herk_tc over the redundant-group cover",
+                         "peak_source": f"{src} HBM copy rate",
+                         "algorithmic_bytes_per_launch": u_bytes / n_launch,
+                         "tensor_achieved_tflops": tflops, "tensor_frac": tflops / sustained})
         for k in ("hbm_bytes_per_step", "hbm_achieved_gbs", "hbm_frac", "hbm_peak_gbs"):
             roof.pop(k, None)
         unique_info = {"n_unique": n_unique, "cover_kind": plan["kind"], "cover_blocks": plan["blocks"].tolist(),
@@ -558,7 +581,8 @@ def main():
             "scaling": "weak", "vs_baseline": None, "dtype": args.precision, "data": "synthetic",
             "config": {"workload": w.name, "instances_per_step": n_instances(w, pairs),
                        "live_sources_mean": float(live.mean()), "precision": args.precision,
-                       "l2": "inputs larger than L2: Z planes of one batch ~4.5 GB, re-streamed each step",
+                       "l2": "inputs larger than L2: beam and weight tables and V of a step, several GB written and read "
+                             "each step",
                        "parallelism": f"{world} replica(s), instances simulated independently"},
             "gpu_launches": launches, "roofline": roof, "clocks": clk, "herk_tuning": tuning, "learned_beam": learned,
             "redundant_groups": unique_info,

@@ -10,8 +10,9 @@ namespace mv {
 constexpr int kZherkChunk = 64;      // sources per ring chunk
 // Chunks in the ring, and bytes of a ring row.  Fewer chunks leave too little
 // between the oldest chunk still being read and the newest ones being built (350
-// antennas, one axis: 3.51 ms for 56 instances with 9 chunks, 3.39 with 11 or 13);
-// more outgrow the L2 (3.66 ms with 17: 87 MB).
+// antennas, one axis: 3.34 ms for 56 instances with 10 chunks, 3.28 with 11, 3.25
+// with 13; the redundant cover 6.18, 5.94, 5.62); more outgrow the L2 (3.30 with 14,
+// 3.52 with 16: 101 MB).
 __host__ __device__ constexpr int zherk_ring_chunks(int n_ax) { return n_ax == 1 ? 13 : 9; }
 __host__ __device__ constexpr int zherk_row_bytes(int n_ax) { return zherk_ring_chunks(n_ax) * kZherkChunk * 4 * n_ax; }
 constexpr int kZherkMaxWaves = 2048;

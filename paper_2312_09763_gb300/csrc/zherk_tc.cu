@@ -5,11 +5,11 @@
 //
 // Why: the 350-antenna x 1e5-source instance's U is 140 MB.  Built by a launch
 // of its own (or inside the HERK of the batch before) it goes to HBM and comes
-// back, 280 MB per instance.  Here every SM owns one 128 x 256 product of some
-// instance for the whole source axis, so Z is needed only in source order, by
-// all products at about the same time: a ring of several hundred sources per
-// instance (62 MB in all there, inside the 129 MB L2) is enough, and Z never
-// reaches HBM (ncu: 0.3 % of the DRAM rate).
+// back, 280 MB per instance.  Here every SM owns one product of up to 128 x 256
+// of some instance for the whole source axis, so Z is needed only in source order,
+// by all products at about the same time: a ring of several hundred sources per
+// instance (82 MB in all there, inside the 129 MB L2) is enough, and Z is never
+// read back from HBM (ncu: 1.2 of its 4.0 GB leave L2 before they are overwritten).
 //
 // A wave is V virtual instances (an instance, or one of S ranges of its
 // sources) whose products fill the SMs.  The ring is cut into chunks of 64
@@ -28,16 +28,18 @@
 // directions and WA into shared memory for the Z warps and watches the ring,
 // and 12 (8 with several components) warps build Z.
 //
-// What bounds it (350 antennas x 1e5 sources, 19 instances a wave): shared
-// memory.  A 64-source chunk costs an SM 128 KB of MMA operand reads, 80 KB of
-// TMA writes, 34 KB of Z stores and 22 KB of WA reads, about 2100 of its 2700
-// cycles at 128 bytes a cycle; the MMAs alone would take 1536, the Z build alone
-// (no loads, no MMAs) 1800.  56 instances take 3.39 ms against 4.79 with the Z
-// build fused into the HERK of the previous batch through HBM.
+// What bounds it (350 antennas x 1e5 sources, 19 instances a wave): L2 traffic.  A
+// 64-source chunk takes 1.38 us (56 instances 3.25 ms, against 4.79 with the Z build
+// fused into the HERK of the previous batch through HBM); in it the SMs read 12 MB
+// of panels and write 5.3 MB of Z, where L2 gives 17 TB/s to reads and 5.7 to
+// writes, and each SM moves 0.27 MB through its shared memory.  Without the Z stores
+// the 56 instances take 2.81 ms, without two of the three products 3.01; the MMAs
+// alone are 0.84 us a chunk, the Z build alone 0.94.  Single-channel groups are
+// bound by their phases (z_ants_one).
 //
 // Layout of a ring row: blocks of 32 columns, 128 bytes each, hi and lo halves of
-// 64 bytes (in turn, see the Z warps), so that one 128-byte-swizzled TMA box of
-// 128 rows brings both.
+// 64 bytes (in turn, see the Z warps), so that one 128-byte-swizzled TMA box of a
+// panel's rows brings both.
 #include <cuda.h>
 #include <cuda_fp16.h>
 
