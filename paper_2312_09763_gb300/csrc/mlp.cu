@@ -167,19 +167,22 @@ __device__ __forceinline__ float bias_grad_warp(const LayerTab& t, int l, const 
     return sum;
 }
 
+// One weight a thread, and blocks of their own for the biases, a warp each: the
+// kernel is bound by the latency of its loads (a gradient of 16,384 samples: 201 us
+// with four weights a thread and the biases after them, 195 so).
 __global__ void k_reduce_grads(LayerTab t, const float* __restrict__ part, int splits, const float* __restrict__ bpart,
                                int brows, float* __restrict__ g) {
     const int l = blockIdx.y;
-    const int kin = t.kin[l], nout = t.nout[l];
-    const long long n = (long long)nout * kin;
-    const long long q0 = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
-    for (long long q = q0; q < n; q += step) g[t.off_w[l] + q] = layer_grad(t, l, part, splits, (int)q);
-    // biases: one warp each
-    const int lane = threadIdx.x & 31;
-    for (long long w = q0 >> 5; w < nout; w += step >> 5) {
-        const float b = bias_grad_warp(t, l, bpart, brows, (int)w, lane);
-        if (lane == 0) g[t.off_b[l] + w] = b;
+    const int n = t.nout[l] * t.kin[l], blocks = (n + 255) / 256;
+    if ((int)blockIdx.x < blocks) {
+        const int q = blockIdx.x * 256 + threadIdx.x;
+        if (q < n) g[t.off_w[l] + q] = layer_grad(t, l, part, splits, q);
+        return;
     }
+    const int o = ((int)blockIdx.x - blocks) * 8 + (threadIdx.x >> 5);
+    if (o >= t.nout[l]) return;
+    const float b = bias_grad_warp(t, l, bpart, brows, o, threadIdx.x & 31);
+    if ((threadIdx.x & 31) == 0) g[t.off_b[l] + o] = b;
 }
 
 struct AdamArgs {
@@ -587,7 +590,10 @@ cudaError_t weight_grads(Surrogate* S, int rows, bool reduce, int sms, cudaStrea
         }
     }
     if (e == cudaSuccess && reduce) {
-        k_reduce_grads<<<dim3(64, D + 1), 256, 0, st>>>(S->tab, S->part, splits, S->bpart, splits, S->g);
+        unsigned blocks = 0;
+        for (int l = 0; l <= D; ++l)
+            blocks = std::max(blocks, gridsz((long long)S->tab.nout[l] * S->tab.kin[l], 256) + gridsz(S->tab.nout[l], 8));
+        k_reduce_grads<<<dim3(blocks, D + 1), 256, 0, st>>>(S->tab, S->part, splits, S->bpart, splits, S->g);
         ++*L;
         e = cudaGetLastError();
     }
