@@ -39,10 +39,12 @@ struct Chan {
 // Live-source tables of the distinct times of a call (structure of arrays,
 // one row of pitch `pitch` per time).
 struct LiveTables {
-    double* e;        // [n_times][pitch] East component of s_hat
-    double* n;        // North
-    double* u;        // Up
-    // s_hat in fixed point for the phase (NULL: not written): component c of
+    // one of the two forms of s_hat is written:
+    // FP64 East, North and Up, [n_times][pitch] each (NULL: fixed point)
+    double* e;
+    double* n;
+    double* u;
+    // in fixed point for the phase (where e is NULL): component c of
     // live source s at time t is sfix[(3 t + c) pitch + s] = S + 2^31 with
     // S = rint(s_c 2^31) (clamped to int32), and seps[...] = s_c - S 2^-31
     unsigned* sfix;
