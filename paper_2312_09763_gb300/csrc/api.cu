@@ -458,8 +458,10 @@ struct Prepared {
 };
 
 // Bytes the ring of Z may take: it has to stay in L2 (129 MB over two dies) beside
-// the WA tables in flight.
-constexpr long long kRingBytes = 96ll << 20;
+// the WA tables in flight.  Only arrays of about 128 antennas reach it (128 antennas x
+// 20,000 sources: 160 pairs 1170 us with 96 MB, 1091 with 112, 1084 with 120; 160
+// channels 780, 797, 804).
+constexpr long long kRingBytes = 112ll << 20;
 
 // Partial tiles of one FP32 HERK launch (at least one instance's).
 constexpr long long kPartialBytes = 1ll << 30;

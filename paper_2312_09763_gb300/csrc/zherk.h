@@ -10,10 +10,10 @@ namespace mv {
 constexpr int kZherkChunk = 64;      // sources per ring chunk
 // Chunks in the ring, and bytes of a ring row.  Fewer chunks leave too little
 // between the oldest chunk still being read and the newest ones being built (350
-// antennas, one axis: 3.34 ms for 56 instances with 10 chunks, 3.28 with 11, 3.25
-// with 13; the redundant cover 6.18, 5.94, 5.62); more outgrow the L2 (3.30 with 14,
-// 3.52 with 16: 101 MB).
-__host__ __device__ constexpr int zherk_ring_chunks(int n_ax) { return n_ax == 1 ? 13 : 9; }
+// antennas, one axis, 256 instances: 16.6 ms with 13 chunks, 16.2 with 14, 15.8 with
+// 15, 15.7 with 16: 82 MB; the redundant cover 6.09, 6.00, 5.88, 5.84); more outgrow
+// the L2 (15.9 and 5.90 with 17, 16.1 and 5.92 with 18).
+__host__ __device__ constexpr int zherk_ring_chunks(int n_ax) { return n_ax == 1 ? 16 : 9; }
 __host__ __device__ constexpr int zherk_row_bytes(int n_ax) { return zherk_ring_chunks(n_ax) * kZherkChunk * 4 * n_ax; }
 constexpr int kZherkMaxWaves = 2048;
 constexpr int kZherkChan = 20;       // channels x components a group may have

@@ -7,7 +7,7 @@
 // of its own (or inside the HERK of the batch before) it goes to HBM and comes
 // back, 280 MB per instance.  Here every SM owns one product of up to 128 x 256
 // of some instance for the whole source axis, so Z is needed only in source order,
-// by all products at about the same time: a ring of several hundred sources per
+// by all products at about the same time: a ring of a thousand sources per
 // instance (82 MB in all there, inside the 129 MB L2) is enough, and Z is never
 // read back from HBM (ncu: 1.2 of its 4.0 GB leave L2 before they are overwritten).
 //
@@ -18,13 +18,16 @@
 // A finished chunk is counted in ready[chunk]; an SM's TMA warp loads it for
 // the SM's own product once every SM of the team has counted it, and counts the
 // SM up in done[chunk] when the loads have landed, which frees the chunk's
-// place in the ring.  Everybody takes the chunks in the same order, so the
-// oldest one never waits for a newer one; the launch is cooperative (all CTAs
-// resident).  Every wait is bounded (tc.cuh).
+// place in the ring.  Both counts are released by the SM that counts itself up and
+// acquired by the warp that looks at them (once they are high enough: looking is
+// relaxed, as an acquire a look made hera 1 % slower), so that the loads come after
+// the stores they are to see, and the next stores after the loads.  Everybody takes the chunks
+// in the same order, so the oldest one never waits for a newer one; the launch is
+// cooperative (all CTAs resident).  Every wait is bounded (tc.cuh).
 //
 // Roles of a CTA (one per SM): warp 0 TMA, warp 1 MMA, warps 2-9 drain the
 // accumulator into FP32 running sums (both in TMEM) every `flush` stages,
-// COUNT_WARP publishes finished chunks, FEED_WARP copies each chunk's source
+// COUNT_WARP publishes finished and loaded chunks, FEED_WARP copies each chunk's source
 // directions and WA into shared memory for the Z warps and watches the ring,
 // and 12 (8 with several components) warps build Z.
 //
@@ -87,14 +90,27 @@ __device__ __forceinline__ int ld_relaxed(const int* p) {
     asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ int ld_acquire(const int* p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+// The same within the CTA, for a word in shared memory.
+__device__ __forceinline__ int ld_acquire_cta(uint32_t p) {
+    int v;
+    asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release_cta(uint32_t p, int v) {
+    asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(p), "r"(v) : "memory");
+}
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
     asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
     return p != 0;
 }
-__device__ __forceinline__ void red_release(int* p, int v) {
-    asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
+// What this thread has done and seen comes before the counts it adds next.
+__device__ __forceinline__ void fence_release() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 __device__ __forceinline__ void red_add(int* p, int v) {
     asm volatile("red.relaxed.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
@@ -409,7 +425,8 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
     uint64_t* bars = reinterpret_cast<uint64_t*>(zsm + 2 * Z_BUF + Z_WARPS * Z_APH_B);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 2 + 3 * MAX_BUF);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    volatile int* freed = reinterpret_cast<volatile int*>(tmem_slot + 2);  // chunks every SM has loaded, in a row
+    const uint32_t freed = smem_u32(tmem_slot + 2);   // chunks every SM has loaded, in a row
+    const uint32_t landed = smem_u32(tmem_slot + 3);  // chunks of this SM's jobs that have landed
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     auto full = [&](int s) { return smem_u32(&bars[s]); };
     auto empty = [&](int s) { return smem_u32(&bars[STAGES + s]); };
@@ -428,7 +445,7 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
         mbar_init(tempty, EPI_WARPS);
         for (int b = 0; b < MAX_BUF; ++b) { mbar_init(zfull(b), 1); mbar_init(zdone(b), Z_WARPS); mbar_init(zfree(b), 1); }
         *abort_flag = 0;
-        *freed = 0;
+        tmem_slot[2] = tmem_slot[3] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -514,23 +531,50 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
             }
         }
     } else if (warp == COUNT_WARP) {
-        // count this SM up for every chunk whose items its Z warps have finished (a
-        // release waits for the SM's stores to reach L2, which would hold up a Z warp)
-        int k = 0;
-        bool ok = true;
-        for (int w = 0; w < P.n_waves && ok; ++w) {
-            const ZShare z = z_share(P, w, Z_WARPS * P.ant_block);
-            if (z.team < 0) continue;
-            const int base = P.wave_base[w], wlen = P.wave_base[w + 1] - base;
-            for (int q = z.team; q < wlen; q += z.teams, ++k) {
-                if (!wait_bounded(zdone(k & zmask), zphase(k), abort_flag, P.err, kTimeoutNs, 100u)) ok = false;
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
+        // Count this SM up for every chunk whose items its Z warps have finished (ready)
+        // and for every chunk that has landed in it (done).  A warp of its own, as the
+        // fence before a count waits for the SM's stores to reach L2: that would hold up
+        // a Z warp, and in the TMA warp the loads (350 antennas, 1e5 sources, 256
+        // instances: 19.7 ms, 15.7 so).
+        int wb = -1, q = 0, base = 0, wlen = 0, k = 0;           // the next chunk built
+        int wl = -1, lq = 0, lbase = 0, llen = 0, counted = 0;   // the next chunk landed
+        ZShare z{1, -1, 0, 0};
+        unsigned long long t0 = gtimer();
+        for (;;) {
+            while (wb < P.n_waves && q >= wlen) {
+                if (++wb == P.n_waves) break;
+                z = z_share(P, wb, Z_WARPS * P.ant_block);
+                base = P.wave_base[wb];
+                wlen = z.team < 0 ? 0 : P.wave_base[wb + 1] - base;
+                q = z.team < 0 ? 0 : z.team;
+            }
+            while (wl < P.n_waves && lq >= llen) {
+                if (++wl == P.n_waves) break;
+                lbase = P.wave_base[wl];
+                llen = has_job(wl) ? P.zv[wl * P.V + J.v].w : 0;
+                lq = 0;
+            }
+            if (wb == P.n_waves && wl == P.n_waves) break;
+            const bool built = wb < P.n_waves && __all_sync(0xffffffffu, mbar_test(zdone(k & zmask), zphase(k)));
+            const int land = min(__shfl_sync(0xffffffffu, ld_acquire_cta(landed), 0) - counted, llen - lq);
+            if (built || land > 0) {
                 if (lane == 0) {
-                    mbar_arrive(zfree(k & zmask));  // (seen: the buffer's barrier may start its next phase)
-                    red_release(P.ready + base + q, 1);
+                    if (built) mbar_arrive(zfree(k & zmask));  // (seen: the buffer's barrier may start its next phase)
+                    fence_release();
+                    if (built) red_add(P.ready + base + q, 1);
+                    for (int i = 0; i < land; ++i) red_add(P.done + lbase + lq + i, 1);
                 }
                 __syncwarp();
+                if (built) {
+                    q += z.teams;
+                    ++k;
+                }
+                lq += land;
+                counted += land;
+                t0 = gtimer();
+            } else {
+                if (__any_sync(0xffffffffu, *abort_flag || gtimer() - t0 > 2 * kTimeoutNs)) break;
+                __nanosleep(20);
             }
         }
     } else if (warp == FEED_WARP) {
@@ -588,7 +632,9 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                 if (adv > 0) {
                     any = true;
                     next += adv;
-                    if (lane == 0) *freed = next;
+                    if (lane < adv) ld_acquire(P.done + c);
+                    __syncwarp();  // (what the lanes acquired comes before the release)
+                    if (lane == 0) st_release_cta(freed, next);
                 }
             }
             if (any) {
@@ -601,10 +647,10 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
     } else {
         if (warp == 0) {
             // The whole warp looks at the next 32 chunks' ready counts with one load, and one
-            // lane issues the copies.  While it waits it counts the chunks that have landed
-            // in this SM (done), ahead of their MMAs, so that their place in the ring is
-            // free about two chunks earlier.
-            int it = 0, landed = 0;  // stages issued, stages seen landed
+            // lane issues the copies.  While it waits it tells COUNT_WARP of the chunks that
+            // have landed in this SM, ahead of their MMAs, so that their place in the ring
+            // is free about two chunks earlier.
+            int it = 0, seen = 0, li = 0, chunks = 0;  // stages issued, stages seen landed, chunks of them
             bool ok = true;
             const int nbox = J.nbox, jv = J.v;
             for (int w = 0; w < P.n_waves && ok; ++w) {
@@ -612,7 +658,7 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                 const int len = P.zv[w * P.V + jv].w;
                 const int base = P.wave_base[w], wlen = P.wave_base[w + 1] - base;
                 const int items = P.wave_items[w] * ((P.m.n_ant + Z_WARPS * P.ant_block - 1) / (Z_WARPS * P.ant_block));
-                if (lane == 0)  // (chunks past this job's sources)
+                if (lane == 0)  // (chunks past this job's sources: never read, nothing to order)
                     for (int q = len; q < wlen; ++q) red_add(P.done + base + q, 1);
                 int y[MAX_BOX], pl[MAX_BOX];
 #pragma unroll
@@ -620,15 +666,15 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                     y[b] = jv * P.map_rows + J.row[b];
                     pl[b] = J.plane[b];
                 }
-                int lq = 0, li = 0;  // chunk of the wave and stage of it that lands next
                 auto land = [&]() {
-                    if (landed >= it) return false;
-                    if (!__all_sync(0xffffffffu, mbar_test(full(landed % STAGES), (uint32_t)(landed / STAGES) & 1u))) return false;
-                    ++landed;
+                    if (seen >= it) return false;
+                    if (!__all_sync(0xffffffffu, mbar_test(full(seen % STAGES), (uint32_t)(seen / STAGES) & 1u))) return false;
+                    ++seen;
                     if (++li == SPC) {
-                        if (lane == 0) red_add(P.done + base + lq, 1);
                         li = 0;
-                        ++lq;
+                        ++chunks;
+                        __syncwarp();
+                        if (lane == 0) st_release_cta(landed, chunks);
                     }
                     return true;
                 };
@@ -661,8 +707,10 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                             return have > q;
                         });
                         if (!ok) break;
-                        // the items' stores were released before they were counted; the
-                        // copies below read them from L2, never from this SM's L1
+                        // the items' stores were released before they were counted: the lanes
+                        // acquire the counts they saw, and the elected lane's copies follow
+                        if (q + lane < have) ld_acquire(P.ready + base + q + lane);
+                        __syncwarp();
                         asm volatile("fence.proxy.async.global;" ::: "memory");
                     }
                     const int x0 = ((base + q) % RC) * SPC * 64;
@@ -672,7 +720,7 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                         const uint32_t ph = ((uint32_t)(it / STAGES) & 1u) ^ 1u;
                         ok = wait_for([&]() { return __all_sync(0xffffffffu, mbar_test(empty(s), ph)) != 0; });
                         if (!ok) break;
-                        while (landed <= it - STAGES && land()) {}  // (the stage was consumed, so it has landed)
+                        while (seen <= it - STAGES && land()) {}  // (the stage was consumed, so it has landed)
                         if (elect_one()) {
                             mbar_expect_tx(full(s), (uint32_t)(nbox * box_b));
 #pragma unroll
@@ -683,7 +731,7 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                         ++it;
                     }
                 }
-                if (ok) ok = wait_for([&]() { return landed >= it; });
+                if (ok) ok = wait_for([&]() { return seen >= it; });
             }
         } else if (warp == 1) {
             // MMA: the whole warp walks the loop (so that descriptors and barriers stay
@@ -776,9 +824,10 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                     const int cq = base + q;
                     if (!wait_bounded(zfull(k & zmask), zphase(k), abort_flag, P.err)) ok = false;
                     // the chunk whose place in the ring this one takes has been read by all
-                    if (__shfl_sync(0xffffffffu, *freed, 0) <= cq - RC) {
+                    auto room = [&]() { return __all_sync(0xffffffffu, ld_acquire_cta(freed) > cq - RC) != 0; };
+                    if (!room()) {
                         const unsigned long long t0 = gtimer();
-                        while (__shfl_sync(0xffffffffu, *freed, 0) <= cq - RC) {
+                        while (!room()) {
                             __nanosleep(20);
                             const bool late = gtimer() - t0 > kTimeoutNs;
                             if (late && lane == 0) {
@@ -1270,16 +1319,16 @@ bool zherk_plan(int N, const std::vector<ZherkTile>& cover, int n_ax, int n_inst
 
 int zherk_ant_block(const ZherkPlan& z, int n_ant, int nc, int groups, int chan, int n_sms) {
     const int most = chan > 1 ? Z_BLOCK / 2 : Z_BLOCK;
-    const int ring_chunks = zherk_ring_chunks(z.n_ax);
+    const int most_teams = z.n_ax == 1 ? 6 : 4;
     int best = 0;
     double t_best = 1e300;
     for (int ab = 1; ab <= most; ++ab) {
         const int ants = z_warps(nc) * ab, teams = n_sms / (groups * ((n_ant + ants - 1) / ants));
         if (teams < 1) continue;
         // cycles per chunk: an item's fixed part and its antennas, over the chunks in
-        // flight, which have to leave the tensor side a few chunks of the ring
+        // flight, which have to leave the tensor side most of the ring
         double t = (800.0 + ab * (250.0 + 110.0 * chan)) / teams;
-        if (teams > ring_chunks / 2) t *= 1.0 + 0.5 * (teams - ring_chunks / 2);
+        if (teams > most_teams) t *= 1.0 + 0.5 * (teams - most_teams);
         if (t < t_best) {
             t_best = t;
             best = ab;
