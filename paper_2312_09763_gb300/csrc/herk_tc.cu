@@ -371,7 +371,7 @@ k_herk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
         int cg = 0;
         for (int n = 0;; ++n) {
             const int qi = n % QD;
-            if (!wait_bounded(qfull(qi), (uint32_t)(n / QD) & 1u, abort_flag, err)) break;
+            if (!wait_warp(qfull(qi), (uint32_t)(n / QD) & 1u, abort_flag, err)) break;
             const int u = qslot[qi];
             __syncwarp();
             if (lane == 0) mbar_arrive(qempty(qi));
@@ -430,7 +430,7 @@ k_herk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
                 for (int kc = w.kb0; kc < w.kb1; kc += flush, ++cg) {
                     const int buf = cg & 1;
                     const uint32_t ph = (uint32_t)(cg >> 1) & 1u;
-                    if (!wait_bounded(tfull(buf), ph, abort_flag, err)) { ok = false; break; }
+                    if (!wait_warp(tfull(buf), ph, abort_flag, err)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t ta = tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(buf * BN + h * 128);
 #pragma unroll
@@ -446,7 +446,7 @@ k_herk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tempty(buf));
                 }
-                if (!ok || *abort_flag) break;
+                if (!ok || warp_aborted(abort_flag)) break;
 #pragma unroll
                 for (int g = 0; g < 4; ++g)
                     if (g * 32 < ncv) write_chunk(std::integral_constant<int, 32>{}, g, run + g * 32);
@@ -459,7 +459,7 @@ k_herk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
                 for (int kc = w.kb0; kc < w.kb1; kc += flush, ++cg) {
                     const int buf = C::SB ? 0 : cg & 1;
                     const uint32_t ph = C::SB ? (uint32_t)cg & 1u : (uint32_t)(cg >> 1) & 1u;
-                    if (!wait_bounded(tfull(buf), ph, abort_flag, err)) { ok = false; break; }
+                    if (!wait_warp(tfull(buf), ph, abort_flag, err)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t ta = tl + (uint32_t)(buf * BN);
 #pragma unroll 1
@@ -483,7 +483,7 @@ k_herk_tc(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CU
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tempty(buf));
                 }
-                if (!ok || *abort_flag) break;
+                if (!ok || warp_aborted(abort_flag)) break;
 #pragma unroll 1
                 for (int g = 0; g < 8 && g * 16 < ncv; ++g) {
                     float x[16];

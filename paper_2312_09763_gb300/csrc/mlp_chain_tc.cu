@@ -407,8 +407,8 @@ k_mlp_chain(const __grid_constant__ Maps maps, const __grid_constant__ Job j, in
             }
             for (int s = 0; s < NS; ++s, ++g) {
                 const int buf = g & 1;
-                if (!wait_bounded(DFULL + 8u * buf, (uint32_t)(g >> 1) & 1u, abort_flag, err, kTimeoutNs, 1000u) ||
-                    !wait_bounded_spin(SDONE, (uint32_t)g & 1u, abort_flag, err)) {
+                if (!wait_warp(DFULL + 8u * buf, (uint32_t)(g >> 1) & 1u, abort_flag, err, kTimeoutNs, 1000u) ||
+                    !wait_warp_spin(SDONE, (uint32_t)g & 1u, abort_flag, err)) {
                     ok = false;
                     break;
                 }
@@ -502,7 +502,7 @@ k_mlp_chain(const __grid_constant__ Maps maps, const __grid_constant__ Job j, in
                     __syncwarp();
                     if (lane == 0) mbar_arrive(TEMPTY + 8u * buf);
                 }
-                if (*abort_flag) {
+                if (warp_aborted(abort_flag)) {
                     ok = false;
                     break;
                 }

@@ -467,7 +467,7 @@ k_mlp_wa(const __grid_constant__ Maps maps, const __grid_constant__ Net net, Mod
             };
             // ---- hidden layers 1 ..: accumulator -> bias, ReLU -> BF16 activations
             for (int l = 1; l < D; ++l) {
-                if (!wait_bounded_spin(my_dfull, (uint32_t)(nd++) & 1u, abort_flag, err)) { ok = false; break; }
+                if (!wait_warp_spin(my_dfull, (uint32_t)(nd++) & 1u, abort_flag, err)) { ok = false; break; }
                 tc_fence_after();
                 if (l == 1) gather();
                 drain_layer(trow, ab, r_loc, c_beg, half, sbias + l * 256);
@@ -479,7 +479,7 @@ k_mlp_wa(const __grid_constant__ Maps maps, const __grid_constant__ Net net, Mod
             if (!ok) break;
             // ---- output layer: accumulator -> registers, then the next tile's
             // h_1 (the accumulator columns are free again), then WA
-            if (!wait_bounded_spin(my_dfull, (uint32_t)(nd++) & 1u, abort_flag, err)) { ok = false; break; }
+            if (!wait_warp_spin(my_dfull, (uint32_t)(nd++) & 1u, abort_flag, err)) { ok = false; break; }
             tc_fence_after();
             if (D == 1) gather();
             float y[8];

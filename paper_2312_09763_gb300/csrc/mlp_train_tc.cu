@@ -260,7 +260,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
         for (int u = blockIdx.x; u < n_units; u += gridDim.x, ++cnt) {
             const UnitPos p = unit_pos(j, u);
             const int buf = buf_of(cnt);
-            if (!wait_bounded_spin(tfull(buf), phase_of(cnt), abort_flag, err)) break;
+            if (!wait_warp_spin(tfull(buf), phase_of(cnt), abort_flag, err)) break;
             tc_fence_after();
             const int m = p.m0 + half * TM + q4 * 32 + lane;
             const bool valid = m < j.M;
@@ -408,7 +408,7 @@ k_gemm_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUt
                 for (int off = 16; off > 0; off >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, off);
                 if (lane == 0 && lsum != 0.f) atomicAdd(e.loss, (double)lsum);
             }
-            if (*abort_flag) break;
+            if (warp_aborted(abort_flag)) break;
         }
     }
     __syncthreads();

@@ -182,7 +182,7 @@ k_wgrad(const __grid_constant__ Maps maps, const __grid_constant__ Job j, int* _
         for (int u = blockIdx.x; u < j.n_units; u += gridDim.x, ++cnt) {
             const Unit x = unit_at(j, u);
             const Prod& P = j.p[x.prod];
-            if (!wait_bounded_spin(TFULL, (uint32_t)cnt & 1u, abort_flag, err)) break;
+            if (!wait_warp_spin(TFULL, (uint32_t)cnt & 1u, abort_flag, err)) break;
             tc_fence_after();
             const int m = x.m0 + q * 32 + lane;
             const bool valid = m < P.M;
@@ -217,7 +217,7 @@ k_wgrad(const __grid_constant__ Maps maps, const __grid_constant__ Job j, int* _
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(TEMPTY);
-            if (*abort_flag) break;
+            if (warp_aborted(abort_flag)) break;
         }
     }
     __syncthreads();

@@ -104,6 +104,21 @@ __device__ __forceinline__ bool wait_bounded_spin(uint32_t bar, uint32_t parity,
         }
     }
 }
+// The same for a warp that goes on to instructions all its lanes have to reach
+// together (tcgen05.ld and .st, shuffles): one answer for the warp.  Each lane waits for
+// itself, so that without a vote one could give up where another has seen the phase
+// complete.
+template <class... A>
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, A... rest) {
+    return __all_sync(0xffffffffu, wait_bounded(bar, parity, abort_flag, err, rest...)) != 0;
+}
+__device__ __forceinline__ bool wait_warp_spin(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err) {
+    return __all_sync(0xffffffffu, wait_bounded_spin(bar, parity, abort_flag, err)) != 0;
+}
+// Whether any lane sees the abort flag raised.
+__device__ __forceinline__ bool warp_aborted(volatile int* abort_flag) {
+    return __any_sync(0xffffffffu, *abort_flag != 0) != 0;
+}
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),

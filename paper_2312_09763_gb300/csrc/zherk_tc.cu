@@ -476,7 +476,7 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
             const int4 v = P.zv[w * P.V + J.v];
             const int n_flush = (v.w * SPC + P.flush - 1) / P.flush;
             for (int f = 0; f < n_flush; ++f, ++cg) {
-                if (!wait_bounded(tfull, (uint32_t)cg & 1u, abort_flag, P.err, kTimeoutNs, 300u)) { ok = false; break; }
+                if (!wait_warp(tfull, (uint32_t)cg & 1u, abort_flag, P.err, kTimeoutNs, 300u)) { ok = false; break; }
                 tc_fence_after();
                 if (h * 128 < jn) {
                     // both loads of a piece go out together; the MMAs wait for this
@@ -504,7 +504,7 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                 __syncwarp();
                 if (lane == 0) mbar_arrive(tempty);
             }
-            if (!ok || *abort_flag) break;
+            if (!ok || warp_aborted(abort_flag)) break;
             if (h * 128 < jn) {
                 // partial tiles, column-major [128][128] (coalesced along rows); the second
                 // product's columns follow the first one's panel
@@ -751,12 +751,11 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
 #pragma unroll
                     for (int i = 0; i < SPC; ++i) {
                         if (ls == 0) {  // the epilogue has drained the accumulator
-                            if (!wait_bounded_spin(tempty, ((uint32_t)cg & 1u) ^ 1u, abort_flag, P.err)) ok = false;
+                            ok = wait_warp_spin(tempty, ((uint32_t)cg & 1u) ^ 1u, abort_flag, P.err);
                             tc_fence_after();
                         }
                         const int s = it % STAGES;
-                        if (ok && !wait_bounded(full(s), (uint32_t)(it / STAGES) & 1u, abort_flag, P.err)) ok = false;
-                        ok = __all_sync(0xffffffffu, ok);
+                        ok = ok && wait_warp(full(s), (uint32_t)(it / STAGES) & 1u, abort_flag, P.err);
                         if (!ok) break;
                         tc_fence_after();
                         const uint32_t so = (uint32_t)s * (STAGE >> 4);
@@ -822,7 +821,7 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                 __syncwarp();
                 for (int q = z.team; q < wlen; q += z.teams, ++k) {
                     const int cq = base + q;
-                    if (!wait_bounded(zfull(k & zmask), zphase(k), abort_flag, P.err)) ok = false;
+                    ok = wait_warp(zfull(k & zmask), zphase(k), abort_flag, P.err);
                     // the chunk whose place in the ring this one takes has been read by all
                     auto room = [&]() { return __all_sync(0xffffffffu, ld_acquire_cta(freed) > cq - RC) != 0; };
                     if (!room()) {
@@ -837,7 +836,6 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
                             if (__any_sync(0xffffffffu, *abort_flag || late)) { ok = false; break; }
                         }
                     }
-                    ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     if (q < g.len && a0 < a1) {
                         const uint8_t* sm = zsm + (k & zmask) * P.z_buf_b;

@@ -1,7 +1,10 @@
 """What cannot be provoked on a GPU without risking a fault or a hang, held in the
-kernels' sources (no GPU): the memory order of hand-overs between SMs."""
+kernels' sources (no GPU): the memory order of hand-overs between SMs, and that a
+warp which gives up a wait does so as a whole."""
 import os
 import re
+
+import pytest
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2312_09763_gb300", "csrc")
 
@@ -37,3 +40,32 @@ def test_ring_counts_are_released_and_acquired():
         assert len(re.findall(r"\b%s\b" % word, kernel)) == 3, word
         assert f"st_release_cta({word}" in kernel and f"ld_acquire_cta({word})" in kernel
     assert len(re.findall(r"P\.(?:ready|done)\b", kernel)) == 7
+
+
+@pytest.mark.parametrize("name", ["herk_tc.cu", "zherk_tc.cu", "mlp_tc.cu", "mlp_train_tc.cu", "mlp_chain_tc.cu",
+                                  "mlp_wgrad_tc.cu"])
+def test_warps_that_read_tensor_memory_give_up_together(name):
+    # tcgen05.ld needs the whole warp: a wait that ran out in one lane only, or an
+    # abort flag that one lane alone has seen, must not part the warp in front of it
+    s = source(name)
+    reads = [m.start() for m in re.finditer(r"\b(?:tmem_ld\d+|drain_layer)\(", s)]
+    waits = [(m.start(), m.group(1)) for m in re.finditer(r"\b(wait_\w+)\((?!uint32_t|auto)", s)]
+    waits = [w for w in waits if w[1].startswith(("wait_bounded", "wait_warp"))]
+    checked = 0
+    for r in reads:
+        before = [w for at, w in waits if at < r]
+        if not before:  # (a helper, defined above the kernel that waits)
+            continue
+        assert before[-1].startswith("wait_warp"), s[r - 200:r]
+        checked += 1
+    assert checked
+    assert not re.search(r"\*abort_flag\) (?:break|\{ ok = false)", s)
+
+
+def test_warp_waits_vote():
+    s = source("tc.cuh")
+    for name in ("wait_warp", "wait_warp_spin"):
+        body = s[s.index(f"bool {name}("):]
+        body = body[:body.index("}")]
+        assert re.search(r"return __all_sync\(0xffffffffu, wait_bounded\w*\(", body), name
+    assert re.search(r"bool warp_aborted\([^)]*\) \{ return __any_sync\(0xffffffffu, \*abort_flag != 0\)", s)
