@@ -97,7 +97,7 @@ struct mv_ctx {
     std::vector<ZherkTile> red_tiles;  // the 128-column tiles, and the limits of their blocks
     std::vector<int2> red_limits;
     // streamed Z build + HERK (zherk_tc.cu): the ring, and the tables of a call
-    Buf ring, ztab, zcount, zscale, zorder, zwave, zamax;
+    Buf ring, ztab, zcount, zscale, zorder, zwave;
     std::map<std::vector<long long>, ZherkPlan> zplans;  // by shape (bounded)
     // model buffers
     std::vector<double> h_flux;  // I at nu_ref (host copy, for the polarised sky's coherency)
@@ -796,8 +796,7 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
         if ((s = ensure(c, c->partial, part))) return s;
         if ((s = ensure(c, c->zwave, sizeof(int) * waves))) return s;
         if ((s = ensure(c, c->zcount, sizeof(int) * 2 * chunks))) return s;
-        if ((s = ensure(c, c->zscale, sizeof(float) * max_slots))) return s;
-        if ((s = ensure(c, c->zamax, sizeof(float) * max_slots))) return s;
+        if ((s = ensure(c, c->zscale, 2 * sizeof(float) * max_slots))) return s;
         if ((s = ensure(c, c->zorder, sizeof(int4) * vinsts))) return s;
     }
     const size_t plane_elems = (size_t)(p.zprec == 0 ? p.f32.rows : p.rows) * p.k_pitch * max_slots;
@@ -1032,7 +1031,7 @@ mv_status enqueue_stream(mv_ctx* c, const Prepared& p, size_t i, bool have_phase
     z.partial = (float*)c->partial.p;
     z.err = (int*)c->err.p;
     Timed th(c, MV_KERNEL_HERK, st);
-    cudaError_t e = launch_zherk_prep(z, (const float*)c->amax[0].p, (float*)c->zamax.p, (float*)c->zscale.p,
+    cudaError_t e = launch_zherk_prep(z, (const float*)c->amax[0].p, c->n_sms, (float*)c->zscale.p,
                                       (int4*)c->zorder.p, (int*)c->zwave.p, (ZherkGroup*)((uint8_t*)c->ztab.p + b.groups),
                                       b.n_groups, p.plan->pairs, 2 * b.max_chunks, st, L);
     if (e == cudaSuccess) e = launch_zherk(z, b.plan->form, c->n_sms, st, L);
@@ -1040,7 +1039,7 @@ mv_status enqueue_stream(mv_ctx* c, const Prepared& p, size_t i, bool have_phase
     f.inst = z.inst;
     f.inst0 = b.inst0;
     f.n_inst = b.n;
-    f.amax = (const float*)c->zamax.p;
+    f.scale = z.scale + b.n;
     f.partial = z.partial;
     f.tiles = (const ZherkTile*)(tab + b.tiles);
     f.tile_of = (const int*)(tab + b.tile_of);
@@ -1215,7 +1214,7 @@ std::vector<long long> graph_key(mv_ctx* c, const Plan& P, const Prepared& p, co
                          &c->wa[1], &c->amax[1], &c->u[1], &c->ulo[1], &c->wa[2], &c->amax[2], &c->partial,
                          &c->planes, &c->grid, &c->err,
                          &c->lsfix, &c->lseps, &c->aph[0], &c->aph[1], &c->pol_m, &c->red_uidx, &c->red_tl[0],
-                         &c->red_tl[1], &c->ring, &c->ztab, &c->zcount, &c->zscale, &c->zorder, &c->zwave, &c->zamax};
+                         &c->red_tl[1], &c->ring, &c->ztab, &c->zcount, &c->zscale, &c->zorder, &c->zwave};
     for (const Buf* b : bufs) k.push_back((long long)(uintptr_t)b->p);
     for (const void* d : {(const void*)c->d_R, (const void*)c->d_chan, (const void*)c->d_inst, (const void*)c->d_groups})
         k.push_back((long long)(uintptr_t)d);
@@ -1563,7 +1562,7 @@ void mv_destroy(mv_ctx* c) {
                   &c->planes, &c->wa[0], &c->amax[0], &c->u[0], &c->ulo[0],
                   &c->wa[1], &c->amax[1], &c->u[1], &c->ulo[1], &c->wa[2], &c->amax[2], &c->vdev, &c->err,
                   &c->partial, &c->sched, &c->lsfix, &c->lseps, &c->aph[0], &c->aph[1], &c->pol_m, &c->ring, &c->ztab,
-                  &c->zcount, &c->zscale, &c->zorder, &c->zwave, &c->zamax, &c->red_e, &c->red_n, &c->red_u, &c->red_b,
+                  &c->zcount, &c->zscale, &c->zorder, &c->zwave, &c->red_e, &c->red_n, &c->red_u, &c->red_b,
                   &c->red_uidx, &c->red_tl[0], &c->red_tl[1]};
     for (Buf* b : all) buf_free(c, *b);
     c->sky_stage.release();

@@ -71,7 +71,7 @@ struct ZherkArgs {
     LiveTables lt;
     const float2* wa;
     long long wa_pitch;
-    const float* scale;              // [n_inst] FP16 scale
+    const float* scale;              // [n_inst] FP16 scale of the Z build, then (V) [n_inst] in all
     const AntPhase* aph;
     int n_phase;
     const int4* zv;                  // virtual instances: slot, time, first source chunk, chunks
@@ -97,7 +97,7 @@ struct ZherkArgs {
 struct ZherkFinalArgs {
     const Inst* inst;
     int inst0, n_inst;
-    const float* amax;               // [n_inst] max |WA| behind the FP16 scale (NULL: no scale)
+    const float* scale;              // [n_inst] FP16 scale of WA in all, a power of two (NULL: none)
     const float* partial;
     const ZherkTile* tiles;
     const int* tile_of;              // gauss: [2][np][np] tile of F_ij and of H_ij (i >= j), np panels
@@ -130,7 +130,8 @@ int zherk_ant_block(const ZherkPlan& z, int n_ant, int nc, int groups, int chan,
 int zherk_input_bytes(int chan, int nc, int n_beam);
 int zherk_input_shift(int bytes);
 cudaError_t zherk_init();
-cudaError_t launch_zherk_prep(const ZherkArgs& P, const float* amax_in, float* amax_out, float* scale, int4* zv,
+// (multiplies WA of instances much weaker than others of their time; scale: 2 n_inst floats)
+cudaError_t launch_zherk_prep(const ZherkArgs& P, const float* amax, int n_sms, float* scale, int4* zv,
                               int* wave_base, ZherkGroup* groups, int n_groups, bool by_length, long long n_counters,
                               cudaStream_t st, long long* launches);
 cudaError_t launch_zherk(const ZherkArgs& P, int form, int n_ctas, cudaStream_t st, long long* launches);

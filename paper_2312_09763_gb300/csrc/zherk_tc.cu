@@ -879,16 +879,58 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
     }
 }
 
+// How the |WA| of an instance is brought into FP16's range: 2^all, from the largest
+// |WA| among the instances of its time (mx), which takes that to 2^13 .. 2^14, and
+// where that leaves the instance's own largest below 2^6 as many times 2^8 more as
+// take it to 2^6 .. 2^14, so that a rounding of FP16's smallest numbers (2^-25) stays
+// below 2^-31 of it.  2^all goes into the Z build's cosines and sines, where it costs
+// nothing and the channels of a group have to share it; 2^more into WA itself, as
+// channels of one beam seldom differ by 2^8 (in the Z build the redundant cover took
+// 4 % longer by it, unevenly spaced channels 4 to 7 %).
+__device__ __forceinline__ void fp16_exponents(float mx, float own, int& all, int& more) {
+    all = fp16_scale_exp(mx);
+    more = own > 0.f && own < 3.0e38f ? max(fp16_scale_exp(own) - all, 0) / 8 * 8 : 0;
+}
+
+// WA of an instance times 2^more: blocks 1 on of the launch below, `per` to an
+// instance.
+__device__ void rescale_wa(const ZherkArgs& P, const float* __restrict__ amax, int slot, int part, int per) {
+    __shared__ int mx;
+    if (threadIdx.x == 0) mx = 0;
+    __syncthreads();
+    const int t = P.inst[P.inst0 + slot].t;
+    for (int j = threadIdx.x; j < P.n_inst; j += blockDim.x) {
+        const float a = amax[j];
+        if (P.inst[P.inst0 + j].t == t && a > 0.f && a < 3.0e38f) atomicMax(&mx, __float_as_int(a));
+    }
+    __syncthreads();
+    int all, more;
+    fp16_exponents(__int_as_float(mx), amax[slot], all, more);
+    if (more == 0) return;
+    const float f = ldexpf(1.f, more / 2);  // (twice: 2^more itself may be no FP32 number)
+    const int rows = P.m.n_beam * P.m.n_feed * P.m.n_ax;
+    const int cols = (P.lt.n_live[t] + 1) / 2;  // source pairs
+    float4* w = reinterpret_cast<float4*>(const_cast<float2*>(P.wa) + (long long)slot * rows * P.wa_pitch);
+    for (int r = 0; r < rows; ++r, w += P.wa_pitch / 2)
+        for (int i = part * blockDim.x + threadIdx.x; i < cols; i += per * blockDim.x) {
+            const float4 v = w[i];
+            w[i] = make_float4(v.x * f * f, v.y * f * f, v.z * f * f, v.w * f * f);
+        }
+}
+
 // Per launch: the order of the instances (by_length: by decreasing live count),
-// the FP16 scale of every instance (one power of two for all instances of one
-// time, from the largest |WA| among them), the source range of every virtual
-// instance and group, and the chunk ranges of the waves.
-__global__ void __launch_bounds__(1024) k_zherk_prep(ZherkArgs P, const float* __restrict__ amax_in,
-                                                     float* __restrict__ amax_out, float* __restrict__ scale,
-                                                     int4* __restrict__ zv, int* __restrict__ wave_base,
+// the FP16 scale of every instance (that of the Z build, then that of V), the
+// source range of every virtual instance and group, and the chunk ranges of the
+// waves.
+__global__ void __launch_bounds__(1024) k_zherk_prep(ZherkArgs P, const float* __restrict__ amax, int per,
+                                                     float* __restrict__ scale, int4* __restrict__ zv, int* __restrict__ wave_base,
                                                      ZherkGroup* __restrict__ groups, int n_groups, int by_length,
                                                      long long n_counters) {
     kernel_chain();
+    if (blockIdx.x > 0) {
+        rescale_wa(P, amax, ((int)blockIdx.x - 1) / per, ((int)blockIdx.x - 1) % per, per);
+        return;
+    }
     for (long long i = threadIdx.x; i < n_counters; i += blockDim.x) P.ready[i] = 0;  // (ready, then done)
     extern __shared__ int sm[];  // t, live count and max |WA| of each instance, then the waves' lengths
     int *st = sm, *sk = sm + P.n_inst, *order = sm + 3 * P.n_inst, *len = sm + 4 * P.n_inst;
@@ -897,7 +939,7 @@ __global__ void __launch_bounds__(1024) k_zherk_prep(ZherkArgs P, const float* _
     for (int i = threadIdx.x; i < P.n_inst; i += blockDim.x) {
         st[i] = P.inst[P.inst0 + i].t;
         sk[i] = P.lt.n_live[st[i]];
-        sa[i] = amax_in[i];
+        sa[i] = amax[i];
     }
     __syncthreads();
     for (int i = threadIdx.x; i < P.n_inst; i += blockDim.x) {
@@ -906,12 +948,14 @@ __global__ void __launch_bounds__(1024) k_zherk_prep(ZherkArgs P, const float* _
         float mx = 0.f;
         for (int j = 0; j < P.n_inst; ++j) {
             rank += (sk[j] > ki) || (sk[j] == ki && j < i);
-            if (st[j] == ti) mx = fmaxf(mx, sa[j]);
+            if (st[j] == ti && sa[j] < 3.0e38f) mx = fmaxf(mx, sa[j]);
         }
         if (by_length) order[rank] = i;
         else order[i] = i;
-        amax_out[i] = mx;
-        scale[i] = ldexpf(1.f, fp16_scale_exp(mx));
+        int all, more;
+        fp16_exponents(mx, sa[i], all, more);
+        scale[i] = ldexpf(1.f, all);
+        scale[P.n_inst + i] = ldexpf(1.f, all + more);
     }
     __syncthreads();
     const int total = P.n_inst * P.S;
@@ -988,7 +1032,7 @@ __global__ void __launch_bounds__(256) k_zherk_final_real(ZherkFinalArgs a) {
         G[c][r + 3] = v.w;
     }
     __syncthreads();
-    const float us = a.amax ? ldexpf(1.f, -fp16_scale_exp(a.amax[slot])) : 1.f;
+    const float us = a.scale ? 1.f / a.scale[slot] : 1.f;
     float2* Vb = a.V + a.inst[a.inst0 + slot].v_off;
     auto entry = [&](int i, int j) {  // product entry (row, column) of the piece
         return t.trans ? G[i][j] : G[j][i];
@@ -1051,7 +1095,7 @@ __global__ void __launch_bounds__(256) k_zherk_final_gauss(ZherkFinalArgs a) {
         }
     }
     __syncthreads();
-    const float us = a.amax ? ldexpf(1.f, -fp16_scale_exp(a.amax[slot])) : 1.f;
+    const float us = a.scale ? 1.f / a.scale[slot] : 1.f;
     float2* Vb = a.V + a.inst[a.inst0 + slot].v_off;
     for (int pass = 0; pass < 2; ++pass)
         for (int k = threadIdx.x; k < 32 * 32; k += 256) {
@@ -1101,12 +1145,17 @@ cudaError_t zherk_init() {
     return e;
 }
 
-cudaError_t launch_zherk_prep(const ZherkArgs& P, const float* amax_in, float* amax_out, float* scale, int4* zv,
+cudaError_t launch_zherk_prep(const ZherkArgs& P, const float* amax, int n_sms, float* scale, int4* zv,
                               int* wave_base, ZherkGroup* groups, int n_groups, bool by_length, long long n_counters,
                               cudaStream_t st, long long* launches) {
     *launches += 1;
-    return launch_chained(k_zherk_prep, dim3(1), dim3(1024), sizeof(int) * (size_t)(P.n_waves + 4 * P.n_inst), st, P, amax_in,
-                          amax_out, scale, zv, wave_base, groups, n_groups, (int)by_length, n_counters);
+    // blocks for rescale_wa: one to 8192 source pairs of an instance as long as that is
+    // one an SM (one instance, or one of every time, is its time's largest: none)
+    const long long pairs = P.wa_pitch / 2 * P.m.n_beam * P.m.n_feed * P.m.n_ax;
+    const int per = (int)std::max(1ll, std::min<long long>((pairs + 8191) / 8192, n_sms / P.n_inst));
+    const unsigned blocks = P.n_inst == 1 || by_length ? 1u : 1u + (unsigned)(P.n_inst * per);
+    return launch_chained(k_zherk_prep, dim3(blocks), dim3(1024), sizeof(int) * (size_t)(P.n_waves + 4 * P.n_inst), st, P, amax,
+                          per, scale, zv, wave_base, groups, n_groups, (int)by_length, n_counters);
 }
 
 int zherk_input_bytes(int chan, int nc, int n_beam) { return Z_SRC_B + (n_beam == 1 ? chan * nc * kZherkChunk * 8 : 0); }
