@@ -47,14 +47,15 @@ __device__ __forceinline__ long long to_fixed(double v) {
 }
 
 // Whether source s is above the horizon at time t: the sign of rot_row, taken from
-// FP32 products (within 1e-6 of their magnitudes' sum) where that is clear of zero.
+// FP32 products (within 1e-6 of their magnitudes' sum) where that is clear of zero
+// and far from FP32's smallest numbers.
 __device__ __forceinline__ bool above(const Model& m, const double* __restrict__ R, int t, long long s) {
     if (s >= m.n_src) return false;
     const double* r = R + 9 * t + 6;
     const double x = m.xeq[s], y = m.xeq[m.n_src + s], z = m.xeq[2 * m.n_src + s];
     const float a = to_float(r[0]) * to_float(x), b = to_float(r[1]) * to_float(y), c = to_float(r[2]) * to_float(z);
     const float up = a + b + c, sum = fabsf(a) + fabsf(b) + fabsf(c);
-    return fabsf(up) > 4e-6f * sum ? up > 0.f : above_exact(r, x, y, z);
+    return fabsf(up) > 4e-6f * sum && sum > 1e-30f ? up > 0.f : above_exact(r, x, y, z);
 }
 
 // The live sources of block blk of time t: their count and, a bit each, which.
