@@ -2,6 +2,8 @@
 // behind it: argument validation, the per-call plan (distinct times and
 // channels, instance batches that share a time), workspace management, and
 // the launch sequence of Algorithm 2 (arXiv:2312.09763, Sec. 3.1).
+#include <cuda.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
@@ -482,6 +484,30 @@ size_t put_table(std::vector<uint8_t>& tab, const void* d, size_t bytes) {
     return at;
 }
 
+// SMs that work on `st` may take: all of them, but on a stream of a green context its
+// share.
+int stream_sms(cudaStream_t st, int all) {
+    auto entry = [](const char* name) {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion(name, &p, 12040, cudaEnableDefault, &q) != cudaSuccess) {
+            cudaGetLastError();
+            return (void*)nullptr;
+        }
+        return q == cudaDriverEntryPointSuccess ? p : nullptr;
+    };
+    using CtxOf = CUresult (*)(CUstream, CUgreenCtx*);
+    using ResourceOf = CUresult (*)(CUgreenCtx, CUdevResource*, CUdevResourceType);
+    static const CtxOf ctx_of = (CtxOf)entry("cuStreamGetGreenCtx");
+    static const ResourceOf resource_of = (ResourceOf)entry("cuGreenCtxGetDevResource");
+    CUgreenCtx g = nullptr;
+    CUdevResource r{};
+    if (!ctx_of || !resource_of || ctx_of((CUstream)st, &g) != CUDA_SUCCESS || !g ||
+        resource_of(g, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS)
+        return all;
+    return (int)r.sm.smCount;
+}
+
 // Plan the streamed schedule: batches of consecutive instances (whose WA tables
 // fit the budget), and for each the jobs, channel groups and Z items of its
 // waves in one table buffer.  Replaces the plan's groups and batches.  False
@@ -628,6 +654,12 @@ HerkCfg chosen_cfg(mv_ctx* c, const Prepared& p) {
     return heuristic_cfg(c, p);
 }
 
+// Whether a call on st may take every SM (its launches are captured on the context's
+// stream where graphs are on).
+bool all_sms(const mv_ctx* c, cudaStream_t st) {
+    return stream_sms(st, c->n_sms) >= c->n_sms && (st == c->stream || stream_sms(c->stream, c->n_sms) >= c->n_sms);
+}
+
 mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_device, cudaStream_t st, Prepared& out,
                   bool allow_stream = true, bool ignore_tuning = false) {
     Model& m = c->model;
@@ -707,12 +739,14 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
         p.ho.n_feed = m.n_feed;
     }
     // the streamed schedule unless an option asks for a particular HERK or
-    // Z-build schedule, or the autotuner timed another one faster for calls of
-    // this shape
+    // Z-build schedule, the autotuner timed another one faster for calls of
+    // this shape, or the call runs on a part of the SMs (the launch needs all of its
+    // blocks resident, one an SM)
     std::vector<uint8_t> ztab;
     const mv_options& o = c->opt;
     if (allow_stream && p.zprec != 0 && o.fuse_zbuild && !o.overlap_batches && o.herk_tile_n == 0 && o.herk_split == 0 &&
-        o.herk_flush_kblocks == 0 && (ignore_tuning || !(tuned_for(c, p) && !c->tuned.stream))) {
+        o.herk_flush_kblocks == 0 && (ignore_tuning || !(tuned_for(c, p) && !c->tuned.stream)) &&
+        all_sms(c, st)) {
         std::vector<ZGroup> groups = P.groups;
         std::vector<Plan::Batch> batches = P.batches;
         const int slots = p.max_slots;
