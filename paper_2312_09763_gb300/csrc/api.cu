@@ -377,33 +377,38 @@ ZGroup make_group(const Plan& P, int i0, int n, int slot0) {
     return g;
 }
 
-int auto_batch(mv_ctx* c, long long slot_bytes) {
-    if (c->opt.max_batch > 0) return std::min(c->opt.max_batch, kMaxBatch);
-    const long long budget = 20ll << 30;  // workspace for the Z planes
-    long long b = budget / std::max(slot_bytes, 1ll);
-    return (int)std::max(1ll, std::min(b, 64ll));
-}
+// Workspace of a batch: the Z planes and WA tables, with FP32 the partial tiles too.
+constexpr long long kBatchBytes = 20ll << 30;
+// Partial tiles of one FP32 HERK launch (at least one instance's), and those of a
+// streamed launch beyond one a product.
+constexpr long long kPartialBytes = 1ll << 30;
 
-// Workspace of one instance slot: the Z planes plus its beam x sqrt(I) table.
-long long slot_bytes_of(mv_ctx* c) {
+// Instances of a batch: as many as fit kBatchBytes, up to 64.
+int auto_batch(mv_ctx* c, mv_precision prec) {
+    if (c->opt.max_batch > 0) return std::min(c->opt.max_batch, kMaxBatch);
+    // one instance: the Z planes (FP16 hi and lo rows Re and Im of every antenna-feed, or
+    // FP32 rows, three with the gauss form) plus its beam x sqrt(I) table
     const Model& m = c->model;
     const long long N = (long long)m.n_feed * m.n_ant;
+    const bool fp32 = prec == MV_PREC_FP32;
     const long long src = std::max<long long>(m.n_src, 1);
     const long long ncomp = (long long)std::max(m.n_beam, 1) * std::max(m.n_feed, 1) * std::max(m.n_ax, 1);
-    return 4ll * 2 * N * round_up((long long)m.n_ax * src, kKPad) + 8ll * ncomp * round_up(src, kKPad);
+    const long long slot = 4ll * (fp32 ? 3 : 2) * N * round_up((long long)m.n_ax * src, kKPad) + 8ll * ncomp * round_up(src, kKPad);
+    const long long b = (kBatchBytes - (fp32 ? kPartialBytes : 0)) / std::max(slot, 1ll);
+    return (int)std::max(1ll, std::min(b, 64ll));
 }
 
 constexpr int kZGroup = 16;  // the fused Z build keeps a group's FP16 scales in 16 floats per warp
 static_assert(kZGroup <= 16, "Z groups of at most 16 instances");
 
 // Every (LST, channel) pair; batches are up to B channels of one LST.
-void plan_grid(mv_ctx* c, int n_t, const double* lst, int n_nu, const double* nu, Plan& P) {
+void plan_grid(mv_ctx* c, int n_t, const double* lst, int n_nu, const double* nu, mv_precision prec, Plan& P) {
     P.lst.assign(lst, lst + n_t);
     P.nu.assign(nu, nu + n_nu);
     const long long N = (long long)c->model.n_feed * c->model.n_ant;
     for (int t = 0; t < n_t; ++t)
         for (int f = 0; f < n_nu; ++f) P.inst.push_back(Inst{t, f, ((long long)t * n_nu + f) * N * N});
-    const int B = auto_batch(c, slot_bytes_of(c));
+    const int B = auto_batch(c, prec);
     for (int t = 0; t < n_t; ++t)
         for (int f0 = 0; f0 < n_nu; f0 += B) {
             const int n = std::min(B, n_nu - f0);
@@ -419,13 +424,13 @@ void plan_grid(mv_ctx* c, int n_t, const double* lst, int n_nu, const double* nu
 }
 
 // Explicit (LST, frequency) pairs; batches of up to B pairs, one group each.
-void plan_pairs(mv_ctx* c, int n_pairs, const double* lst, const double* nu, Plan& P) {
+void plan_pairs(mv_ctx* c, int n_pairs, const double* lst, const double* nu, mv_precision prec, Plan& P) {
     P.lst.assign(lst, lst + n_pairs);
     P.nu.assign(nu, nu + n_pairs);
     P.pairs = true;
     const long long N = (long long)c->model.n_feed * c->model.n_ant;
     for (int i = 0; i < n_pairs; ++i) P.inst.push_back(Inst{i, i, (long long)i * N * N});
-    const int B = auto_batch(c, slot_bytes_of(c));
+    const int B = auto_batch(c, prec);
     for (int i0 = 0; i0 < n_pairs; i0 += B) {
         const int n = std::min(B, n_pairs - i0);
         Plan::Batch b{i0, n, (int)P.groups.size(), n};
@@ -464,9 +469,6 @@ struct Prepared {
 // 20,000 sources: 160 pairs 1170 us with 96 MB, 1091 with 112, 1084 with 120; 160
 // channels 780, 797, 804).
 constexpr long long kRingBytes = 112ll << 20;
-
-// Partial tiles of one FP32 HERK launch (at least one instance's).
-constexpr long long kPartialBytes = 1ll << 30;
 
 // Where the product of panels (i, j) of F (kind 0) and H (kind 1) is in a gauss tile list.
 std::vector<int> gauss_tile_of(const std::vector<ZherkTile>& tiles, int np, int panel) {
@@ -527,7 +529,7 @@ bool plan_stream(mv_ctx* c, Plan& P, Prepared& p, std::vector<uint8_t>& tab) {
         auto it = c->zplans.find(key);
         if (it == c->zplans.end()) {
             ZherkPlan z;
-            if (!zherk_plan(p.N, cover, m.n_ax, n, 0.5 * (double)m.n_src, c->n_sms, kRingBytes, z)) z.V = 0;
+            if (!zherk_plan(p.N, cover, m.n_ax, n, 0.5 * (double)m.n_src, c->n_sms, kRingBytes, kPartialBytes, z)) z.V = 0;
             it = c->zplans.emplace(key, std::move(z)).first;
         }
         return it->second.V > 0 ? &it->second : nullptr;
@@ -762,7 +764,9 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
 
     mv_status s;
     if (p.zprec == 0) {
-        p.f32 = herk_fp32_plan(p.N, m.n_ax, max_slots, 0.5 * (double)m.n_src, c->n_sms);
+        // (the gauss form where its planes fit: a batch that the caller sized may be larger)
+        const bool gauss = 12ll * p.N * p.k_pitch * max_slots <= kBatchBytes;
+        p.f32 = herk_fp32_plan(p.N, m.n_ax, max_slots, 0.5 * (double)m.n_src, c->n_sms, gauss, kPartialBytes);
         const size_t slot = sizeof(float) * 128 * 128 * p.f32.tiles.size() * p.f32.split;
         p.f32_slots = (int)std::max(1ll, std::min<long long>(max_slots, kPartialBytes / (long long)slot));
         p.f32_tiles = put_table(ztab, p.f32.tiles.data(), p.f32.tiles.size() * sizeof(ZherkTile));
@@ -1910,7 +1914,7 @@ mv_status mv_simulate_unique(mv_ctx* c, int n_t, const double* lst, int n_nu, co
     if (!c->have_red) return fail(MV_ERR_STATE, "no redundancy plan (mv_set_redundancy)");
     DeviceGuard g(c->device);
     Plan P;
-    plan_grid(c, n_t, lst, n_nu, nu, P);
+    plan_grid(c, n_t, lst, n_nu, nu, prec, P);
     P.unique = true;
     const long long per = (long long)c->red.rep_a.size() * c->model.n_feed * c->model.n_feed;
     for (size_t i = 0; i < P.inst.size(); ++i) P.inst[i].v_off = (long long)i * per;
@@ -1961,7 +1965,7 @@ mv_status mv_simulate(mv_ctx* c, int n_t, const double* lst, int n_nu, const dou
     if (n_t < 0 || n_nu < 0 || (n_t > 0 && !lst) || (n_nu > 0 && !nu)) return fail(MV_ERR_ARG, "bad time/frequency lists");
     DeviceGuard g(c->device);
     Plan P;
-    plan_grid(c, n_t, lst, n_nu, nu, P);
+    plan_grid(c, n_t, lst, n_nu, nu, prec, P);
     cudaStream_t st = stream ? (cudaStream_t)stream : c->stream;
     return run(c, P, prec, V, V_on_device, st);
 }
@@ -1973,7 +1977,7 @@ mv_status mv_simulate_pairs(mv_ctx* c, int n_pairs, const double* lst, const dou
     if (n_pairs < 0 || (n_pairs > 0 && (!lst || !nu))) return fail(MV_ERR_ARG, "bad pair lists");
     DeviceGuard g(c->device);
     Plan P;
-    plan_pairs(c, n_pairs, lst, nu, P);
+    plan_pairs(c, n_pairs, lst, nu, prec, P);
     cudaStream_t st = stream ? (cudaStream_t)stream : c->stream;
     return run(c, P, prec, V, V_on_device, st);
 }
@@ -1986,8 +1990,8 @@ mv_status mv_autotune(mv_ctx* c, int n_t, const double* lst, int n_nu, const dou
         return fail(MV_ERR_ARG, "bad time/frequency lists");
     DeviceGuard g(c->device);
     Plan P;
-    if (pairs) plan_pairs(c, n_t, lst, nu, P);
-    else plan_grid(c, n_t, lst, n_nu, nu, P);
+    if (pairs) plan_pairs(c, n_t, lst, nu, prec, P);
+    else plan_grid(c, n_t, lst, n_nu, nu, prec, P);
     return autotune(c, P, prec, c->stream, out);
 }
 

@@ -199,10 +199,10 @@ static double blocks_of(int ra, int rb, bool diag) {
     return diag ? 0.5 * ni * (ni + 1) : (double)ni * nj;
 }
 
-Fp32Plan herk_fp32_plan(int N, int n_ax, int n_inst, double est_live, int n_sms) {
+Fp32Plan herk_fp32_plan(int N, int n_ax, int n_inst, double est_live, int n_sms, bool gauss, long long split_budget) {
     Fp32Plan best;
     double t_best = 1e300;
-    for (int form = kZherkReal; form <= kZherkGauss; ++form) {
+    for (int form = kZherkReal; form <= (gauss ? kZherkGauss : kZherkReal); ++form) {
         Fp32Plan z;
         z.form = form;
         z.tiles = form == kZherkReal ? zherk_triangle(2 * N, BT) : zherk_gauss_tiles(N, BT);
@@ -215,6 +215,7 @@ Fp32Plan herk_fp32_plan(int N, int n_ax, int n_inst, double est_live, int n_sms)
         const double units = (double)n_inst * (double)z.tiles.size();
         double t_form = 1e300;
         for (int S = 1; S <= 64 && (S == 1 || stages / S >= 4); ++S) {
+            if (S > 1 && (long long)z.tiles.size() * S * (BT * BT * 4) > split_budget) break;
             // us: rounds of units over the SMs, each a fill, its stages (2.2 us for a whole tile's) and
             // its partial tile; the partial tiles read back; the rows of Z written and read
             const double t = std::ceil(units * S / n_sms) * (4.0 + stages / S * 2.2 * area / (64.0 * z.tiles.size())) +

@@ -119,10 +119,11 @@ std::vector<ZherkTile> zherk_gauss_tiles(int N, int panel);
 
 // Plan for n_inst instances; cover: the real-form tiles to compute (empty: the
 // whole V of N antenna-feeds, in either form).  est_live: live sources
-// expected per instance; ring_budget: bytes the ring may take.  False where
-// the tiles of one instance do not fit the SMs.
+// expected per instance; ring_budget: bytes the ring may take; split_budget: bytes
+// the partial tiles may take where the sources are split (one tile a product is
+// always taken).  False where the tiles of one instance do not fit the SMs.
 bool zherk_plan(int N, const std::vector<ZherkTile>& cover, int n_ax, int n_inst, double est_live, int n_sms,
-                long long ring_budget, ZherkPlan& out);
+                long long ring_budget, long long split_budget, ZherkPlan& out);
 // Antennas per Z warp for groups of up to `chan` channels, `groups` of them in
 // a wave (0: no choice fits); nc: feeds x axes.
 int zherk_ant_block(const ZherkPlan& z, int n_ant, int nc, int groups, int chan, int n_sms);
@@ -144,7 +145,9 @@ struct Fp32Plan {
     int form = kZherkReal, rows = 0, plane_rows = 0, split = 1;
     std::vector<ZherkTile> tiles;
 };
-Fp32Plan herk_fp32_plan(int N, int n_ax, int n_inst, double est_live, int n_sms);
+// gauss: whether that form may be taken; split_budget: bytes of one instance's partial
+// tiles up to which the sources may be split.
+Fp32Plan herk_fp32_plan(int N, int n_ax, int n_inst, double est_live, int n_sms, bool gauss, long long split_budget);
 cudaError_t herk_fp32_init();
 // Partial tiles [n_inst][n_tiles][split][128][128] of U's products.
 cudaError_t launch_herk_fp32(const Inst* d_inst, int inst0, int n_inst, LiveTables lt, int n_ax, const float* d_u,

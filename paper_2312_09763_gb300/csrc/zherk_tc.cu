@@ -1313,7 +1313,7 @@ void make_jobs(std::vector<ZherkTile>& tiles, int plane_rows, int panel, std::ve
 }  // namespace
 
 bool zherk_plan(int N, const std::vector<ZherkTile>& cover, int n_ax, int n_inst, double est_live, int n_sms,
-                long long ring_budget, ZherkPlan& out) {
+                long long ring_budget, long long split_budget, ZherkPlan& out) {
     if (n_inst < 1) return false;
     const double chunks = std::max(1.0, std::ceil(est_live / kZherkChunk));
     double best = 1e300;
@@ -1337,6 +1337,7 @@ bool zherk_plan(int N, const std::vector<ZherkTile>& cover, int n_ax, int n_inst
         const int vcap = (int)std::min<long long>(n_sms / nj, ring_budget / ((long long)zherk_row_bytes(n_ax) * z.rows));
         if (vcap < 1) continue;
         for (int S = 1; S <= 64 && (S == 1 || chunks / S >= 4); ++S) {
+            if (S > 1 && (long long)n_inst * T * S * (128 * 128 * 4) > split_budget) break;
             const int total = n_inst * S, V = std::min(vcap, total), waves = (total + V - 1) / V;
             if (waves > kZherkMaxWaves) continue;
             // us: a chunk of a job (its MMAs at about 80 % of the tensor rate; the Z build
