@@ -232,7 +232,8 @@ mv_status mv_simulate_pairs(mv_ctx *ctx, int n_pairs, const double *lst, const d
  * k-blocks), and the streamed schedule (see mv_options.fuse_zbuild) on up to 64
  * instances of the call where the options allow it, with CUDA events on the
  * context's stream, and keeps the fastest for later calls with the same matrix
- * size, batch size and precision.
+ * size, batch size and precision.  Whether such a call streams is kept for what was
+ * timed alone: a grid or pairs, all of V, a sky of as many sources.
  * Synchronises.  prec must be a tensor-core precision.  out may be NULL. */
 mv_status mv_autotune(mv_ctx *ctx, int n_t, const double *lst, int n_nu, const double *nu,
                       mv_precision prec, int pairs, mv_tuning *out);

@@ -128,6 +128,8 @@ struct mv_ctx {
         HerkCfg cfg;
         bool fuse = true;  // the timed schedule: fused Z build, or separate Z-side launches
         bool stream = false;  // or the streamed one
+        bool pairs = false;   // what was timed: pairs or a grid, of a sky of n_src sources
+        long long n_src = 0;
         double ms = 0;
     } tuned;
     // captured launch sequence of the last call shape
@@ -636,6 +638,15 @@ bool tuned_for(const mv_ctx* c, const Prepared& p) {
     return c->tuned.valid && c->tuned.rows == p.rows && c->tuned.slots == p.max_slots && c->tuned.zprec == p.zprec;
 }
 
+// Whether the autotuner timed another schedule faster than the streamed one, for calls
+// of this kind: how the streamed one does beside the others depends on the products
+// of an instance (all of V, or a redundant array's cover), on whether instances share
+// their channels' spacing (a grid) or not (pairs), and on the sources.
+bool tuned_away(const mv_ctx* c, const Prepared& p) {
+    return tuned_for(c, p) && !c->tuned.stream && !p.plan->unique && c->tuned.pairs == p.plan->pairs &&
+           c->tuned.n_src == c->model.n_src;
+}
+
 HerkCfg chosen_cfg(mv_ctx* c, const Prepared& p) {
     if (p.ho.uidx) {
         // the redundant-group cover: its own tile count, 128 columns unless
@@ -652,7 +663,7 @@ HerkCfg chosen_cfg(mv_ctx* c, const Prepared& p) {
                       : (int)std::max(1ll, std::min((4ll * c->n_sms + base - 1) / base, est_kb / 32));
         return h;
     }
-    if (tuned_for(c, p)) return c->tuned.cfg;
+    if (tuned_for(c, p) && !c->tuned.stream) return c->tuned.cfg;
     return heuristic_cfg(c, p);
 }
 
@@ -747,8 +758,7 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
     std::vector<uint8_t> ztab;
     const mv_options& o = c->opt;
     if (allow_stream && p.zprec != 0 && o.fuse_zbuild && !o.overlap_batches && o.herk_tile_n == 0 && o.herk_split == 0 &&
-        o.herk_flush_kblocks == 0 && (ignore_tuning || !(tuned_for(c, p) && !c->tuned.stream)) &&
-        all_sms(c, st)) {
+        o.herk_flush_kblocks == 0 && (ignore_tuning || !tuned_away(c, p)) && all_sms(c, st)) {
         std::vector<ZGroup> groups = P.groups;
         std::vector<Plan::Batch> batches = P.batches;
         const int slots = p.max_slots;
@@ -801,7 +811,7 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
     // short to hide the next batch's Z build (350-antenna array, 9 of 21
     // tiles: 250 ms per step fused against 210 ms separate)
     p.fuse = !p.stream && c->opt.fuse_zbuild && p.zprec != 0 && P.batches.size() > 1 &&
-             herk_tc_fusable(128, p.zprec, m.n_ax, m.n_feed) && !(tuned_for(c, p) && !c->tuned.fuse) &&
+             herk_tc_fusable(128, p.zprec, m.n_ax, m.n_feed) && !(tuned_for(c, p) && !c->tuned.stream && !c->tuned.fuse) &&
              (!P.unique || c->red.kind == 0);
     p.nbuf = (!p.stream && P.batches.size() > 1 && (c->opt.overlap_batches || p.fuse)) ? 2 : 1;
     // antenna phase factors: per batch, groups x wavenumbers per group x antennas
@@ -1505,6 +1515,8 @@ mv_status autotune(mv_ctx* c, Plan& P, mv_precision prec, cudaStream_t st, mv_tu
     if ((s = mv_check_device_status(c, st))) return s;
     c->tuned.valid = true;
     c->tuned.stream = best_stream;
+    c->tuned.pairs = P.pairs;
+    c->tuned.n_src = c->model.n_src;
     c->tuned.rows = p.rows;
     c->tuned.slots = p.max_slots;
     c->tuned.zprec = p.zprec;
