@@ -263,6 +263,12 @@ mv_status upload(mv_ctx* c, Buf& b, const void* h, size_t bytes, cudaStream_t st
     return cuda_check(cudaMemcpyAsync(b.p, h, bytes, cudaMemcpyHostToDevice, st), "upload");
 }
 
+// Work queued on the context's stream from here on waits for the last call's kernels,
+// on whatever stream they run: what a set-up call overwrites they may still read.
+mv_status after_last_call(mv_ctx* c) {
+    return cuda_check(cudaStreamWaitEvent(c->stream, c->ev_read, 0), "event wait");
+}
+
 struct DeviceGuard {
     int prev = -1;
     explicit DeviceGuard(int dev) {
@@ -1359,7 +1365,7 @@ mv_status run(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_device, c
     } else {
         if ((s = enqueue_all(c, P, p, h, st, &L))) return s;
     }
-    {   // (a new sky waits for the kernels that read the old one)
+    {   // (set-up calls wait for the kernels that read what they overwrite)
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
         else if (cs == cudaStreamCaptureStatusNone && (s = cuda_check(cudaEventRecord(c->ev_read, st), "event"))) return s;
@@ -1692,7 +1698,7 @@ mv_status mv_init_sky(mv_ctx* c, int64_t n_src, const double* ra, const double* 
     if ((s = ensure(c, c->xeq, sizeof(double) * 3 * (size_t)n_src))) return s;
     if ((s = ensure(c, c->sqrt_flux, sizeof(float) * (size_t)n_src))) return s;
     if ((s = ensure(c, c->half_alpha, sizeof(float) * (size_t)n_src))) return s;
-    if ((s = cuda_check(cudaStreamWaitEvent(c->stream, c->ev_read, 0), "event wait"))) return s;
+    if ((s = after_last_call(c))) return s;
     for (int64_t s0 = 0; s0 < n_src; s0 += kSkyChunk) {
         const int64_t m = std::min<int64_t>(kSkyChunk, n_src - s0);
         if (n_src > kSkyChunk) parallel_for(m, [&](int64_t b, int64_t e, int) { convert(s0, m, b, e); });
@@ -1751,6 +1757,7 @@ mv_status mv_set_sky_polarisation(mv_ctx* c, int64_t n_src, const double* q, con
         const double m11 = d > 0.0 ? std::sqrt(d) : 0.0;
         M[i] = make_float4((float)m00, (float)m10r, (float)m10i, (float)m11);
     }
+    if ((s = after_last_call(c))) return s;
     if ((s = upload(c, c->pol_m, M.data(), M.size() * sizeof(float4), c->stream))) return s;
     if ((s = cuda_check(cudaStreamSynchronize(c->stream), "set_sky_polarisation"))) return s;
     c->model.pol_m = (const float4*)c->pol_m.p;
@@ -1787,6 +1794,7 @@ mv_status mv_set_beam_grid(mv_ctx* c, int n_beam, int n_feed, int n_ax, int n_nu
     if (bad < (int64_t)(2 * n)) return fail(MV_ERR_ARG, "beam value %zu not finite", (size_t)bad / 2);
     DeviceGuard g(c->device);
     mv_status s;
+    if ((s = after_last_call(c))) return s;
     if ((s = upload(c, c->grid, values, n * sizeof(float2), c->stream))) return s;
     if ((s = cuda_check(cudaStreamSynchronize(c->stream), "set_beam_grid"))) return s;
     Model& m = c->model;
@@ -1826,6 +1834,7 @@ mv_status mv_set_antennas(mv_ctx* c, int n_ant, const double* enu, const int32_t
     }
     DeviceGuard g(c->device);
     mv_status s;
+    if ((s = after_last_call(c))) return s;
     if ((s = upload(c, c->ant_e, e.data(), n_ant * sizeof(double), c->stream))) return s;
     if ((s = upload(c, c->ant_n, no.data(), n_ant * sizeof(double), c->stream))) return s;
     if ((s = upload(c, c->ant_u, u.data(), n_ant * sizeof(double), c->stream))) return s;
@@ -1900,6 +1909,7 @@ mv_status mv_set_redundancy(mv_ctx* c, double tol_m, int64_t* n_unique) {
     }
     DeviceGuard g(c->device);
     mv_status s;
+    if ((s = after_last_call(c))) return s;
     if ((s = upload(c, c->red_e, e.data(), n * sizeof(double), c->stream))) return s;
     if ((s = upload(c, c->red_n, no.data(), n * sizeof(double), c->stream))) return s;
     if ((s = upload(c, c->red_u, u.data(), n * sizeof(double), c->stream))) return s;
@@ -2124,6 +2134,8 @@ mv_status mv_surrogate_train(mv_ctx* c, int steps, int batch, float lr0, float l
     DeviceGuard g(c->device);
     double l0 = 0, l1 = 0;
     long long L = 0;
+    mv_status s;
+    if ((s = after_last_call(c))) return s;
     cudaError_t e = surrogate_train(c->sur, c->model, (const float2*)c->grid.p, c->grid_nu0, c->grid_dnu, steps, batch,
                                     lr0, lr1, seed, c->stream, &l0, &l1, &L);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -2166,7 +2178,8 @@ mv_status mv_surrogate_set_params(mv_ctx* c, const float* host) {
     if (!c || !host) return fail(MV_ERR_ARG, "NULL argument");
     if (!c->sur) return fail(MV_ERR_STATE, "no surrogate");
     DeviceGuard g(c->device);
-    cudaError_t e = surrogate_set_params(c->sur, host);
+    cudaError_t e = cudaEventSynchronize(c->ev_read);
+    if (e == cudaSuccess) e = surrogate_set_params(c->sur, host);
     if (e != cudaSuccess) return fail(MV_ERR_CUDA, "parameter copy: %s", cudaGetErrorString(e));
     return MV_OK;
 }
@@ -2200,6 +2213,7 @@ mv_status mv_surrogate_eval(mv_ctx* c, int n, const int32_t* beam, const double*
     if (s) return s;
     if (!out) return fail(MV_ERR_ARG, "out is NULL");
     DeviceGuard g(c->device);
+    if ((s = after_last_call(c))) return s;
     cudaError_t e = surrogate_eval(c->sur, n, beam, faz.data(), fza.data(), fnu.data(), out, c->stream);
     if (e != cudaSuccess) return fail(MV_ERR_CUDA, "surrogate evaluation: %s", cudaGetErrorString(e));
     return MV_OK;
@@ -2213,6 +2227,7 @@ mv_status mv_surrogate_grad(mv_ctx* c, int n, const int32_t* beam, const double*
     if (s) return s;
     if (n % 8 || !target || !grads || !loss) return fail(MV_ERR_ARG, "n a multiple of 8; target, grads, loss");
     DeviceGuard g(c->device);
+    if ((s = after_last_call(c))) return s;
     cudaError_t e = surrogate_grad(c->sur, n, beam, faz.data(), fza.data(), fnu.data(), target, grads, loss, c->stream);
     if (e != cudaSuccess) return fail(MV_ERR_CUDA, "surrogate gradient: %s", cudaGetErrorString(e));
     return MV_OK;
