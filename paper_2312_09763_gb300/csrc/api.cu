@@ -531,6 +531,11 @@ bool plan_stream(mv_ctx* c, Plan& P, Prepared& p, std::vector<uint8_t>& tab) {
     const long long budget = 8ll << 30;
     int B = (int)std::max(1ll, std::min<long long>(kMaxBatch, budget / wa_slot));
     if (c->opt.max_batch > 0) B = std::min(B, c->opt.max_batch);
+    // a batch's copy to page-locked memory runs beside the next batch: at most 64
+    // instances, or 16 MB of V, a batch (350 antennas x 5000 sources x 256 instances, 0.25
+    // GB: 2366 us in one batch, 1621 so; 64 antennas x 1000 sources, 8 MB: 176 us in one
+    // batch, 218 in four)
+    if (p.Vhost) B = std::min(B, (int)std::max(64ll, std::min<long long>(kMaxBatch, (16ll << 20) / (8 * p.per_inst))));
     auto plan_for = [&](int n) -> const ZherkPlan* {
         std::vector<long long> key = {p.rows, m.n_ax, n, m.n_src};
         for (const ZherkTile& t : cover) key.push_back((long long)t.r0 << 32 | (unsigned)t.c0);
@@ -757,6 +762,14 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
         p.ho.n_ant = m.n_ant;
         p.ho.n_feed = m.n_feed;
     }
+    p.Vhost = nullptr;
+    if (!V_on_device) {
+        // page-locked host output: each batch's V is copied as soon as its HERK ends
+        cudaPointerAttributes pa{};
+        if (cudaPointerGetAttributes(&pa, V) == cudaSuccess && pa.type == cudaMemoryTypeHost)
+            p.Vhost = static_cast<float2*>(V);
+        cudaGetLastError();
+    }
     // the streamed schedule unless an option asks for a particular HERK or
     // Z-build schedule, the autotuner timed another one faster for calls of
     // this shape, or the call runs on a part of the SMs (the launch needs all of its
@@ -875,15 +888,9 @@ mv_status prepare(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_devic
         return s;
     p.Vout = static_cast<float2*>(V);
     p.v_bytes = sizeof(float2) * (size_t)p.n_inst * p.per_inst;
-    p.Vhost = nullptr;
     if (!V_on_device) {
         if ((s = ensure(c, c->vdev, p.v_bytes))) return s;
         p.Vout = static_cast<float2*>(c->vdev.p);
-        // page-locked host output: each batch's V is copied as soon as its HERK ends
-        cudaPointerAttributes pa{};
-        if (cudaPointerGetAttributes(&pa, V) == cudaSuccess && pa.type == cudaMemoryTypeHost)
-            p.Vhost = static_cast<float2*>(V);
-        cudaGetLastError();
     }
     LiveTables& lt = p.lt;
     lt.sfix = (unsigned*)c->lsfix.p;
