@@ -1010,7 +1010,7 @@ mv_status enqueue_wa(mv_ctx* c, const Prepared& p, const Plan::Batch& b, int k, 
                          (float2*)c->wa[k].p, p.pitch, (float*)c->amax[k].p, (int*)c->err.p, c->n_sms, st, L);
     else
         e = launch_wa(m, (const float2*)c->planes.p, c->d_chan, d_inst, b.inst0, b.n, p.lt,
-                      (float2*)c->wa[k].p, p.pitch, (float*)c->amax[k].p, st, L);
+                      (float2*)c->wa[k].p, p.pitch, (float*)c->amax[k].p, c->n_sms, st, L);
     tw.end();
     return launched(e, "beam evaluation", st);
 }

@@ -145,7 +145,7 @@ __device__ __forceinline__ void put_wa(float2* row, long long s, float2 v) {
 // slot's components, as float bits.
 cudaError_t launch_wa(const Model& m, const float2* d_planes, const Chan* d_chan, const Inst* d_inst,
                       int inst0, int n_inst, LiveTables lt, float2* d_wa, long long wa_pitch,
-                      float* d_amax, cudaStream_t st, long long* launches);
+                      float* d_amax, int n_sms, cudaStream_t st, long long* launches);
 // A group of instances of one time whose Z matrices are built together (the
 // FP64 path length x_a . s_hat is formed once per antenna and source).
 struct ZGroup {

@@ -427,10 +427,10 @@ cudaError_t launch_front(const FrontArgs& args, int n_times, LiveTables lt, cuda
 
 cudaError_t launch_wa(const Model& m, const float2* d_planes, const Chan* d_chan, const Inst* d_inst,
                       int inst0, int n_inst, LiveTables lt, float2* d_wa, long long wa_pitch, float* d_amax,
-                      cudaStream_t st, long long* launches) {
+                      int n_sms, cudaStream_t st, long long* launches) {
     // slots per thread: as many as leave four blocks of 128 sources for every SM
     const long long bx = (lt.pitch + 127) / 128;
-    const int per = (int)std::max(1ll, std::min<long long>(4, bx * n_inst / (4 * 152)));
+    const int per = (int)std::max(1ll, std::min<long long>(4, bx * n_inst / (4ll * n_sms)));
     const dim3 grid((unsigned)bx, (unsigned)((n_inst + per - 1) / per));
     *launches += 1;
     return launch_chained(m.interp == 0 ? k_wa<4> : k_wa<2>, grid, dim3(128), 0, st, m, d_planes, d_chan, d_inst, inst0,

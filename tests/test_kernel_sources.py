@@ -69,3 +69,25 @@ def test_warp_waits_vote():
         body = body[:body.index("}")]
         assert re.search(r"return __all_sync\(0xffffffffu, wait_bounded\w*\(", body), name
     assert re.search(r"bool warp_aborted\([^)]*\) \{ return __any_sync\(0xffffffffu, \*abort_flag != 0\)", s)
+
+
+def _poly(text, name):
+    """The FP32 literals of the statement that sets `name`, in order."""
+    i = text.index(name)
+    return [float(v) for v in re.findall(r"(-?\d+\.\d+)f", text[i:text.index(";", i)])]
+
+
+def test_packed_sincos_has_the_pinned_coefficients():
+    # the streamed schedule's packed cos / sin holds the polynomials of zcore.cuh,
+    # whose error bound tests/test_oracle_pins.py checks
+    z, p = source("zcore.cuh"), source("zherk_tc.cu")
+    z, p = z[z.index("cos_sin_turns"):], p[p.index("cos_sin_turns2("):]
+    sin, cos = _poly(z, "const float sp"), _poly(z, "const float cp")
+    assert len(sin) == 4 and len(cos) == 5
+    assert _poly(p, "const F2 sp") == sin
+    assert _poly(p, "const F2 cp") == cos
+
+
+def test_no_kernel_launch_assumes_a_number_of_sms():
+    for name in sorted(os.listdir(CSRC)):
+        assert not re.search(r"\b152\b", source(name)), name
