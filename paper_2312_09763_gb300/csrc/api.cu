@@ -120,6 +120,7 @@ struct mv_ctx {
     // copies of each batch's V to pinned host memory, overlapping the next batches
     cudaStream_t cstream = nullptr;
     cudaEvent_t ev_vdone = nullptr, ev_cdone = nullptr, ev_read = nullptr;  // ev_read: the last call's kernels
+    cudaStream_t last_stream = nullptr;  // and the stream they run on
     int n_sms = 148;
     // autotuned HERK configuration, valid for calls of the same shape
     struct Tuned {
@@ -263,10 +264,21 @@ mv_status upload(mv_ctx* c, Buf& b, const void* h, size_t bytes, cudaStream_t st
     return cuda_check(cudaMemcpyAsync(b.p, h, bytes, cudaMemcpyHostToDevice, st), "upload");
 }
 
-// Work queued on the context's stream from here on waits for the last call's kernels,
-// on whatever stream they run: what a set-up call overwrites they may still read.
-mv_status after_last_call(mv_ctx* c) {
-    return cuda_check(cudaStreamWaitEvent(c->stream, c->ev_read, 0), "event wait");
+// Whether a caller records st into a graph of its own (no event of ours may enter it).
+bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
+    return cs != cudaStreamCaptureStatusNone;
+}
+
+// Work queued on st from here on waits for the last call's kernels, on whatever stream
+// they run: what a set-up call overwrites they may still read, and the next call works
+// in the same buffers.  (A stream that outlives the context is in order by itself;
+// another one's handle may have been given to a new stream since.)
+mv_status after_last_call(mv_ctx* c, cudaStream_t st) {
+    if (st == c->last_stream && (st == c->stream || st == cudaStreamLegacy)) return MV_OK;
+    if (capturing(st)) return MV_OK;
+    return cuda_check(cudaStreamWaitEvent(st, c->ev_read, 0), "event wait");
 }
 
 struct DeviceGuard {
@@ -1335,7 +1347,9 @@ mv_status run(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_device, c
     c->launches = 0;
     ModelSwap swap(c, P.unique);
     Prepared p;
-    mv_status s = prepare(c, P, prec, V, V_on_device, st, p);
+    mv_status s = after_last_call(c, st);
+    if (s) return s;
+    s = prepare(c, P, prec, V, V_on_device, st, p);
     if (s || p.n_inst == 0) return s;
     const HerkCfg h = chosen_cfg(c, p);
 
@@ -1372,10 +1386,9 @@ mv_status run(mv_ctx* c, Plan& P, mv_precision prec, void* V, int V_on_device, c
     } else {
         if ((s = enqueue_all(c, P, p, h, st, &L))) return s;
     }
-    {   // (set-up calls wait for the kernels that read what they overwrite)
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();
-        else if (cs == cudaStreamCaptureStatusNone && (s = cuda_check(cudaEventRecord(c->ev_read, st), "event"))) return s;
+    if (!capturing(st)) {
+        if ((s = cuda_check(cudaEventRecord(c->ev_read, st), "event"))) return s;
+        c->last_stream = st;
     }
     c->launches = L;
     c->last_inst_t.clear();
@@ -1411,6 +1424,7 @@ mv_status autotune(mv_ctx* c, Plan& P, mv_precision prec, cudaStream_t st, mv_tu
     c->tuned.valid = false;
     Prepared p;
     mv_status s;
+    if ((s = after_last_call(c, st))) return s;
     if ((s = ensure(c, c->vdev, sizeof(float2)))) return s;
     // V for the trial runs: the context's staging buffer
     if ((s = prepare(c, P, prec, c->vdev.p, 0, st, p, false))) return s;
@@ -1705,7 +1719,7 @@ mv_status mv_init_sky(mv_ctx* c, int64_t n_src, const double* ra, const double* 
     if ((s = ensure(c, c->xeq, sizeof(double) * 3 * (size_t)n_src))) return s;
     if ((s = ensure(c, c->sqrt_flux, sizeof(float) * (size_t)n_src))) return s;
     if ((s = ensure(c, c->half_alpha, sizeof(float) * (size_t)n_src))) return s;
-    if ((s = after_last_call(c))) return s;
+    if ((s = after_last_call(c, c->stream))) return s;
     for (int64_t s0 = 0; s0 < n_src; s0 += kSkyChunk) {
         const int64_t m = std::min<int64_t>(kSkyChunk, n_src - s0);
         if (n_src > kSkyChunk) parallel_for(m, [&](int64_t b, int64_t e, int) { convert(s0, m, b, e); });
@@ -1764,7 +1778,7 @@ mv_status mv_set_sky_polarisation(mv_ctx* c, int64_t n_src, const double* q, con
         const double m11 = d > 0.0 ? std::sqrt(d) : 0.0;
         M[i] = make_float4((float)m00, (float)m10r, (float)m10i, (float)m11);
     }
-    if ((s = after_last_call(c))) return s;
+    if ((s = after_last_call(c, c->stream))) return s;
     if ((s = upload(c, c->pol_m, M.data(), M.size() * sizeof(float4), c->stream))) return s;
     if ((s = cuda_check(cudaStreamSynchronize(c->stream), "set_sky_polarisation"))) return s;
     c->model.pol_m = (const float4*)c->pol_m.p;
@@ -1801,7 +1815,7 @@ mv_status mv_set_beam_grid(mv_ctx* c, int n_beam, int n_feed, int n_ax, int n_nu
     if (bad < (int64_t)(2 * n)) return fail(MV_ERR_ARG, "beam value %zu not finite", (size_t)bad / 2);
     DeviceGuard g(c->device);
     mv_status s;
-    if ((s = after_last_call(c))) return s;
+    if ((s = after_last_call(c, c->stream))) return s;
     if ((s = upload(c, c->grid, values, n * sizeof(float2), c->stream))) return s;
     if ((s = cuda_check(cudaStreamSynchronize(c->stream), "set_beam_grid"))) return s;
     Model& m = c->model;
@@ -1841,7 +1855,7 @@ mv_status mv_set_antennas(mv_ctx* c, int n_ant, const double* enu, const int32_t
     }
     DeviceGuard g(c->device);
     mv_status s;
-    if ((s = after_last_call(c))) return s;
+    if ((s = after_last_call(c, c->stream))) return s;
     if ((s = upload(c, c->ant_e, e.data(), n_ant * sizeof(double), c->stream))) return s;
     if ((s = upload(c, c->ant_n, no.data(), n_ant * sizeof(double), c->stream))) return s;
     if ((s = upload(c, c->ant_u, u.data(), n_ant * sizeof(double), c->stream))) return s;
@@ -1916,7 +1930,7 @@ mv_status mv_set_redundancy(mv_ctx* c, double tol_m, int64_t* n_unique) {
     }
     DeviceGuard g(c->device);
     mv_status s;
-    if ((s = after_last_call(c))) return s;
+    if ((s = after_last_call(c, c->stream))) return s;
     if ((s = upload(c, c->red_e, e.data(), n * sizeof(double), c->stream))) return s;
     if ((s = upload(c, c->red_n, no.data(), n * sizeof(double), c->stream))) return s;
     if ((s = upload(c, c->red_u, u.data(), n * sizeof(double), c->stream))) return s;
@@ -2142,7 +2156,7 @@ mv_status mv_surrogate_train(mv_ctx* c, int steps, int batch, float lr0, float l
     double l0 = 0, l1 = 0;
     long long L = 0;
     mv_status s;
-    if ((s = after_last_call(c))) return s;
+    if ((s = after_last_call(c, c->stream))) return s;
     cudaError_t e = surrogate_train(c->sur, c->model, (const float2*)c->grid.p, c->grid_nu0, c->grid_dnu, steps, batch,
                                     lr0, lr1, seed, c->stream, &l0, &l1, &L);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -2220,7 +2234,7 @@ mv_status mv_surrogate_eval(mv_ctx* c, int n, const int32_t* beam, const double*
     if (s) return s;
     if (!out) return fail(MV_ERR_ARG, "out is NULL");
     DeviceGuard g(c->device);
-    if ((s = after_last_call(c))) return s;
+    if ((s = after_last_call(c, c->stream))) return s;
     cudaError_t e = surrogate_eval(c->sur, n, beam, faz.data(), fza.data(), fnu.data(), out, c->stream);
     if (e != cudaSuccess) return fail(MV_ERR_CUDA, "surrogate evaluation: %s", cudaGetErrorString(e));
     return MV_OK;
@@ -2234,7 +2248,7 @@ mv_status mv_surrogate_grad(mv_ctx* c, int n, const int32_t* beam, const double*
     if (s) return s;
     if (n % 8 || !target || !grads || !loss) return fail(MV_ERR_ARG, "n a multiple of 8; target, grads, loss");
     DeviceGuard g(c->device);
-    if ((s = after_last_call(c))) return s;
+    if ((s = after_last_call(c, c->stream))) return s;
     cudaError_t e = surrogate_grad(c->sur, n, beam, faz.data(), fza.data(), fnu.data(), target, grads, loss, c->stream);
     if (e != cudaSuccess) return fail(MV_ERR_CUDA, "surrogate gradient: %s", cudaGetErrorString(e));
     return MV_OK;
