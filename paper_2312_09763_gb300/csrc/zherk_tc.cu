@@ -535,7 +535,9 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
         // and for every chunk that has landed in it (done).  A warp of its own, as the
         // fence before a count waits for the SM's stores to reach L2: that would hold up
         // a Z warp, and in the TMA warp the loads (350 antennas, 1e5 sources, 256
-        // instances: 19.7 ms, 15.7 so).
+        // instances: 19.7 ms, 15.7 so).  Landed chunks are counted with a finished one or
+        // two at a time, unless no more are to land in this wave (15.6 one at a time or
+        // three, 15.5 so; none of those kept back is waited for before the next one lands).
         int wb = -1, q = 0, base = 0, wlen = 0, k = 0;           // the next chunk built
         int wl = -1, lq = 0, lbase = 0, llen = 0, counted = 0;   // the next chunk landed
         ZShare z{1, -1, 0, 0};
@@ -556,7 +558,8 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
             }
             if (wb == P.n_waves && wl == P.n_waves) break;
             const bool built = wb < P.n_waves && __all_sync(0xffffffffu, mbar_test(zdone(k & zmask), zphase(k)));
-            const int land = min(__shfl_sync(0xffffffffu, ld_acquire_cta(landed), 0) - counted, llen - lq);
+            int land = min(__shfl_sync(0xffffffffu, ld_acquire_cta(landed), 0) - counted, llen - lq);
+            if (!built && land < 2 && lq + land < llen) land = 0;
             if (built || land > 0) {
                 if (lane == 0) {
                     if (built) mbar_arrive(zfree(k & zmask));  // (seen: the buffer's barrier may start its next phase)
@@ -593,18 +596,21 @@ k_zherk(const __grid_constant__ CUtensorMap map, const __grid_constant__ ZherkAr
             const int c = next + lane;
             const bool look = next < total - RC && c < total;
             if (look) d = ld_relaxed(P.done + c);
-            while (more && q >= wlen) {  // the next wave this SM builds for
-                if (++w >= P.n_waves) {
-                    more = false;
-                    break;
+            // (as many buffers as are free but for one: a look takes as long as a short chunk;
+            // 12 antennas x 84 pairs x 70,000 sources 657 us with one a look, 600 so)
+            for (int fed = 0; fed < zmask; ++fed) {
+                while (more && q >= wlen) {  // the next wave this SM builds for
+                    if (++w >= P.n_waves) {
+                        more = false;
+                        break;
+                    }
+                    z = z_share(P, w, Z_WARPS * P.ant_block);
+                    base = P.wave_base[w];
+                    wlen = z.team < 0 ? 0 : P.wave_base[w + 1] - base;
+                    q = z.team < 0 ? 0 : z.team;
+                    if (z.team >= 0) g = P.groups + P.wave_group0[w] + z.gi;
                 }
-                z = z_share(P, w, Z_WARPS * P.ant_block);
-                base = P.wave_base[w];
-                wlen = z.team < 0 ? 0 : P.wave_base[w + 1] - base;
-                q = z.team < 0 ? 0 : z.team;
-                if (z.team >= 0) g = P.groups + P.wave_group0[w] + z.gi;
-            }
-            if (more && (k <= zmask || __all_sync(0xffffffffu, mbar_test(zfree(k & zmask), zphase(k) ^ 1u)))) {
+                if (!more || !(k <= zmask || __all_sync(0xffffffffu, mbar_test(zfree(k & zmask), zphase(k) ^ 1u)))) break;
                 any = true;
                 const uint32_t bar = zfull(k & zmask), dst = smem_u32(zsm + (k & zmask) * P.z_buf_b);
                 if (q < g->len) {
