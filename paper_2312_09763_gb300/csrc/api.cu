@@ -543,11 +543,6 @@ bool plan_stream(mv_ctx* c, Plan& P, Prepared& p, std::vector<uint8_t>& tab) {
     const long long budget = 8ll << 30;
     int B = (int)std::max(1ll, std::min<long long>(kMaxBatch, budget / wa_slot));
     if (c->opt.max_batch > 0) B = std::min(B, c->opt.max_batch);
-    // a batch's copy to page-locked memory runs beside the next batch: at most 64
-    // instances, or 16 MB of V, a batch (350 antennas x 5000 sources x 256 instances, 0.25
-    // GB: 2366 us in one batch, 1621 so; 64 antennas x 1000 sources, 8 MB: 176 us in one
-    // batch, 218 in four)
-    if (p.Vhost) B = std::min(B, (int)std::max(64ll, std::min<long long>(kMaxBatch, (16ll << 20) / (8 * p.per_inst))));
     auto plan_for = [&](int n) -> const ZherkPlan* {
         std::vector<long long> key = {p.rows, m.n_ax, n, m.n_src};
         for (const ZherkTile& t : cover) key.push_back((long long)t.r0 << 32 | (unsigned)t.c0);
@@ -562,6 +557,19 @@ bool plan_stream(mv_ctx* c, Plan& P, Prepared& p, std::vector<uint8_t>& tab) {
     if (c->zplans.size() > 64) c->zplans.clear();
     const ZherkPlan* whole = plan_for(std::min(B, p.n_inst));
     if (!whole) return false;
+    // a batch's copy to page-locked memory runs beside the next batch: at most 64
+    // instances, or 16 MB of V, a batch (350 antennas x 5000 sources x 256 instances, 0.25
+    // GB: 2366 us in one batch, 1621 so; 64 antennas x 1000 sources, 8 MB: 176 us in one
+    // batch, 218 in four).  Pairs of one launch are put in waves by their length, which
+    // a cut disturbs: only where the copy (180 GB/s) is a quarter of the work or more
+    // (256 pairs of 1e5 sources, with a new sky each: 22.5 ms in one batch, 23.9 in five).
+    const long long v_inst = 8 * p.per_inst;
+    const int cut = (int)std::max(64ll, std::min<long long>(kMaxBatch, (16ll << 20) / v_inst));
+    if (p.Vhost && cut < std::min(B, p.n_inst) && (!P.pairs || (double)v_inst * std::min(B, p.n_inst) / 180e3 >= 0.25 * whole->us)) {
+        B = cut;
+        whole = plan_for(B);
+        if (!whole) return false;
+    }
     // full batches hold whole waves
     if (p.n_inst > B && whole->S == 1 && B > whole->V) B = B / whole->V * whole->V;
     P.groups.clear();

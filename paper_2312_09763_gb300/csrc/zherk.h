@@ -60,6 +60,7 @@ struct ZherkPlan {
     int rows = 0, panel = 128;       // ring rows per instance, rows of a panel
     int V = 0, S = 0, waves = 0;     // instances per wave, source ranges per instance
     int n_jobs = 0, n_jobs_last = 0;
+    double us = 0;                   // what it is expected to take
     std::vector<ZherkTile> tiles;
     std::vector<ZherkJob> jobs;      // n_sms entries; the last wave runs those with v < its instances
 };

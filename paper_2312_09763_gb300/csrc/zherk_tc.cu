@@ -1352,6 +1352,7 @@ bool zherk_plan(int N, const std::vector<ZherkTile>& cover, int n_ax, int n_inst
             if (t < best) {
                 best = t;
                 out = z;
+                out.us = t;
                 out.V = V;
                 out.S = S;
                 out.waves = waves;

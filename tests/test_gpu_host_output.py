@@ -33,3 +33,22 @@ def test_page_locked_output_comes_in_batches(n_ant, n_times, n_chan):
             assert rel_err(V[it, ic], D[it, ic]) <= 1e-5, (it, ic)
     for it, ic in ((0, 0), (n_times - 1, n_chan - 1)):
         assert rel_err(V[it, ic][pa, pb], oracle.vis(P, w.lsts[it], w.freqs[ic], pairs=(pa, pb))[:, 0, 0]) <= 1e-5
+
+
+def test_long_pairs_stay_in_one_batch():
+    # pairs are put in waves by their live counts; where the products far outlast the
+    # copy, cutting them into batches would only disturb that
+    import torch
+    w = synth.batched_uneven(n_pairs=80, n_ant=200, n_src=60_000, n_za=46, n_az=120)
+    sim = simulator(w)
+    on_device = sim.simulate_pairs(w.lsts, w.freqs)
+    one = sim.last_launch_count()
+    out = torch.empty(on_device.shape, dtype=torch.complex64, pin_memory=True)
+    sim.simulate_pairs(w.lsts, w.freqs, out=out, host=True)
+    assert sim.last_launch_count() == one
+    assert np.array_equal(out.numpy(), on_device.cpu().numpy())
+    # short ones are cut as a grid is
+    w = synth.batched_uneven(n_pairs=80, n_ant=350, n_src=500, n_za=46, n_az=120)
+    sim = simulator(w)
+    sim.simulate_pairs(w.lsts, w.freqs, out=torch.empty((80, 350, 350), dtype=torch.complex64, pin_memory=True), host=True)
+    assert sim.last_launch_count() >= one + 5
