@@ -52,9 +52,9 @@ MLP_DRAM_BYTES_PER_LAUNCH = 53.68e6 + 499.97e6
 # profiles/k_herk_tc_redundant_cover_350ant_1e5src_16ch.txt.
 UNIQUE_DRAM_BYTES_PER_INSTANCE = (2.3149e9 + 0.0433e9) / 16
 # k_zherk on the same workload (19 instances: one wave of the streamed schedule):
-# 9.2 MB read + 1.2435 GB written (chunks of the ring that leave L2 before they are
+# 21.9 MB read + 3.0832 GB written (chunks of the ring that leave L2 before they are
 # overwritten), summarised in profiles/k_zherk_350ant_1e5src_19ch.txt.
-STREAM_DRAM_BYTES_PER_INSTANCE = (0.0092e9 + 1.2435e9) / 19
+STREAM_DRAM_BYTES_PER_INSTANCE = (0.0219e9 + 3.0832e9) / 19
 METRIC = "vis/s (bl·chan·time) at 350 ant×1e5 src; split-prec TC vs FP32 @1e-5 rel err"
 UNIT = "vis/s"
 
@@ -460,9 +460,14 @@ def main():
     if args.precision == "fp32":
         roof = None
     else:
-        # algorithmic flops of one step: three real products over the lower
-        # triangle of the 2N x 2N real Gram matrix, for every instance
-        flops_step = float(np.sum(3 * 2.0 * rows * (rows + 1) / 2 * K))
+        # flops of one step, as the schedule's form of the products needs them, three
+        # FP16 products each, for every instance: the lower triangle of the 2N x 2N real
+        # Gram matrix, or (streamed) F = X Y^T and the lower triangle of H = S S^T of N
+        # antenna-feeds
+        nfd = rows // 2
+        area = nfd * nfd + nfd * (nfd + 1) / 2 if streams(args, hk, tuning, w, pairs, n_h / args.steps) \
+            else rows * (rows + 1) / 2
+        flops_step = float(np.sum(3 * 2.0 * area * K))
         achieved = flops_step * args.steps / (ms_h / 1e3) / 1e12
         # with the fused Z build (the schedule the autotuner timed faster, or
         # the default for a forced 128-column tile) the timed HERK launches
@@ -483,6 +488,8 @@ def main():
                           "its partial tiles)" if streamed else
                           "k_herk_tc" + (" (fused with the next batch's Z build)" if fused else ""),
                 "launches": n_h, "avg_launch_ms": ms_h / max(n_h, 1),
+                "flops_counted": "F and H of N antenna-feeds, three products each" if streamed else
+                                 "lower triangle of the 2N x 2N Gram matrix, three products",
                 "peak_source": f"{src} bf16 sustained (kernel timed inside a long step)"}
         if fused:
             # its second bound: the U planes written (next batch) and read (this
@@ -535,6 +542,7 @@ def main():
             traffic = UNIQUE_DRAM_BYTES_PER_INSTANCE * n_instances(w, pairs) / n_launch
         if streamed:  # Z stays in L2: the sub-matrix products against the tensor rate
             roof.update({"achieved": tflops, "frac": tflops / sustained, "traffic": None,
+                         "flops_counted": "the cover's blocks, three products",
                          "kernel": "k_zherk over the redundant-group cover"})
         else:
             roof.update({"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,

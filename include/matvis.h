@@ -96,15 +96,16 @@ typedef struct {
                                    on a second stream while the HERK of the previous one runs (two
                                    workspace sets); 0 (default): one set, strictly in order */
     int fuse_zbuild;            /* 1 (default): with a tensor-core precision the launch that computes
-                                   V also builds Z.  With the herk_* options at 0 it streams Z of
-                                   many instances through a ring that stays in L2 (Z is never held
-                                   as a whole); with one of them set, or where mv_autotune timed it
-                                   faster, the HERK launch of batch b builds the Z matrices of batch
-                                   b + 1 on extra warps of every SM (two or more batches, two
-                                   workspace sets; one feed and one axis, or two and two), unless
-                                   mv_autotune timed separate launches faster for the call's shape;
-                                   0: the Z build runs as its own launch.  Takes precedence over
-                                   overlap_batches. */
+                                   V also builds Z.  With the herk_* options and overlap_batches at
+                                   0 it streams Z of many instances through a ring that stays in L2
+                                   (Z is never held as a whole; the array's products have to fit the
+                                   SMs, and the stream all of them).  Else, or where mv_autotune
+                                   timed it faster, the HERK launch of batch b builds the Z matrices
+                                   of batch b + 1 on extra warps of every SM (two or more batches,
+                                   two workspace sets; one feed and one axis, or two and two; over
+                                   overlap_batches), unless mv_autotune timed separate launches
+                                   faster for the call's shape; 0: the Z build runs as its own
+                                   launch. */
 } mv_options;
 
 /* A tensor-core HERK configuration chosen by mv_autotune. */

@@ -161,7 +161,7 @@ k_cull_scan(const int* __restrict__ counts, int* __restrict__ offsets, int* __re
 // clock and SM) would bound it: rotating and converting every source before the
 // cut took 390 us for 48 times of 1e5 sources (count and compaction), only the live
 // ones 257.  So directions are 64-bit fixed point, rotated with integer products
-// (to 2^-60, finer than FP64's 2^-53): 143 us.  FP64 East, North and Up go out
+// (within 5 x 2^-60, finer than FP64's 2^-53): 143 us.  FP64 East, North and Up go out
 // only where the caller has asked for them.
 __global__ void __launch_bounds__(kCullThreads)
 k_cull_scatter(Model m, const double* __restrict__ R, CullWork w, int bpt, LiveTables lt) {

@@ -10,9 +10,9 @@ namespace mv {
 constexpr int kZherkChunk = 64;      // sources per ring chunk
 // Chunks in the ring, and bytes of a ring row.  Fewer chunks leave too little
 // between the oldest chunk still being read and the newest ones being built (350
-// antennas, one axis, 256 instances: 16.6 ms with 13 chunks, 16.2 with 14, 15.8 with
-// 15, 15.7 with 16: 82 MB; the redundant cover 6.09, 6.00, 5.88, 5.84); more outgrow
-// the L2 (15.9 and 5.90 with 17, 16.1 and 5.92 with 18).
+// antennas, one axis, 256 instances: 17.1 ms with 13 chunks, 16.2 with 14, 15.7 with
+// 15, 15.5 with 16: 82 MB; the redundant cover 6.11, 5.98, 5.85, 5.78); more outgrow
+// the L2 (15.7 and 5.82 with 17).
 __host__ __device__ constexpr int zherk_ring_chunks(int n_ax) { return n_ax == 1 ? 16 : 9; }
 __host__ __device__ constexpr int zherk_row_bytes(int n_ax) { return zherk_ring_chunks(n_ax) * kZherkChunk * 4 * n_ax; }
 constexpr int kZherkMaxWaves = 2048;

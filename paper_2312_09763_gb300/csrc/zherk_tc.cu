@@ -9,7 +9,7 @@
 // of some instance for the whole source axis, so Z is needed only in source order,
 // by all products at about the same time: a ring of a thousand sources per
 // instance (82 MB in all there, inside the 129 MB L2) is enough, and Z is never
-// read back from HBM (ncu: 1.2 of its 4.0 GB leave L2 before they are overwritten).
+// read back from HBM (ncu: 3.1 of its 4.0 GB leave L2 before they are overwritten).
 //
 // A wave is V virtual instances (an instance, or one of S ranges of its
 // sources) whose products fill the SMs.  The ring is cut into chunks of 64
@@ -32,13 +32,15 @@
 // and 12 (8 with several components) warps build Z.
 //
 // What bounds it (350 antennas x 1e5 sources, 19 instances a wave): L2 traffic.  A
-// 64-source chunk takes 1.38 us (56 instances 3.25 ms, against 4.79 with the Z build
-// fused into the HERK of the previous batch through HBM); in it the SMs read 12 MB
-// of panels and write 5.3 MB of Z, where L2 gives 17 TB/s to reads and 5.7 to
-// writes, and each SM moves 0.27 MB through its shared memory.  Without the Z stores
-// the 56 instances take 2.81 ms, without two of the three products 3.01; the MMAs
-// alone are 0.84 us a chunk, the Z build alone 0.94.  Single-channel groups are
-// bound by their phases (z_ants_one).
+// 64-source chunk takes 1.38 us (256 instances 15.1 ms, of 14 waves of 782 chunks;
+// 56 instances 3.33, against 4.79 with the Z build fused into the HERK of the previous
+// batch through HBM); in it the SMs read 12 MB of panels and write 5.3 MB of Z, where
+// L2 gives 17 TB/s to reads and 5.7 to writes, and each SM moves 0.27 MB through its
+// shared memory.  Copies of the kernel without one part (before its counts were
+// released and acquired, when the 56 instances took 3.25 ms): without the Z stores
+// 2.81, without two of the three products 3.01; the MMAs alone are 0.84 us a chunk,
+// the Z build alone 0.94.  Single-channel groups are bound by their phases
+// (z_ants_one).
 //
 // Layout of a ring row: blocks of 32 columns, 128 bytes each, hi and lo halves of
 // 64 bytes (in turn, see the Z warps), so that one 128-byte-swizzled TMA box of a
